@@ -56,6 +56,9 @@ struct af_handle {
   int pipe_ctas;         // CTAs of the persistent pipelined fused kernel (0: off)
   TileMaps* tmaps;       // tensor maps of the input planes of state[0], state[1]
   int tma;               // 1: the pipelined kernel stages interior tiles by tensor copies
+  int geom;              // tile geometry of the fused step (STEP_GEOMS; -1: 32 x 32 tiles,
+                         // pipelined where the grid allows it)
+  TileMaps* tmaps_geom;  // tensor maps of `geom` where its box differs from tmaps' (else null)
   int zero_copy;         // 1: pinned host planes are converted in place (AF_ZERO_COPY=0: copies)
   void* adj_arena;       // adjoint arena (lazy): LAM_PLANES planes, see AdjView
   int adj_clean;         // 1: its node and increment records are zero (left so by
@@ -252,21 +255,37 @@ void launch_ref_step(af_handle* h, double dt) {
   k_average<T, COMP><<<grd, blk, 0, s>>>(a);
 }
 
+// One fused FP32 step on the handle's tile geometry.
+template <bool COMP>
+void launch_fused(af_handle* h, double dt) {
+  StepArgs<float> a = step_args<float>(h, dt);
+  const TileMaps* maps = h->tma ? &h->tmaps[h->cur] : nullptr;
+  const bool late = h->late_once;  // testing only: one step on the pipelined kernel
+  if (late) {
+    a.late_first_wait = 1;
+    h->late_once = 0;
+  }
+  if (late || h->geom < 0 || h->geom == GEOM_PIPE_32x32 || h->geom == GEOM_32x32) {
+    launch_fused_step<COMP>(h->stream, a, h->pipe_ctas > 0, h->pipe_ctas, maps);
+  } else if (h->geom == GEOM_PIPE_32x28) {
+    launch_pipe_28<COMP>(h->stream, a, h->pipe_ctas,
+                         h->tma ? &h->tmaps_geom[h->cur] : nullptr);
+  } else {
+    a.prefetch_wave = 0;  // (one wave, or two: the tiles of the second are read once)
+    launch_small_tiles<COMP>(h->geom, h->stream, a);
+  }
+}
+
 void launch_step(af_handle* h, double dt) {
   switch (h->prec) {
     case AF_FP64: launch_ref_step<double, false>(h, dt); break;
     case AF_FP32:
     case AF_FP32_COMP:
       if (h->fused) {
-        StepArgs<float> a = step_args<float>(h, dt);
-        a.late_first_wait = h->late_once;  // testing only, one step
-        h->late_once = 0;
         if (h->prec == AF_FP32_COMP)
-          launch_fused_step<true>(h->stream, a, h->pipe_ctas > 0, h->pipe_ctas,
-                                  h->tma ? &h->tmaps[h->cur] : nullptr);
+          launch_fused<true>(h, dt);
         else
-          launch_fused_step<false>(h->stream, a, h->pipe_ctas > 0, h->pipe_ctas,
-                                   h->tma ? &h->tmaps[h->cur] : nullptr);
+          launch_fused<false>(h, dt);
       } else if (h->prec == AF_FP32_COMP) {
         launch_ref_step<float, true>(h, dt);
       } else {
@@ -679,6 +698,24 @@ af_status af_init(af_handle** out, const af_grid* g, double gamma, const af_stat
     }
     h->tma = enc ? 1 : 0;
   }
+  // tile geometry by the grid's size; an explicit AF_PIPE keeps the 32 x 32 tiles
+  h->geom = -1;
+  if (prec != AF_FP64 && !getenv("AF_PIPE")) {
+    StepArgs<float> a = {};
+    a.in = planes_of<float>(h, 0);
+    a.nx = h->nx;
+    a.ny = h->ny;
+    h->geom = choose_step_geometry(a, h->pipe_ctas);
+    if (h->geom == GEOM_PIPE_32x28 && h->tma) {
+      h->tmaps_geom = new (std::nothrow) TileMaps[2];
+      bool enc = h->tmaps_geom != nullptr;
+      for (int b = 0; b < 2 && enc; ++b) {
+        a.in = planes_of<float>(h, b);
+        enc = encode_tile_maps(a, &h->tmaps_geom[b], STEP_GEOMS[h->geom].ty);
+      }
+      if (!enc) h->geom = -1;
+    }
+  }
   if (prec == AF_FP32_COMP || prec == AF_FP32) {
     // zero the lo planes once (unused in AF_FP32)
     for (int s = 0; s < 2; ++s)
@@ -1021,6 +1058,7 @@ void af_destroy(af_handle* h) {
   }
   if (h->h_red) cudaFreeHost(h->h_red);
   delete[] h->tmaps;
+  delete[] h->tmaps_geom;
   delete h;
 }
 

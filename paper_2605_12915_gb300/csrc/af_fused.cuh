@@ -931,9 +931,18 @@ __device__ __forceinline__ bool fused_tile(const StepArgs<float>& a, PipeCtx& pc
   return true;
 }
 
+// Programmatic dependent launch: the next kernel of the stream may be scheduled
+// now (its blocks then sit in pdl_wait), and this one's input is complete.  A
+// kernel launched without the attribute passes both at once.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 template <int TX, int TY, int NT, int MINB, bool COMP>
 __global__ void __launch_bounds__(NT, MINB)
     k_fused_step(const __grid_constant__ StepArgs<float> a) {
+  pdl_wait();
   // prefetch into L2 the tile of the CTA that starts one wave later
   int pi0 = -1, pj0 = -1;
   const int nxt = blockIdx.y * gridDim.x + blockIdx.x + a.prefetch_wave;
@@ -972,6 +981,7 @@ __global__ void __launch_bounds__(NT, MINB)
   if (pc.tm && (threadIdx.x & 31) == 0)
     for (int p = threadIdx.x >> 5; p < 20; p += NT / 32)
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tm.m[p]) : "memory");
+  pdl_wait();
   __syncthreads();
   const int tcols = (a.nx + TX - 1) / TX, ntiles = tcols * ((a.ny + TY - 1) / TY);
   int tile = blockIdx.x;

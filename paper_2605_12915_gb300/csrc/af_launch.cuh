@@ -24,9 +24,10 @@ inline cudaError_t allow_smem(size_t bytes) {
   return e;
 }
 
-// The pipelined kernel's conditions on the grid and the input planes.
-inline bool pipe_eligible(const StepArgs<float>& a) {
-  if ((a.nx & 3) != 0 || a.nx < FUSED_TX + 8 || a.ny < FUSED_TY + 6) return false;
+// The pipelined kernel's conditions on the grid (tiles of FUSED_TX x ty cells) and
+// the input planes.
+inline bool pipe_eligible(const StepArgs<float>& a, int ty = FUSED_TY) {
+  if ((a.nx & 3) != 0 || a.nx < FUSED_TX + 8 || a.ny < ty + 6) return false;
   uintptr_t bits = 0;
   for (int q = 0; q < 4; ++q) bits |= (uintptr_t)a.in.avg[q] | (uintptr_t)a.in.lo[q];
   for (int f = 0; f < 3; ++f)
@@ -35,9 +36,9 @@ inline bool pipe_eligible(const StepArgs<float>& a) {
 }
 
 // Encodes the tensor maps of the 20 input planes in `a` (row-major nx x ny
-// floats, staging box of the fused tile geometry); false if the driver lacks the
-// encoder or rejects a map.
-inline bool encode_tile_maps(const StepArgs<float>& a, TileMaps* out) {
+// floats, staging box of tiles of FUSED_TX x ty cells); false if the driver lacks
+// the encoder or rejects a map.
+inline bool encode_tile_maps(const StepArgs<float>& a, TileMaps* out, int ty = FUSED_TY) {
   typedef CUresult (*Encode)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
                              const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
                              const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -57,7 +58,7 @@ inline bool encode_tile_maps(const StepArgs<float>& a, TileMaps* out) {
   using G = FusedGeom<FUSED_TX, FUSED_TY>;
   const cuuint64_t dims[2] = {(cuuint64_t)a.nx, (cuuint64_t)a.ny};
   const cuuint64_t strides[1] = {(cuuint64_t)a.nx * sizeof(float)};
-  const cuuint32_t box[2] = {(cuuint32_t)G::SW, (cuuint32_t)G::CH}, unit[2] = {1, 1};
+  const cuuint32_t box[2] = {(cuuint32_t)G::SW, (cuuint32_t)(ty + 6)}, unit[2] = {1, 1};
   for (int p = 0; p < 20; ++p) {
     float* base = p < 12 ? a.in.pt[p >> 2][p & 3] : p < 16 ? a.in.avg[p - 12] : a.in.lo[p - 16];
     if (enc(&out->m[p], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, unit,
@@ -68,32 +69,112 @@ inline bool encode_tile_maps(const StepArgs<float>& a, TileMaps* out) {
   return true;
 }
 
-// One step of the grid described by `a`: the persistent pipelined kernel on
-// `ctas` CTAs when `pipe` is set and the grid allows it (tensor-copy staging
-// when `maps` is given), else one CTA per tile.  INTER (pipelined kernel
-// only) also stores the intermediates the adjoint needs.
+// Launches `kern` so that it may be scheduled while the stream's previous kernel
+// drains (programmatic dependent launch); the kernel itself waits for that
+// kernel's results (pdl_wait) before it touches memory.  Saves the launch gap
+// between steps: 8.35 -> 6.54 us per step at 64 x 64 cells, 18.6 -> 16.8 at 256^2.
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int threads, size_t smem,
+                                    cudaStream_t s, const A&... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute at[1] = {};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kern, args...);
+}
+
+// One CTA per tile of TX x TY cells.
+template <int TX, int TY, int NT, int MINB, bool COMP>
+inline cudaError_t launch_step_tiles(cudaStream_t s, const StepArgs<float>& a) {
+  using G = FusedGeom<TX, TY>;
+  constexpr auto kern = k_fused_step<TX, TY, NT, MINB, COMP>;
+  const cudaError_t e = allow_smem<kern>(G::SMEM);
+  if (e != cudaSuccess) return e;
+  return launch_dependent(kern, dim3((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY), NT, G::SMEM, s,
+                          a);
+}
+
+// Persistent pipelined CTAs over the tiles of TX x TY cells (tensor-copy staging
+// when `maps` is given).
+template <int TX, int TY, int NT, int MINB, bool COMP, bool INTER>
+inline cudaError_t launch_step_pipe(cudaStream_t s, const StepArgs<float>& a, int ctas,
+                                    const TileMaps* maps) {
+  using G = FusedGeom<TX, TY>;
+  constexpr auto kern = k_fused_step_pipe<TX, TY, NT, MINB, COMP, INTER>;
+  const cudaError_t e = allow_smem<kern>(G::SMEM_PIPE);
+  if (e != cudaSuccess) return e;
+  static TileMaps none;
+  const int ntiles = ((a.nx + TX - 1) / TX) * ((a.ny + TY - 1) / TY);
+  return launch_dependent(kern, dim3(ntiles < ctas ? ntiles : ctas), NT, G::SMEM_PIPE, s, a,
+                          maps ? *maps : none, maps ? 1 : 0);
+}
+
+// Tile geometries of a lone grid's step.  Results do not depend on the choice
+// (every value a tile recomputes for its halo rounds the same way).
+//
+// A step is a sequence of dependent phases, and its time is (waves of one tile per
+// SM) x (time of one tile): a tile of 32 x 32 cells takes 28 us however few of
+// them a grid has, so a grid too small to give every SM one of those runs faster
+// on smaller tiles although they recompute more halo.  `us` is the measured time
+// of one wave (FP32_COMP, GB300); the geometry with the smallest sum is taken.
+// Measured per step, 32 x 32 tiles -> chosen: 32^2 27.4 -> 5.3 us (8 x 4), 64^2 30.8 -> 6.5
+// (8 x 8), 128^2 30.8 -> 7.6 (16 x 8), 192^2 30.9 -> 11.2 (16 x 16), 256^2 30.9 -> 16.8
+// (32 x 16), 333 x 250 30.8 -> 21.8 (32 x 24), 448^2 57.7 -> 42.4 (32 x 24).
+struct StepGeometry {
+  int tx, ty;
+  int pipe;      // persistent CTAs with the next tile's input staged asynchronously
+  float us;      // time of one wave
+  float fill;    // once per step (pipelined: the first tile's input)
+};
+enum { GEOM_8x4, GEOM_8x8, GEOM_16x8, GEOM_16x16, GEOM_32x16, GEOM_32x24, GEOM_32x32,
+       GEOM_PIPE_32x28, GEOM_PIPE_32x32, N_STEP_GEOMS };
+constexpr StepGeometry STEP_GEOMS[N_STEP_GEOMS] = {
+    {8, 4, 0, 5.9f, 0.f},   {8, 8, 0, 6.6f, 0.f},   {16, 8, 0, 7.5f, 0.f},
+    {16, 16, 0, 11.2f, 0.f}, {32, 16, 0, 16.7f, 0.f}, {32, 24, 0, 21.6f, 0.f},
+    {FUSED_TX, FUSED_TY, 0, 28.5f, 0.f},
+    {FUSED_TX, 28, 1, 22.5f, 4.f}, {FUSED_TX, FUSED_TY, 1, 25.5f, 4.f}};
+
+inline int choose_step_geometry(const StepArgs<float>& a, int sms) {
+  int best = GEOM_32x32;
+  float best_us = 1e30f;
+  for (int g = 0; g < N_STEP_GEOMS; ++g) {
+    const StepGeometry& q = STEP_GEOMS[g];
+    if (q.pipe && !pipe_eligible(a, q.ty)) continue;
+    const int64_t tiles = (int64_t)((a.nx + q.tx - 1) / q.tx) * ((a.ny + q.ty - 1) / q.ty);
+    const float us = (float)((tiles + sms - 1) / sms) * q.us + q.fill;
+    if (us < best_us) {
+      best_us = us;
+      best = g;
+    }
+  }
+  return best;
+}
+
+// The steps of the geometries smaller than 32 x 32 (af_tiles.cu).
+template <bool COMP>
+cudaError_t launch_small_tiles(int geom, cudaStream_t s, const StepArgs<float>& a);
+template <bool COMP>
+cudaError_t launch_pipe_28(cudaStream_t s, const StepArgs<float>& a, int ctas,
+                           const TileMaps* maps);
+
+// One step of the grid described by `a` with 32 x 32 tiles: the persistent
+// pipelined kernel on `ctas` CTAs when `pipe` is set and the grid allows it
+// (tensor-copy staging when `maps` is given), else one CTA per tile.  INTER
+// (pipelined kernel only) also stores the intermediates the adjoint needs.
 template <bool COMP, bool INTER = false>
 inline cudaError_t launch_fused_step(cudaStream_t s, const StepArgs<float>& a, bool pipe,
                                      int ctas, const TileMaps* maps) {
-  using G = FusedGeom<FUSED_TX, FUSED_TY>;
-  const int tcols = (a.nx + FUSED_TX - 1) / FUSED_TX, trows = (a.ny + FUSED_TY - 1) / FUSED_TY;
-  if (pipe && ctas > 0 && pipe_eligible(a)) {
-    constexpr auto kern = k_fused_step_pipe<FUSED_TX, FUSED_TY, FUSED_NT, AF_FUSED_MINB, COMP, INTER>;
-    const cudaError_t e = allow_smem<kern>(G::SMEM_PIPE);
-    if (e != cudaSuccess) return e;
-    static TileMaps none;
-    const int ntiles = tcols * trows;
-    kern<<<ntiles < ctas ? ntiles : ctas, FUSED_NT, G::SMEM_PIPE, s>>>(a, maps ? *maps : none,
-                                                                         maps ? 1 : 0);
-    return cudaGetLastError();
-  }
+  if (pipe && ctas > 0 && pipe_eligible(a))
+    return launch_step_pipe<FUSED_TX, FUSED_TY, FUSED_NT, AF_FUSED_MINB, COMP, INTER>(s, a, ctas,
+                                                                                      maps);
   if (INTER) return cudaErrorNotSupported;
-  constexpr auto kern = k_fused_step<FUSED_TX, FUSED_TY, FUSED_NT, AF_FUSED_MINB, COMP>;
-  const cudaError_t e = allow_smem<kern>(G::SMEM);
-  if (e != cudaSuccess) return e;
-  dim3 grd(tcols, trows);
-  kern<<<grd, FUSED_NT, G::SMEM, s>>>(a);
-  return cudaGetLastError();
+  return launch_step_tiles<FUSED_TX, FUSED_TY, FUSED_NT, AF_FUSED_MINB, COMP>(s, a);
 }
 
 // Tile geometries available to the batched launch (the autotuner picks one):
