@@ -26,7 +26,7 @@ using namespace af;
 
 namespace af {
 // foot-centred point update of the three point families (af_fc.cu)
-cudaError_t launch_fc_points(const StepArgs<double>& a, dim3 grd, dim3 blk, cudaStream_t s);
+cudaError_t launch_fc_points(const StepArgs<double>& a, cudaStream_t s);
 }  // namespace af
 
 struct af_handle {
@@ -237,7 +237,7 @@ void launch_ref_step(af_handle* h, double dt) {
   if constexpr (std::is_same<T, double>::value) {
     if (h->var == AF_FC) {  // foot-centred: no nodal increments, points from the foot disks
       k_center<T, COMP><<<grd, blk, 0, s>>>(a);
-      launch_fc_points(a, grd, blk, s);
+      launch_fc_points(a, s);
       k_flux<T><<<grd, blk, 0, s>>>(a);
       k_average<T, COMP><<<grd, blk, 0, s>>>(a);
       return;
