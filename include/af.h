@@ -112,7 +112,7 @@ enum {
  * later call of this handle runs.  On error *out is NULL.
  *
  * The handle allocates two states and the step's scratch planes here (about
- * 88 planes of nx * ny values of the working precision); af_adjoint_step
+ * 84 planes of nx * ny values of the working precision); af_adjoint_step
  * allocates its own work area (92 planes) on its first call, host transfers
  * of pageable planes a staging buffer of 16 FP64 planes on their first use,
  * af_exchange_state another 16 FP64 planes and a second stream with host
@@ -229,7 +229,7 @@ const char *af_status_string(af_status s);
  * t^n (`in`) and receives the state at t^n + dt (`out`), both FP64 device
  * arrays in the layout above, on the current device, not overlapping.  The
  * intermediate values live in one work area compiled into the library (a
- * static device array of about 6.3 MB that every GPU loading the library holds
+ * static device array of about 5.8 MB that every GPU loading the library holds
  * until the process exits); no cudaMalloc, cudaFree or other allocating call
  * is made.  The first call on a device looks up the work area's address on
  * that device.  Every call shares the one work area: calls that overlap on the GPU (other streams,

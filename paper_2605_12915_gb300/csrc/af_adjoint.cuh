@@ -51,11 +51,6 @@ constexpr int LAM_LU = 92;
 constexpr int LAM_PLANES = 96;
 constexpr int SCR_INC = 4, SCR_HALF = 28;
 
-// family of lattice offset (a, b) from a cell's vertex: V, E_v, E_h, C
-__host__ __device__ constexpr int fam_of(int a, int b) {
-  return (a & 1) ? ((b & 1) ? 3 : 2) : ((b & 1) ? 1 : 0);
-}
-
 // cell index wrapped into [0, n): one conditional step for |i| < 2n
 __device__ __forceinline__ int wrapc(int i, int n) {
   const int w = i < 0 ? i + n : (i >= n ? i - n : i);
@@ -75,7 +70,7 @@ __device__ __forceinline__ Prim<T> node_w(const AdjView<T>& v, int fam, size_t i
   return w;
 }
 
-// increments (du, dv, dp) of duration s at the node of family fam of cell id
+// increments (u + du, v + dv, dp) of duration s at the node of family fam of cell id
 template <typename T>
 __device__ __forceinline__ void node_d(const AdjView<T>& v, int s, int fam, size_t id, T d[3]) {
   const T* b = v.scr + (size_t)(SCR_INC + 12 * s + 3 * fam) * v.ps + id;
@@ -397,8 +392,12 @@ __device__ __forceinline__ void point_adj(const AdjView<T>& v, const Acc& acc, i
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
         const int n = 3 * b + q;
-        T dot = nf[n].r * lwf[0] + nf[n].u * lwf[1] + nf[n].v * lwf[2] + nf[n].p * lwf[3];
-        if (v.variant == 0) dot += df[n][0] * ld[0] + df[n][1] * ld[1] + df[n][2] * ld[2];
+        // (u and du enter the transported update with the same weight, and the
+        // increment planes hold u + du, v + dv)
+        T dot = v.variant == 0
+                    ? nf[n].r * lwf[0] + df[n][0] * lwf[1] + df[n][1] * lwf[2] +
+                          nf[n].p * lwf[3] + df[n][2] * ld[2]
+                    : nf[n].r * lwf[0] + nf[n].u * lwf[1] + nf[n].v * lwf[2] + nf[n].p * lwf[3];
         lxi += dx3[q] * lyb[b] * dot;
         leta += lx[q] * dy3[b] * dot;
       }
@@ -457,27 +456,6 @@ __global__ void __launch_bounds__(256, 2) k_adj_points(const __grid_constant__ A
 // Acoustic increments (Sec. 6.1 step 1), reversed: Horner in r_s = c tau_s / h,
 // freezing c = sqrt(gamma p / rho), Z = rho c, and the transposed stencils.
 // ---------------------------------------------------------------------------
-// Wrapped neighbourhood of cell (ci, cj): columns ci-1, ci, ci+1 and row
-// offsets (cj-1) nx, cj nx, (cj+1) nx; a lattice offset resolves at compile
-// time to one of them.
-struct Nbhd {
-  int col[3];
-  size_t row[3];
-  __device__ __forceinline__ size_t at(int dc, int dr) const { return row[dr + 1] + col[dc + 1]; }
-};
-
-__device__ __forceinline__ Nbhd nbhd(int ci, int cj, int nx, int ny) {
-  Nbhd b;
-  b.col[1] = ci;
-  b.col[0] = ci == 0 ? nx - 1 : ci - 1;
-  b.col[2] = ci + 1 == nx ? 0 : ci + 1;
-  const int rm = cj == 0 ? ny - 1 : cj - 1, rp = cj + 1 == ny ? 0 : cj + 1;
-  b.row[0] = (size_t)rm * nx;
-  b.row[1] = (size_t)cj * nx;
-  b.row[2] = (size_t)rp * nx;
-  return b;
-}
-
 // node values (.p, .u, .v) at lattice offset (dx, dy) from the node of family
 // FAM of the neighbourhood's centre cell
 template <int FAM, typename T>
@@ -592,7 +570,7 @@ __device__ __forceinline__ void acoustic_adj(const AdjView<T>& v, const Acc& acc
   const Nbhd nb = nbhd(i, j, v.nx, v.ny);
   const LoadAdjPUV<FAM, T> ldr = {&v, nb};
   sac_family<FAM, T>(ldr, wk.p, wk.u, wk.v, Gp, Guv);
-  // polynomial coefficients c_o[q] (q = 1..4 stored at 0..3), as in increments_at
+  // polynomial coefficients c_o[q] (q = 1..4 stored at 0..3), as in acoustic_node
   T co[3][4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {

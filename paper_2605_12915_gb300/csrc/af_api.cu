@@ -42,7 +42,7 @@ struct af_handle {
   void* arena;           // all device planes of this handle
   void* state[2][20];    // ping-pong state planes: 16 (+4 lo)
   int cur;               // index of the current state
-  void* scratch[48];     // wc 4, inc 24, half 12, fx 4, gy 4
+  void* scratch[44];     // wc 4, inc 24, half 12, fx 4
   double* staging;       // 16 FP64 planes for host/device exchange (lazy)
   unsigned* d_flags;
   unsigned* h_flags;     // pinned mirror, written asynchronously after each step
@@ -211,12 +211,12 @@ StepArgs<T> step_args(af_handle* h, double dt) {
   for (int f = 0; f < 3; ++f)
     for (int k = 0; k < 4; ++k) a.half[f][k] = (T*)h->scratch[s++];
   for (int k = 0; k < 4; ++k) a.fx[k] = (T*)h->scratch[s++];
-  for (int k = 0; k < 4; ++k) a.gy[k] = (T*)h->scratch[s++];
   a.flags = h->d_flags;
   a.nx = h->nx;
   a.ny = h->ny;
   a.h = (T)h->h;
   a.dt = (T)dt;
+  a.dth = a.dt / a.h;
   a.gas.gamma = (T)h->gamma;
   a.gas.gm1 = (T)(h->gamma - 1.0);
   a.gas.gm1inv = (T)(1.0 / (h->gamma - 1.0));
@@ -229,30 +229,22 @@ StepArgs<T> step_args(af_handle* h, double dt) {
   return a;
 }
 
-template <typename T, bool COMP>
-void launch_ref_step(af_handle* h, double dt) {
-  StepArgs<T> a = step_args<T>(h, dt);
-  dim3 blk(32, 8), grd((h->nx + 31) / 32, (h->ny + 7) / 8);
-  cudaStream_t s = h->stream;
-  if constexpr (std::is_same<T, double>::value) {
-    if (h->var == AF_FC) {  // foot-centred: no nodal increments, points from the foot disks
-      k_center<T, COMP><<<grd, blk, 0, s>>>(a);
-      launch_fc_points(a, s);
-      k_flux<T><<<grd, blk, 0, s>>>(a);
-      k_average<T, COMP><<<grd, blk, 0, s>>>(a);
-      return;
-    }
+// One foot-centred step: no nodal increments, points from the foot disks, the
+// nodes' fluxes kept in the increment planes.
+void launch_fc_step(af_handle* h, double dt) {
+  const StepArgs<double> a = step_args<double>(h, dt);
+  const unsigned b = ref_blocks(a);
+  NodeFlux<double> n;
+  for (int k = 0; k < 4; ++k) {
+    n.vx[k] = (double*)h->scratch[4 + k];
+    n.vy[k] = (double*)h->scratch[8 + k];
+    n.ex[k] = (double*)h->scratch[12 + k];
+    n.ey[k] = (double*)h->scratch[16 + k];
   }
-  k_center<T, COMP><<<grd, blk, 0, s>>>(a);
-  k_acoustic<0, T><<<grd, blk, 0, s>>>(a);
-  k_acoustic<1, T><<<grd, blk, 0, s>>>(a);
-  k_acoustic<2, T><<<grd, blk, 0, s>>>(a);
-  k_acoustic<3, T><<<grd, blk, 0, s>>>(a);
-  k_points<0, T><<<grd, blk, 0, s>>>(a);
-  k_points<1, T><<<grd, blk, 0, s>>>(a);
-  k_points<2, T><<<grd, blk, 0, s>>>(a);
-  k_flux<T><<<grd, blk, 0, s>>>(a);
-  k_average<T, COMP><<<grd, blk, 0, s>>>(a);
+  launch_dependent(k_center<double, false>, dim3(b), REF_THREADS, 0, h->stream, a);
+  launch_fc_points(a, h->stream);
+  launch_dependent(k_node_flux<double>, dim3(b), REF_THREADS, 0, h->stream, a, n);
+  launch_dependent(k_average<double, false>, dim3(b), REF_THREADS, 0, h->stream, a, n);
 }
 
 // One fused FP32 step on the handle's tile geometry.
@@ -278,7 +270,12 @@ void launch_fused(af_handle* h, double dt) {
 
 void launch_step(af_handle* h, double dt) {
   switch (h->prec) {
-    case AF_FP64: launch_ref_step<double, false>(h, dt); break;
+    case AF_FP64:
+      if (h->var == AF_FC)
+        launch_fc_step(h, dt);
+      else
+        launch_ref_step<double, false>(step_args<double>(h, dt), h->stream);
+      break;
     case AF_FP32:
     case AF_FP32_COMP:
       if (h->fused) {
@@ -287,9 +284,9 @@ void launch_step(af_handle* h, double dt) {
         else
           launch_fused<false>(h, dt);
       } else if (h->prec == AF_FP32_COMP) {
-        launch_ref_step<float, true>(h, dt);
+        launch_ref_step<float, true>(step_args<float>(h, dt), h->stream);
       } else {
-        launch_ref_step<float, false>(h, dt);
+        launch_ref_step<float, false>(step_args<float>(h, dt), h->stream);
       }
       break;
   }
@@ -552,14 +549,7 @@ af_status adjoint_impl(af_handle* h, double dt, const af_state_f64* lin, const a
     }
   }
   if (!fused_inter) {
-    k_center<T, COMP><<<grd, blk, 0, s>>>(f);
-    k_acoustic<0, T><<<grd, blk, 0, s>>>(f);
-    k_acoustic<1, T><<<grd, blk, 0, s>>>(f);
-    k_acoustic<2, T><<<grd, blk, 0, s>>>(f);
-    k_acoustic<3, T><<<grd, blk, 0, s>>>(f);
-    k_points<0, T><<<grd, blk, 0, s>>>(f);
-    k_points<1, T><<<grd, blk, 0, s>>>(f);
-    k_points<2, T><<<grd, blk, 0, s>>>(f);
+    if (launch_ref_intermediates<T, COMP>(f, s) != cudaSuccess) return cuda_fail(h);
   }
   // reverse sweep: the centre and increment records start at zero (planes
   // LAM_NODE + 12 ... LAM_INC + 31 are contiguous; the sweep writes the other
@@ -661,9 +651,9 @@ af_status af_init(af_handle** out, const af_grid* g, double gamma, const af_stat
     const char* lw = getenv("AF_TEST_LATE_WAIT");
     h->late_once = (lw && lw[0] == '1') ? 1 : 0;
   }
-  // 2 x 20 state planes + 48 scratch planes, each padded to 256 bytes
+  // 2 x 20 state planes + 44 scratch planes, each padded to 256 bytes
   size_t plane = (h->N * h->esize + 255) & ~(size_t)255;
-  size_t nplanes = 2 * 20 + 48;
+  size_t nplanes = 2 * 20 + 44;
   if (cudaMalloc(&h->arena, plane * nplanes) != cudaSuccess) {
     delete h;
     return AF_ERR_ALLOC;
@@ -671,7 +661,7 @@ af_status af_init(af_handle** out, const af_grid* g, double gamma, const af_stat
   char* base = (char*)h->arena;
   for (int s = 0; s < 2; ++s)
     for (int p = 0; p < 20; ++p) h->state[s][p] = base + plane * (size_t)(20 * s + p);
-  for (int p = 0; p < 48; ++p) h->scratch[p] = base + plane * (size_t)(40 + p);
+  for (int p = 0; p < 44; ++p) h->scratch[p] = base + plane * (size_t)(40 + p);
   h->red_blocks = 152 * 4;
   bool ok = cudaMalloc(&h->d_flags, sizeof(unsigned)) == cudaSuccess &&
             cudaMallocHost(&h->h_flags, sizeof(unsigned)) == cudaSuccess &&
@@ -969,10 +959,9 @@ af_status af_reduce_invariants(af_handle* h, double* out) {
   if (wait_outgoing(h) != AF_OK) return AF_ERR_CUDA;
   double* partial = h->d_red;
   double* res = h->d_red + (size_t)RED_VALS * h->red_blocks;
-  dim3 blk(32, 8), grd((h->nx + 31) / 32, (h->ny + 7) / 8);
   if (h->prec == AF_FP64) {
     StepArgs<double> a = step_args<double>(h, 1.0);
-    k_center<double, false><<<grd, blk, 0, h->stream>>>(a);
+    k_center<double, false><<<ref_blocks(a), REF_THREADS, 0, h->stream>>>(a);
     RedArgs<double> r;
     r.st = a.in;
     for (int k = 0; k < 4; ++k) r.wc[k] = a.wc[k];
@@ -987,10 +976,10 @@ af_status af_reduce_invariants(af_handle* h, double* out) {
     r.nx = h->nx; r.ny = h->ny; r.gamma = h->gamma; r.h = h->h; r.partial = partial;
     r.rho_ref = h->rho_ref; r.p_ref = h->p_ref; r.e_ref = h->p_ref / (h->gamma - 1.0);
     if (h->prec == AF_FP32_COMP) {
-      k_center<float, true><<<grd, blk, 0, h->stream>>>(a);
+      k_center<float, true><<<ref_blocks(a), REF_THREADS, 0, h->stream>>>(a);
       k_inv_partial<float, true><<<h->red_blocks, RED_THREADS, 0, h->stream>>>(r);
     } else {
-      k_center<float, false><<<grd, blk, 0, h->stream>>>(a);
+      k_center<float, false><<<ref_blocks(a), REF_THREADS, 0, h->stream>>>(a);
       k_inv_partial<float, false><<<h->red_blocks, RED_THREADS, 0, h->stream>>>(r);
     }
   }

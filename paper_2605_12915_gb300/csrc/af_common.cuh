@@ -54,6 +54,48 @@ struct Gas {
   T rho_ref, p_ref;
 };
 
+// The absolute value of a stored offset.  In FP64 the offsets' reference is 0 and
+// the value is the stored one (no addition).
+__device__ __forceinline__ float with_ref(float ref, float x) { return ref + x; }
+__device__ __forceinline__ double with_ref(double, double x) { return x; }
+
+// Tests on the bits of a double: a comparison is an instruction of the FP64 unit,
+// which takes 64 cycles for a warp here (two lanes per cycle and SM), an integer
+// one takes one or two.  Same answers as the comparisons, NaN included.
+__device__ __forceinline__ bool is_positive(float x) { return x > 0.f; }
+__device__ __forceinline__ bool is_positive(double x) {
+  const long long b = __double_as_longlong(x);
+  return b > 0 && b <= 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool is_finite(float x) { return isfinite(x); }
+__device__ __forceinline__ bool is_finite(double x) {
+  return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
+}
+// |x| > lim for a positive finite lim (false for NaN)
+__device__ __forceinline__ bool abs_above(float x, float lim) { return fabsf(x) > lim; }
+__device__ __forceinline__ bool abs_above(double x, double lim) {
+  const long long b = __double_as_longlong(x) & 0x7fffffffffffffffll;
+  return b > __double_as_longlong(lim) && b <= 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool is_negative(float x) { return x < 0.f; }
+__device__ __forceinline__ bool is_negative(double x) {
+  const long long b = __double_as_longlong(x);
+  return b < 0 && b != (long long)0x8000000000000000ull;
+}
+__device__ __forceinline__ bool at_least_one(float x) { return x >= 1.f; }
+__device__ __forceinline__ bool at_least_one(double x) { return __double2hiint(x) >= 0x3ff00000; }
+
+__device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double rsqrt_t(double x) { return rsqrt(x); }
+
+// Programmatic dependent launch: the next kernel of the stream may be scheduled
+// now (its blocks then sit in pdl_wait), and this one's input is complete.  A
+// kernel launched without the attribute passes both at once.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // The helpers below spell out their fused multiply-adds: the library is built
 // without contraction, so every copy of an expression rounds the same way (a
 // value computed by two thread blocks must agree bitwise for conservation).
@@ -62,7 +104,7 @@ struct Gas {
 // (rho~, u, v, p~): E~ = E - p_ref/(gamma-1) = p~/(gamma-1) + rho |u|^2 / 2
 template <typename T>
 __device__ __forceinline__ void cons_from_stored(const Prim<T>& w, const Gas<T>& g, T u[4]) {
-  const T rho = g.rho_ref + w.r;
+  const T rho = with_ref(g.rho_ref, w.r);
   u[0] = w.r;
   u[1] = rho * w.u;
   u[2] = rho * w.v;
@@ -82,14 +124,14 @@ __device__ __forceinline__ Prim<T> stored_from_cons_inv(const T u[4], const Gas<
 
 template <typename T>
 __device__ __forceinline__ Prim<T> stored_from_cons(const T u[4], const Gas<T>& g) {
-  return stored_from_cons_inv(u, g, T(1) / (g.rho_ref + u[0]));
+  return stored_from_cons_inv(u, g, T(1) / with_ref(g.rho_ref, u[0]));
 }
 
 // Euler fluxes F (x) and G (y) of a stored primitive.  The constant p_ref is
 // left out of the momentum fluxes: it cancels in every flux difference.
 template <typename T>
 __device__ __forceinline__ void flux_x(const Prim<T>& w, const Gas<T>& g, T f[4]) {
-  const T rho = g.rho_ref + w.r, p = g.p_ref + w.p;
+  const T rho = with_ref(g.rho_ref, w.r), p = with_ref(g.p_ref, w.p);
   const T m = rho * w.u;
   f[0] = m;
   f[1] = fma(m, w.u, w.p);
@@ -99,7 +141,7 @@ __device__ __forceinline__ void flux_x(const Prim<T>& w, const Gas<T>& g, T f[4]
 
 template <typename T>
 __device__ __forceinline__ void flux_y(const Prim<T>& w, const Gas<T>& g, T f[4]) {
-  const T rho = g.rho_ref + w.r, p = g.p_ref + w.p;
+  const T rho = with_ref(g.rho_ref, w.r), p = with_ref(g.p_ref, w.p);
   const T m = rho * w.v;
   f[0] = m;
   f[1] = m * w.u;
@@ -141,21 +183,6 @@ struct LatticeG {
     w.v = f[fam][2][id];
     w.p = f[fam][3][id];
     return w;
-  }
-};
-
-// Global-memory view of lattice increments (du, dv, dp) per family.
-template <typename T>
-struct IncrG {
-  const T* f[4][3];
-  int nx, ny;
-  __device__ __forceinline__ void at(int I, int J, T d[3]) const {
-    int fam = lattice_family(I, J);
-    int i = wrapi(I >> 1, nx), j = wrapi(J >> 1, ny);
-    size_t id = (size_t)j * nx + i;
-    d[0] = f[fam][0][id];
-    d[1] = f[fam][1][id];
-    d[2] = f[fam][2][id];
   }
 };
 

@@ -644,7 +644,7 @@ __device__ __forceinline__ bool fused_tile(const StepArgs<float>& a, PipeCtx& pc
       // pressure increment dp (the velocity increments are only ever added to
       // the interpolated velocity, so they are interpolated together with it)
       // r-polynomial coefficients of (du, dv, dp), shared by both durations
-      // (the same operations as increments_at)
+      // (the same operations as acoustic_node)
       float cu[4], cv[4], cp[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -657,7 +657,7 @@ __device__ __forceinline__ bool fused_tile(const StepArgs<float>& a, PipeCtx& pc
         d[0] = r * fmaf(r, fmaf(r, fmaf(r, cu[3], cu[2]), cu[1]), cu[0]);
         d[1] = r * fmaf(r, fmaf(r, fmaf(r, cv[3], cv[2]), cv[1]), cv[0]);
       };
-      float d[3];
+      float d[3] = {0.f, 0.f, 0.f};
       float2* D0 = reinterpret_cast<float2*>(D + fam * 3 * DPL) + dc;
       float2* D1 = reinterpret_cast<float2*>(D + (4 + fam) * 3 * DPL) + dc;
       float* D0p = D + fam * 3 * DPL + 2 * DPL + dc;
@@ -666,16 +666,20 @@ __device__ __forceinline__ bool fused_tile(const StepArgs<float>& a, PipeCtx& pc
       const int gi = i0 - 1 + dx, gj = j0 - 1 + dy;
       const bool own = INTER && dx >= 1 && dx <= TX && dy >= 1 && dy <= TY && gi < nx && gj < ny;
       const size_t gid = own ? (size_t)gj * nx + gi : 0;
+      auto store = [&](int s, float2* Duv, float* Dp) {
+        const float2 uv = make_float2(wk.x + d[0], wk.y + d[1]);
+        *Duv = uv;
+        *Dp = d[2];
+        if (own) {
+          a.inc[s][fam][0][gid] = uv.x;
+          a.inc[s][fam][1][gid] = uv.y;
+          a.inc[s][fam][2][gid] = d[2];
+        }
+      };
       horner(0.5f * r1, d);
-      *D0 = make_float2(wk.x + d[0], wk.y + d[1]);
-      *D0p = d[2];
-      if (own)
-        for (int k = 0; k < 3; ++k) a.inc[0][fam][k][gid] = d[k];
+      store(0, D0, D0p);
       horner(r1, d);
-      *D1 = make_float2(wk.x + d[0], wk.y + d[1]);
-      *D1p = d[2];
-      if (own)
-        for (int k = 0; k < 3; ++k) a.inc[1][fam][k][gid] = d[k];
+      store(1, D1, D1p);
     }
   }
   __syncthreads();
@@ -929,14 +933,6 @@ __device__ __forceinline__ bool fused_tile(const StepArgs<float>& a, PipeCtx& pc
   }
   if (bad) atomicOr(a.flags, bad);
   return true;
-}
-
-// Programmatic dependent launch: the next kernel of the stream may be scheduled
-// now (its blocks then sit in pdl_wait), and this one's input is complete.  A
-// kernel launched without the attribute passes both at once.
-__device__ __forceinline__ void pdl_wait() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 template <int TX, int TY, int NT, int MINB, bool COMP>

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "af_fused.cuh"
+#include "af_ref_launch.cuh"
 
 namespace af {
 
@@ -67,26 +68,6 @@ inline bool encode_tile_maps(const StepArgs<float>& a, TileMaps* out, int ty = F
       return false;
   }
   return true;
-}
-
-// Launches `kern` so that it may be scheduled while the stream's previous kernel
-// drains (programmatic dependent launch); the kernel itself waits for that
-// kernel's results (pdl_wait) before it touches memory.  Saves the launch gap
-// between steps: 8.35 -> 6.54 us per step at 64 x 64 cells, 18.6 -> 16.8 at 256^2.
-template <typename... P, typename... A>
-inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int threads, size_t smem,
-                                    cudaStream_t s, const A&... args) {
-  cudaLaunchConfig_t c = {};
-  c.gridDim = grid;
-  c.blockDim = dim3(threads);
-  c.dynamicSmemBytes = smem;
-  c.stream = s;
-  cudaLaunchAttribute at[1] = {};
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  c.attrs = at;
-  c.numAttrs = 1;
-  return cudaLaunchKernelEx(&c, kern, args...);
 }
 
 // One CTA per tile of TX x TY cells.

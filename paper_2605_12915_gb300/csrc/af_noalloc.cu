@@ -5,7 +5,7 @@
 // that owns every allocation on the device and forbids stray cudaMalloc calls.
 // For them this entry point runs the FP64 multi-kernel step on buffers the
 // caller provides, and keeps its intermediate values (recovered centres,
-// acoustic increments, half-step point values, edge fluxes, error word) in one
+// acoustic increments, node fluxes, error word) in one
 // fixed work area compiled into this library: a file-scope __device__ array
 // that every GPU loading the library holds until the process exits.
 #include <cuda_runtime.h>
@@ -13,7 +13,7 @@
 #include <mutex>
 
 #include "../../include/af.h"
-#include "af_ref_kernels.cuh"
+#include "af_ref_launch.cuh"
 #include "af_state_util.h"
 
 using namespace af;
@@ -21,8 +21,8 @@ using namespace af;
 namespace {
 
 constexpr size_t kMaxCells = AF_NOALLOC_MAX_CELLS;
-// planes: centres 4, increments 2 x 4 x 3, half-step points 3 x 4, fluxes 4 + 4
-constexpr size_t kPlanes = 4 + 24 + 12 + 8;
+// planes: centres 4, increments 2 x 4 x 3, node fluxes 3 x 4 + 4
+constexpr size_t kPlanes = 4 + 24 + 12 + 4;
 constexpr size_t kFlagsOffset = kPlanes * kMaxCells;  // in doubles, 256-byte aligned
 constexpr size_t kWords = kFlagsOffset + 32;
 
@@ -111,15 +111,12 @@ extern "C" af_status af_step_noalloc(const af_grid* g, double gamma, double dt, 
     a.fx[k] = p;
     p += N;
   }
-  for (int k = 0; k < 4; ++k) {
-    a.gy[k] = p;
-    p += N;
-  }
   a.flags = reinterpret_cast<unsigned*>(work + kFlagsOffset);
   a.nx = g->nx;
   a.ny = g->ny;
   a.h = g->h;
   a.dt = dt;
+  a.dth = dt / g->h;
   a.gas.gamma = gamma;
   a.gas.gm1 = gamma - 1.0;
   a.gas.gm1inv = 1.0 / (gamma - 1.0);
@@ -133,17 +130,7 @@ extern "C" af_status af_step_noalloc(const af_grid* g, double gamma, double dt, 
   cudaStream_t s = (cudaStream_t)cuda_stream;
   // the work area keeps the previous call's contents: the error word must start at 0
   if (cudaMemsetAsync(a.flags, 0, sizeof(unsigned), s) != cudaSuccess) return AF_ERR_CUDA;
-  dim3 blk(32, 8), grd((g->nx + 31) / 32, (g->ny + 7) / 8);
-  k_center<double, false><<<grd, blk, 0, s>>>(a);
-  k_acoustic<0, double><<<grd, blk, 0, s>>>(a);
-  k_acoustic<1, double><<<grd, blk, 0, s>>>(a);
-  k_acoustic<2, double><<<grd, blk, 0, s>>>(a);
-  k_acoustic<3, double><<<grd, blk, 0, s>>>(a);
-  k_points<0, double><<<grd, blk, 0, s>>>(a);
-  k_points<1, double><<<grd, blk, 0, s>>>(a);
-  k_points<2, double><<<grd, blk, 0, s>>>(a);
-  k_flux<double><<<grd, blk, 0, s>>>(a);
-  k_average<double, false><<<grd, blk, 0, s>>>(a);
+  if (launch_ref_step<double, false>(a, s) != cudaSuccess) return AF_ERR_CUDA;
   if (cudaGetLastError() != cudaSuccess) return AF_ERR_CUDA;
   unsigned flags = 0;
   if (cudaMemcpyAsync(&flags, a.flags, sizeof(unsigned), cudaMemcpyDeviceToHost, s) !=

@@ -1,12 +1,27 @@
-// af_ref_kernels.cuh -- the RB-TAI / RB step as separate simple kernels, one
-// thread per cell, intermediate values in global scratch.  It is the FP64
-// path and the reference layout for the fused kernel:
+// af_ref_kernels.cuh -- the RB-TAI / RB step as separate kernels, one thread per
+// node or cell, intermediate values in global scratch.  It is the FP64 path and
+// the reference layout for the fused kernel:
 //   k_center    centre recovery by Simpson inversion        (Eq. center-node)
 //   k_acoustic  node-centred exact acoustic increments      (Sec. 6.1 step 1)
 //   k_points    two-Picard foot + transported / additive    (Sec. 6.1 steps 2-4,
 //               point update at tau = dt/2 and dt           Eq. barsukow-additive)
-//   k_flux      space-time Simpson edge fluxes              (Sec. 3.1, Sec. 6.1)
+//               and the time-integrated fluxes of the node  (Sec. 3.1)
 //   k_average   conservative average update                 (Eq. af-average-update)
+//
+// What bounds them in FP64: the FP64 unit, two lanes per cycle and SM, so a warp
+// instruction holds its scheduler's unit for 64 cycles while everything else
+// (loads, integer work, launches of other warps) is all but free.  Comparisons,
+// conversions, floor and min / max of doubles run on that unit too.  So the FP64
+// instructions are what is counted here: comparisons and floor are done on the
+// bits, 1/Z and c come from one reciprocal square root, increments are kept as
+// (u + du, v + dv, dp) and interpolated together with the velocity (five fields
+// at the foot instead of seven), the nine Q2 weights are formed once, and each
+// node's fluxes are integrated in time once instead of in both edges it bounds.
+// Small grids are bound by the same unit on the few SMs that hold their warps:
+// the families share a launch (blockIdx.y) and blocks are two warps.
+// GB300, FP64: a step at 512^2 takes 1.01 ms (1.40 with ten launches, comparisons
+// and floor in FP64, separate increments and per-edge fluxes); a whole
+// set-step-get call at 32^2 from pinned host memory 91 us (277).
 #pragma once
 
 #include "af_common.cuh"
@@ -19,19 +34,22 @@ struct StepArgs {
   Planes<T> in;       // state at t^n
   Planes<T> out;      // state at t^{n+1}
   T* wc[4];           // recovered centre (rho, u, v, p)
-  T* inc[2][4][3];    // [tau index][family V,Ev,Eh,C][du, dv, dp]
-  T* half[3][4];      // point values at t^n + dt/2, [family][rho,u,v,p]
-  T* fx[4];           // (dt/h) * time-integrated flux through vertical edge (i,j)
-  T* gy[4];           // (dt/h) * time-integrated flux through horizontal edge (i,j)
+  T* inc[2][4][3];    // [tau index][family V,Ev,Eh,C][u + du, v + dv, dp]
+  T* half[3][4];      // point values at t^n + dt/2, [family][rho,u,v,p] (adjoint and AF_FC);
+                      // the step keeps the fluxes of the vertices (x, then y) and of the
+                      // x-edge midpoints there
+  T* fx[4];           // fluxes of the y-edge midpoints
   unsigned* flags;
   int nx, ny;
-  T h, dt;
+  T h, dt, dth;       // dth = dt / h
   Gas<T> gas;
   int variant;        // 0 TAI, 1 RB
   int prefetch_wave;  // fused kernel: blocks per wave for the L2 prefetch (0: none)
   int late_first_wait;  // pipelined kernels, testing only: each CTA's first wait for a
                         // tensor-copied tile reports a timeout at once (0: off)
 };
+
+constexpr int REF_THREADS = 64;
 
 template <typename T>
 __device__ __forceinline__ LatticeG<T> lattice_of(const StepArgs<T>& a) {
@@ -48,23 +66,62 @@ __device__ __forceinline__ void raise_flag(unsigned* flags, unsigned bits) {
   if (bits) atomicOr(flags, bits);
 }
 
+// family of lattice offset (a, b) from a cell's vertex: V, E_v, E_h, C
+__host__ __device__ constexpr int fam_of(int a, int b) {
+  return (a & 1) ? ((b & 1) ? 3 : 2) : ((b & 1) ? 1 : 0);
+}
+
+// the calling thread's cell (false: beyond the grid)
+template <typename T>
+__device__ __forceinline__ bool cell_of_thread(const StepArgs<T>& a, int& i, int& j, size_t& id) {
+  id = (size_t)blockIdx.x * REF_THREADS + threadIdx.x;
+  if (id >= (size_t)a.nx * a.ny) return false;
+  j = (int)(id / (unsigned)a.nx);
+  i = (int)(id - (size_t)j * a.nx);
+  return true;
+}
+
+// Wrapped neighbourhood of cell (ci, cj): columns ci-1, ci, ci+1 and row
+// offsets (cj-1) nx, cj nx, (cj+1) nx; a lattice offset resolves at compile
+// time to one of them.
+struct Nbhd {
+  int col[3];
+  size_t row[3];
+  __device__ __forceinline__ size_t at(int dc, int dr) const { return row[dr + 1] + col[dc + 1]; }
+};
+
+__device__ __forceinline__ Nbhd nbhd(int ci, int cj, int nx, int ny) {
+  Nbhd b;
+  b.col[1] = ci;
+  b.col[0] = ci == 0 ? nx - 1 : ci - 1;
+  b.col[2] = ci + 1 == nx ? 0 : ci + 1;
+  const int rm = cj == 0 ? ny - 1 : cj - 1, rp = cj + 1 == ny ? 0 : cj + 1;
+  b.row[0] = (size_t)rm * nx;
+  b.row[1] = (size_t)cj * nx;
+  b.row[2] = (size_t)rp * nx;
+  return b;
+}
+
 // ---------------------------------------------------------------------------
-// Centre recovery (Eq. center-node) in the algebraically equal deviation form
-// U_c = Ubar + 1/16 sum_corners (Ubar - U_V) + 1/4 sum_edges (Ubar - U_E).
+// Centre recovery (Eq. center-node).  FP32 in the deviation form
+// U_c = Ubar + 1/16 sum_corners (Ubar - U_V) + 1/4 sum_edges (Ubar - U_E), which
+// keeps the cancellation small; FP64 as U_c = 9/4 Ubar - sum_corners U_V / 16 -
+// sum_edges U_E / 4 (half the operations).
 // ---------------------------------------------------------------------------
 template <typename T, bool COMP>
-__global__ void k_center(StepArgs<T> a) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  int j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i >= a.nx || j >= a.ny) return;
-  int ip = wrapi(i + 1, a.nx), jp = wrapi(j + 1, a.ny);
-  size_t id = (size_t)j * a.nx + i;
+__global__ void __launch_bounds__(REF_THREADS) k_center(const __grid_constant__ StepArgs<T> a) {
+  pdl_wait();
+  int i, j;
+  size_t id;
+  if (!cell_of_thread(a, i, j, id)) return;
+  const int ip = i + 1 == a.nx ? 0 : i + 1, jp = j + 1 == a.ny ? 0 : j + 1;
   auto P = [&](int f, int ii, int jj) {
     size_t q = (size_t)jj * a.nx + ii;
     Prim<T> w = {a.in.pt[f][0][q], a.in.pt[f][1][q], a.in.pt[f][2][q], a.in.pt[f][3][q]};
     return w;
   };
   T ub[4], lo[4], uc[4], c[4], e[4];
+#pragma unroll
   for (int k = 0; k < 4; ++k) {
     ub[k] = a.in.avg[k][id];
     lo[k] = COMP ? a.in.lo[k][id] : T(0);
@@ -73,34 +130,64 @@ __global__ void k_center(StepArgs<T> a) {
   }
   const Prim<T> corners[4] = {P(0, i, j), P(0, ip, j), P(0, i, jp), P(0, ip, jp)};
   const Prim<T> edges[4] = {P(2, i, j), P(2, i, jp), P(1, i, j), P(1, ip, j)};
-  for (int n = 0; n < 4; ++n) {
+  if constexpr (sizeof(T) == 8) {
     T u[4];
-    cons_from_stored(corners[n], a.gas, u);
-    for (int k = 0; k < 4; ++k) c[k] += (ub[k] - u[k]) + lo[k];
-    cons_from_stored(edges[n], a.gas, u);
-    for (int k = 0; k < 4; ++k) e[k] += (ub[k] - u[k]) + lo[k];
+    cons_from_stored(corners[0], a.gas, c);
+    cons_from_stored(edges[0], a.gas, e);
+#pragma unroll
+    for (int n = 1; n < 4; ++n) {
+      cons_from_stored(corners[n], a.gas, u);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) c[k] += u[k];
+      cons_from_stored(edges[n], a.gas, u);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) e[k] += u[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      uc[k] = fma(T(2.25), ub[k], fma(T(-0.0625), c[k], T(-0.25) * e[k]));
+  } else {
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+      T u[4];
+      cons_from_stored(corners[n], a.gas, u);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) c[k] += (ub[k] - u[k]) + lo[k];
+      cons_from_stored(edges[n], a.gas, u);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) e[k] += (ub[k] - u[k]) + lo[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      uc[k] = (ub[k] + lo[k]) + (T(0.0625) * c[k] + T(0.25) * e[k]);
   }
-  for (int k = 0; k < 4; ++k) uc[k] = (ub[k] + lo[k]) + (T(0.0625) * c[k] + T(0.25) * e[k]);
   Prim<T> w = stored_from_cons(uc, a.gas);
   a.wc[0][id] = w.r;
   a.wc[1][id] = w.u;
   a.wc[2][id] = w.v;
   a.wc[3][id] = w.p;
-  raise_flag(a.flags, (a.gas.rho_ref + w.r > T(0) && a.gas.p_ref + w.p > T(0)) ? 0u
-                                                                             : FLAG_NONPHYSICAL);
+  raise_flag(a.flags, (is_positive(with_ref(a.gas.rho_ref, w.r)) &&
+                       is_positive(with_ref(a.gas.p_ref, w.p)))
+                          ? 0u
+                          : FLAG_NONPHYSICAL);
 }
 
 // ---------------------------------------------------------------------------
-// Exact frozen acoustic increments at the nodes of one family, for tau = dt/2
-// and tau = dt (Sec. 6.1 step 1).  The r^q sums are shared by both durations.
+// Exact frozen acoustic increments of the nodes of the family blockIdx.y, for
+// tau = dt/2 and tau = dt (Sec. 6.1 step 1).  The r^q sums are shared by both.
 // ---------------------------------------------------------------------------
-template <typename T>
+// node values (.p, .u, .v) at lattice offset (dx, dy) from the node of family
+// FAM of the neighbourhood's centre cell
+template <int FAM, typename T>
 struct LoadPUV {
-  const LatticeG<T>* L;
-  int I, J;
+  const StepArgs<T>* a;
+  Nbhd b;
   __device__ __forceinline__ PUV<T> operator()(int dx, int dy) const {
-    Prim<T> w = L->at(I + dx, J + dy);
-    PUV<T> o = {w.p, w.u, w.v};
+    const int ax = ((FAM == 2 || FAM == 3) ? 1 : 0) + dx, by = ((FAM == 1 || FAM == 3) ? 1 : 0) + dy;
+    const int f = fam_of(ax, by);
+    const size_t q = b.at(ax >> 1, by >> 1);
+    T* const* pl = f < 3 ? a->in.pt[f] : a->wc;
+    PUV<T> o = {pl[3][q], pl[1][q], pl[2][q]};
     return o;
   }
 };
@@ -108,16 +195,28 @@ struct LoadPUV {
 template <int FAM, typename T, typename Load>
 __device__ __forceinline__ void sac_family(const Load& L, T pK, T uK, T vK, T Gp[3][4],
                                            T Guv[3][4]) {
-  if (FAM == 0) af_sac_V<T>(L, pK, uK, vK, Gp, Guv);
-  if (FAM == 1) af_sac_EV<T>(L, pK, uK, vK, Gp, Guv);
-  if (FAM == 2) af_sac_EH<T>(L, pK, uK, vK, Gp, Guv);
-  if (FAM == 3) af_sac_C<T>(L, pK, uK, vK, Gp, Guv);
+  if constexpr (FAM == 0) af_sac_V<T>(L, pK, uK, vK, Gp, Guv);
+  if constexpr (FAM == 1) af_sac_EV<T>(L, pK, uK, vK, Gp, Guv);
+  if constexpr (FAM == 2) af_sac_EH<T>(L, pK, uK, vK, Gp, Guv);
+  if constexpr (FAM == 3) af_sac_C<T>(L, pK, uK, vK, Gp, Guv);
 }
 
-// Horner evaluation of the increments: dp = sum_q r^q (Gp0 + Z Guv0), etc.
-template <typename T>
-__device__ __forceinline__ void increments_at(const T Gp[3][4], const T Guv[3][4], T Z, T Zinv,
-                                              T r, T d[3]) {
+template <int FAM, typename T>
+__device__ __forceinline__ void acoustic_node(const StepArgs<T>& a, int i, int j, size_t id) {
+  T* const* own = FAM < 3 ? a.in.pt[FAM < 3 ? FAM : 0] : a.wc;
+  const Prim<T> wk = {own[0][id], own[1][id], own[2][id], own[3][id]};
+  unsigned bad = 0;
+  const T rk = with_ref(a.gas.rho_ref, wk.r), pk = with_ref(a.gas.p_ref, wk.p);
+  if (!(is_positive(rk) && is_positive(pk))) bad |= FLAG_NONPHYSICAL;
+  // Z^2 = gamma p rho, c = gamma p / Z
+  const T gp = a.gas.gamma * pk, z2 = gp * rk;
+  const T Zinv = rsqrt_t(z2), Z = z2 * Zinv, c = gp * Zinv;
+  const T r1 = c * a.dth;
+  if (abs_above(r1, T(0.5))) bad |= FLAG_CFL;
+  T Gp[3][4], Guv[3][4];
+  const LoadPUV<FAM, T> ld = {&a, nbhd(i, j, a.nx, a.ny)};
+  sac_family<FAM, T>(ld, wk.p, wk.u, wk.v, Gp, Guv);
+  // polynomial coefficients: dp = sum_q r^q (Gp0 + Z Guv0), du = sum_q r^q (Gp1 / Z + Guv1)
   T cp[4], cu[4], cv[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
@@ -125,39 +224,28 @@ __device__ __forceinline__ void increments_at(const T Gp[3][4], const T Guv[3][4
     cu[q] = fma(Zinv, Gp[1][q], Guv[1][q]);
     cv[q] = fma(Zinv, Gp[2][q], Guv[2][q]);
   }
-  d[2] = r * fma(r, fma(r, fma(r, cp[3], cp[2]), cp[1]), cp[0]);
-  d[0] = r * fma(r, fma(r, fma(r, cu[3], cu[2]), cu[1]), cu[0]);
-  d[1] = r * fma(r, fma(r, fma(r, cv[3], cv[2]), cv[1]), cv[0]);
-}
-
-template <int FAM, typename T>
-__global__ void k_acoustic(StepArgs<T> a) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  int j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i >= a.nx || j >= a.ny) return;
-  LatticeG<T> L = lattice_of(a);
-  const int I = 2 * i + ((FAM == 2 || FAM == 3) ? 1 : 0);
-  const int J = 2 * j + ((FAM == 1 || FAM == 3) ? 1 : 0);
-  Prim<T> wk = L.at(I, J);
-  unsigned bad = 0;
-  const T rk = a.gas.rho_ref + wk.r, pk = a.gas.p_ref + wk.p;
-  if (!(rk > T(0) && pk > T(0))) bad |= FLAG_NONPHYSICAL;
-  T c = sqrt(a.gas.gamma * pk / rk);
-  T Z = rk * c, Zinv = T(1) / Z;
-  T r1 = c * a.dt / a.h;
-  if (r1 > T(0.5)) bad |= FLAG_CFL;
-  T Gp[3][4], Guv[3][4];
-  LoadPUV<T> ld = {&L, I, J};
-  sac_family<FAM, T>(ld, wk.p, wk.u, wk.v, Gp, Guv);
-  size_t id = (size_t)j * a.nx + i;
+#pragma unroll
   for (int s = 0; s < 2; ++s) {
-    T d[3];
-    increments_at(Gp, Guv, Z, Zinv, s == 0 ? T(0.5) * r1 : r1, d);
-    a.inc[s][FAM][0][id] = d[0];
-    a.inc[s][FAM][1][id] = d[1];
-    a.inc[s][FAM][2][id] = d[2];
+    const T r = s == 0 ? T(0.5) * r1 : r1;
+    a.inc[s][FAM][0][id] = fma(r, fma(r, fma(r, fma(r, cu[3], cu[2]), cu[1]), cu[0]), wk.u);
+    a.inc[s][FAM][1][id] = fma(r, fma(r, fma(r, fma(r, cv[3], cv[2]), cv[1]), cv[0]), wk.v);
+    a.inc[s][FAM][2][id] = r * fma(r, fma(r, fma(r, cp[3], cp[2]), cp[1]), cp[0]);
   }
   raise_flag(a.flags, bad);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(REF_THREADS) k_acoustic(const __grid_constant__ StepArgs<T> a) {
+  pdl_wait();
+  int i, j;
+  size_t id;
+  if (!cell_of_thread(a, i, j, id)) return;
+  switch (blockIdx.y) {
+    case 0: acoustic_node<0>(a, i, j, id); break;
+    case 1: acoustic_node<1>(a, i, j, id); break;
+    case 2: acoustic_node<2>(a, i, j, id); break;
+    default: acoustic_node<3>(a, i, j, id); break;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -207,147 +295,269 @@ __device__ __forceinline__ Prim<T> eval_w(const LatticeG<T>& L, const FootCell<T
   return s;
 }
 
+// One axis of a foot displaced by d cells from lattice offset O (0 or 1 half
+// cell): the cell offset floor(f), f = O/2 + d, and the local coordinate
+// 2 (f - floor(f)) - 1.  Within the reach (|d| <= 1) floor(f) is -1, 0 or 1,
+// read off the bits; beyond it (flagged by the caller) by floor itself.
+template <int O, typename T>
+__device__ __forceinline__ T foot_coord(T d, int& cell) {
+  const T f = O ? d + T(0.5) : d;
+  if (abs_above(d, T(1)) || !is_finite(d)) {
+    const T fl = floor(f);
+    cell = (int)fl;
+    return fma(T(2), f - fl, T(-1));
+  }
+  const bool neg = is_negative(f), one = at_least_one(f);
+  cell = neg ? -1 : (one ? 1 : 0);
+  return fma(T(2), f, neg ? T(1) : (one ? T(-3) : T(-1)));
+}
+
 template <typename T>
-__device__ __forceinline__ void eval_d(const IncrG<T>& D, const FootCell<T>& c, T out[3]) {
-  T lx[3], ly[3];
-  lagrange3(c.xi, lx);
-  lagrange3(c.eta, ly);
-  out[0] = out[1] = out[2] = T(0);
-  for (int b = 0; b < 3; ++b) {
-    T row[3] = {T(0), T(0), T(0)};
-    for (int q = 0; q < 3; ++q) {
-      T d[3];
-      D.at(2 * c.ci + q, 2 * c.cj + b, d);
-      for (int k = 0; k < 3; ++k) row[k] = fma(lx[q], d[k], row[k]);
-    }
-    for (int k = 0; k < 3; ++k) out[k] = fma(ly[b], row[k], out[k]);
+__device__ __forceinline__ void lagrange3_fma(T s, T l[3]) {
+  const T hs = T(0.5) * s;
+  l[0] = fma(hs, s, -hs);
+  l[1] = fma(-s, s, T(1));
+  l[2] = fma(hs, s, hs);
+}
+
+// the cells (c0, c0 + 1) x (r0, r0 + 1), wrapped, that hold the nine nodes of the
+// cell (i + cx, j + cy): node (q, b) is the family fam_of(q, b) of cell n[b / 2][q / 2]
+struct FootNodes {
+  size_t n[2][2];
+};
+__device__ __forceinline__ FootNodes foot_nodes(int c, int r, int nx, int ny) {
+  if ((unsigned)(c + 1) > (unsigned)nx) c = wrapi(c, nx);  // beyond [-1, nx)
+  if ((unsigned)(r + 1) > (unsigned)ny) r = wrapi(r, ny);
+  c = c < 0 ? c + nx : (c == nx ? 0 : c);
+  r = r < 0 ? r + ny : (r == ny ? 0 : r);
+  const size_t r0 = (size_t)r * nx, r1 = r + 1 == ny ? 0 : r0 + nx;
+  const int c1 = c + 1 == nx ? 0 : c + 1;
+  FootNodes f = {{{r0 + c, r0 + c1}, {r1 + c, r1 + c1}}};
+  return f;
+}
+
+// sum_qb w_qb f_qb with f_qb the plane of the node's family, pl(fam)
+template <typename T, typename Plane>
+__device__ __forceinline__ T nine_sum(const FootNodes& c, const T w[9], const Plane& pl) {
+  T s = w[0] * pl(0)[c.n[0][0]];
+#pragma unroll
+  for (int m = 1; m < 9; ++m) {
+    const int q = m % 3, b = m / 3;
+    s = fma(w[m], pl(fam_of(q, b))[c.n[b >> 1][q >> 1]], s);
+  }
+  return s;
+}
+// the same with separate weights (rows first)
+template <typename T, typename Plane>
+__device__ __forceinline__ T row_sum(const FootNodes& c, const T lx[3], const T ly[3],
+                                     const Plane& pl) {
+  T r[3];
+#pragma unroll
+  for (int b = 0; b < 3; ++b)
+    r[b] = fma(lx[0], pl(fam_of(0, b))[c.n[b >> 1][0]],
+               fma(lx[1], pl(fam_of(1, b))[c.n[b >> 1][0]],
+                   lx[2] * pl(fam_of(2, b))[c.n[b >> 1][1]]));
+  return fma(ly[0], r[0], fma(ly[1], r[1], ly[2] * r[2]));
+}
+
+// Adds wt times the node's fluxes (x for V and E_v, y for V and E_h) to S.
+template <int FAM, typename T>
+__device__ __forceinline__ void add_flux(const Prim<T>& w, const Gas<T>& g, T wt, T S[2][4]) {
+  T f[4];
+  if (FAM != 2) {
+    flux_x(w, g, f);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) S[0][k] = fma(wt, f[k], S[0][k]);
+  }
+  if (FAM != 1) {
+    flux_y(w, g, f);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) S[1][k] = fma(wt, f[k], S[1][k]);
   }
 }
 
-template <int FAM, typename T>
-__global__ void k_points(StepArgs<T> a) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  int j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i >= a.nx || j >= a.ny) return;
-  LatticeG<T> L = lattice_of(a);
-  const int I = 2 * i + (FAM == 2 ? 1 : 0);
-  const int J = 2 * j + (FAM == 1 ? 1 : 0);
-  const Prim<T> wp = L.at(I, J);
-  const T hinv = T(1) / a.h;
-  size_t id = (size_t)j * a.nx + i;
+// Point of family FAM of cell (i, j), both durations.  FLUX: the half-step point
+// stays in registers and the node's fluxes, summed over time with weights
+// 1, 4, 1, are stored; otherwise the half-step point is (for the adjoint).
+template <int FAM, bool FLUX, typename T>
+__device__ __forceinline__ void point_node(const StepArgs<T>& a, int i, int j, size_t id) {
+  const int nx = a.nx, ny = a.ny;
+  const Gas<T>& g = a.gas;
+  constexpr int OX = FAM == 2 ? 1 : 0, OY = FAM == 1 ? 1 : 0;
+  const Prim<T> wp = {a.in.pt[FAM][0][id], a.in.pt[FAM][1][id], a.in.pt[FAM][2][id],
+                      a.in.pt[FAM][3][id]};
   unsigned bad = 0;
+  T S[2][4] = {};
+  if (FLUX) add_flux<FAM>(wp, g, T(1), S);
+#pragma unroll 1
   for (int s = 0; s < 2; ++s) {
-    const T tau = s == 0 ? T(0.5) * a.dt : a.dt;
-    const T th = tau * hinv;
-    IncrG<T> D;
-    for (int f = 0; f < 4; ++f)
-      for (int k = 0; k < 3; ++k) D.f[f][k] = a.inc[s][f][k];
-    D.nx = a.nx;
-    D.ny = a.ny;
+    const T th = s == 0 ? T(0.5) * a.dth : a.dth;
+    auto plane = [&](int k) {
+      return [&a, k](int f) { return f < 3 ? a.in.pt[f][k] : a.wc[k]; };
+    };
+    auto incr = [&](int k) { return [&a, s, k](int f) { return a.inc[s][f][k]; }; };
     // two-Picard convective foot from the time-n reconstruction (Eq. adv-footpoint)
-    T d1x = -th * wp.u, d1y = -th * wp.v;
-    Prim<T> w1 = eval_w(L, locate<T>(I, J, d1x, d1y));
-    T dfx = -th * w1.u, dfy = -th * w1.v;
-    if (fabs(d1x) > T(1) || fabs(d1y) > T(1) || fabs(dfx) > T(1) || fabs(dfy) > T(1))
+    int cx, cy;
+    T lx[3], ly[3];
+    const T d1x = -th * wp.u, d1y = -th * wp.v;
+    lagrange3_fma(foot_coord<OX>(d1x, cx), lx);
+    lagrange3_fma(foot_coord<OY>(d1y, cy), ly);
+    FootNodes c = foot_nodes(i + cx, j + cy, nx, ny);
+    const T dfx = -th * row_sum(c, lx, ly, plane(1)), dfy = -th * row_sum(c, lx, ly, plane(2));
+    if (abs_above(d1x, T(1)) || abs_above(d1y, T(1)) || abs_above(dfx, T(1)) ||
+        abs_above(dfy, T(1)))
       bad |= FLAG_REACH;
-    FootCell<T> fc = locate<T>(I, J, dfx, dfy);
-    Prim<T> wf = eval_w(L, fc);
+    lagrange3_fma(foot_coord<OX>(dfx, cx), lx);
+    lagrange3_fma(foot_coord<OY>(dfy, cy), ly);
+    c = foot_nodes(i + cx, j + cy, nx, ny);
+    T w[9];
+#pragma unroll
+    for (int m = 0; m < 9; ++m) w[m] = lx[m % 3] * ly[m / 3];
+    const T rft = nine_sum(c, w, plane(0)), pft = nine_sum(c, w, plane(3));
     Prim<T> nw;
     if (a.variant == 0) {
-      // transported increment evaluated at the foot; rho from dp / c_f^2
-      T d[3];
-      eval_d(D, fc, d);
-      const T rf = a.gas.rho_ref + wf.r, pf = a.gas.p_ref + wf.p;
-      if (!(rf > T(0) && pf > T(0))) bad |= FLAG_NONPHYSICAL;
-      nw.r = wf.r + d[2] * rf / (a.gas.gamma * pf);
-      nw.u = wf.u + d[0];
-      nw.v = wf.v + d[1];
-      nw.p = wf.p + d[2];
+      // transported increment evaluated at the foot; rho from dp / c_f^2.  The
+      // velocity's increments are interpolated together with it: u_f + du_f =
+      // I_h(u + du)(P_f), both interpolants sharing the basis
+      const T dp = nine_sum(c, w, incr(2));
+      const T rf = with_ref(g.rho_ref, rft), pf = with_ref(g.p_ref, pft);
+      if (!(is_positive(rf) && is_positive(pf))) bad |= FLAG_NONPHYSICAL;
+      nw.r = rft + dp * rf / (g.gamma * pf);
+      nw.u = nine_sum(c, w, incr(0));
+      nw.v = nine_sum(c, w, incr(1));
+      nw.p = pft + dp;
     } else {
       // additive update: S_ac(P) + S_adv(P) - W(P), acoustic rho closure at P
-      T d[3];
-      D.at(I, J, d);
-      nw.r = wf.r + d[2] * (a.gas.rho_ref + wp.r) / (a.gas.gamma * (a.gas.p_ref + wp.p));
-      nw.u = wf.u + d[0];
-      nw.v = wf.v + d[1];
-      nw.p = wf.p + d[2];
+      const T dp = a.inc[s][FAM][2][id];
+      nw.r = rft + dp * with_ref(g.rho_ref, wp.r) / (g.gamma * with_ref(g.p_ref, wp.p));
+      nw.u = nine_sum(c, w, plane(1)) + (a.inc[s][FAM][0][id] - wp.u);
+      nw.v = nine_sum(c, w, plane(2)) + (a.inc[s][FAM][1][id] - wp.v);
+      nw.p = pft + dp;
     }
-    if (!(isfinite(nw.r) && isfinite(nw.u) && isfinite(nw.v) && isfinite(nw.p)))
+    if (!(is_finite(nw.r) && is_finite(nw.u) && is_finite(nw.v) && is_finite(nw.p)))
       bad |= FLAG_NONFINITE;
-    T* const* dst = s == 0 ? a.half[FAM] : a.out.pt[FAM];
-    dst[0][id] = nw.r;
-    dst[1][id] = nw.u;
-    dst[2][id] = nw.v;
-    dst[3][id] = nw.p;
+    if (FLUX) add_flux<FAM>(nw, g, s == 0 ? T(4) : T(1), S);
+    if (s == 1 || !FLUX) {
+      T* const* dst = s == 0 ? a.half[FAM] : a.out.pt[FAM];
+      dst[0][id] = nw.r;
+      dst[1][id] = nw.u;
+      dst[2][id] = nw.v;
+      dst[3][id] = nw.p;
+    }
+  }
+  if (FLUX) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (FAM == 0) {
+        a.half[0][k][id] = S[0][k];
+        a.half[1][k][id] = S[1][k];
+      } else if (FAM == 1) {
+        a.half[2][k][id] = S[0][k];
+      } else {
+        a.fx[k][id] = S[1][k];
+      }
+    }
   }
   raise_flag(a.flags, bad);
 }
 
-// ---------------------------------------------------------------------------
-// Space-time Simpson fluxes (Sec. 3.1, Sec. 6.1), scaled by dt/h.
-// ---------------------------------------------------------------------------
-template <typename T>
-__device__ __forceinline__ Prim<T> load_pt(T* const* pl, size_t q) {
-  Prim<T> w = {pl[0][q], pl[1][q], pl[2][q], pl[3][q]};
-  return w;
+template <typename T, bool FLUX>
+__global__ void __launch_bounds__(REF_THREADS) k_points(const __grid_constant__ StepArgs<T> a) {
+  pdl_wait();
+  int i, j;
+  size_t id;
+  if (!cell_of_thread(a, i, j, id)) return;
+  switch (blockIdx.y) {
+    case 0: point_node<0, FLUX>(a, i, j, id); break;
+    case 1: point_node<1, FLUX>(a, i, j, id); break;
+    default: point_node<2, FLUX>(a, i, j, id); break;
+  }
 }
 
+// ---------------------------------------------------------------------------
+// Time-integrated fluxes of the nodes (weights 1, 4, 1) and the average update.
+// ---------------------------------------------------------------------------
 template <typename T>
-__global__ void k_flux(StepArgs<T> a) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  int j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i >= a.nx || j >= a.ny) return;
-  size_t id = (size_t)j * a.nx + i;
-  size_t up = (size_t)wrapi(j + 1, a.ny) * a.nx + i;
-  size_t rt = (size_t)j * a.nx + wrapi(i + 1, a.nx);
-  T* const* lev[3][3] = {{a.in.pt[0], a.in.pt[1], a.in.pt[2]},
-                         {a.half[0], a.half[1], a.half[2]},
-                         {a.out.pt[0], a.out.pt[1], a.out.pt[2]}};
-  const T wt[3] = {T(1), T(4), T(1)};
-  T F[4] = {T(0), T(0), T(0), T(0)}, G[4] = {T(0), T(0), T(0), T(0)};
+struct NodeFlux {
+  T *vx[4], *vy[4], *ex[4], *ey[4];  // V (x, y), E_v (x), E_h (y), per component
+};
+
+// the planes k_points<T, true> stores them in
+template <typename T>
+inline NodeFlux<T> node_flux_of(const StepArgs<T>& a) {
+  NodeFlux<T> n;
+  for (int k = 0; k < 4; ++k) {
+    n.vx[k] = a.half[0][k];
+    n.vy[k] = a.half[1][k];
+    n.ex[k] = a.half[2][k];
+    n.ey[k] = a.fx[k];
+  }
+  return n;
+}
+
+// ... of states whose half-step points are in a.half (AF_FC)
+template <typename T>
+__global__ void __launch_bounds__(REF_THREADS)
+    k_node_flux(const __grid_constant__ StepArgs<T> a, const __grid_constant__ NodeFlux<T> n) {
+  pdl_wait();
+  int i, j;
+  size_t id;
+  if (!cell_of_thread(a, i, j, id)) return;
+  auto node = [&](T* const* pl) {
+    Prim<T> w = {pl[0][id], pl[1][id], pl[2][id], pl[3][id]};
+    return w;
+  };
+  T SV[2][4] = {}, SX[2][4] = {}, SY[2][4] = {};
+#pragma unroll
   for (int s = 0; s < 3; ++s) {
-    T fa[4], fm[4], fb[4];
-    // vertical edge x = x_i: V(i,j), E_v(i,j), V(i,j+1)
-    flux_x(load_pt<T>(lev[s][0], id), a.gas, fa);
-    flux_x(load_pt<T>(lev[s][1], id), a.gas, fm);
-    flux_x(load_pt<T>(lev[s][0], up), a.gas, fb);
-    for (int k = 0; k < 4; ++k) F[k] = fma(wt[s], fa[k] + T(4) * fm[k] + fb[k], F[k]);
-    // horizontal edge y = y_j: V(i,j), E_h(i,j), V(i+1,j)
-    flux_y(load_pt<T>(lev[s][0], id), a.gas, fa);
-    flux_y(load_pt<T>(lev[s][2], id), a.gas, fm);
-    flux_y(load_pt<T>(lev[s][0], rt), a.gas, fb);
-    for (int k = 0; k < 4; ++k) G[k] = fma(wt[s], fa[k] + T(4) * fm[k] + fb[k], G[k]);
+    T* const* const lev[3] = {s == 0 ? a.in.pt[0] : s == 1 ? a.half[0] : a.out.pt[0],
+                              s == 0 ? a.in.pt[1] : s == 1 ? a.half[1] : a.out.pt[1],
+                              s == 0 ? a.in.pt[2] : s == 1 ? a.half[2] : a.out.pt[2]};
+    const T wt = s == 1 ? T(4) : T(1);
+    add_flux<0>(node(lev[0]), a.gas, wt, SV);
+    add_flux<1>(node(lev[1]), a.gas, wt, SX);
+    add_flux<2>(node(lev[2]), a.gas, wt, SY);
   }
-  const T lam = a.dt / (T(36) * a.h);
+#pragma unroll
   for (int k = 0; k < 4; ++k) {
-    a.fx[k][id] = lam * F[k];
-    a.gy[k][id] = lam * G[k];
+    n.vx[k][id] = SV[0][k];
+    n.vy[k][id] = SV[1][k];
+    n.ex[k][id] = SX[0][k];
+    n.ey[k][id] = SY[1][k];
   }
 }
 
-// Conservative average update (Eq. af-average-update).  COMP: hi + lo pairs
-// updated by error-free sums of the four edge terms, so that each edge value
-// enters its two cells with opposite signs exactly.
+// Conservative average update (Eq. af-average-update): the edges' Simpson sums of
+// their nodes' fluxes, each formed the same way in the two cells it bounds.
+// COMP: hi + lo pairs updated by error-free sums of the four edge terms, so that
+// each edge value enters its two cells with opposite signs exactly.
 template <typename T, bool COMP>
-__global__ void k_average(StepArgs<T> a) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  int j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i >= a.nx || j >= a.ny) return;
-  size_t id = (size_t)j * a.nx + i;
-  size_t up = (size_t)wrapi(j + 1, a.ny) * a.nx + i;
-  size_t rt = (size_t)j * a.nx + wrapi(i + 1, a.nx);
+__global__ void __launch_bounds__(REF_THREADS)
+    k_average(const __grid_constant__ StepArgs<T> a, const __grid_constant__ NodeFlux<T> n) {
+  pdl_wait();
+  int i, j;
+  size_t id;
+  if (!cell_of_thread(a, i, j, id)) return;
+  const int ip = i + 1 == a.nx ? 0 : i + 1, jp = j + 1 == a.ny ? 0 : j + 1;
+  const size_t up = (size_t)jp * a.nx + i, rt = (size_t)j * a.nx + ip, ur = (size_t)jp * a.nx + ip;
+  const T lam = a.dth / T(36);
   unsigned bad = 0;
+#pragma unroll
   for (int k = 0; k < 4; ++k) {
+    const T *vx = n.vx[k], *vy = n.vy[k], *ex = n.ex[k], *ey = n.ey[k];
+    // edge sums at x_i, x_{i+1}, y_j, y_{j+1}
+    T fl = fma(T(4), ex[id], vx[id] + vx[up]), fr = fma(T(4), ex[rt], vx[rt] + vx[ur]);
+    T gb = fma(T(4), ey[id], vy[id] + vy[rt]), gt = fma(T(4), ey[up], vy[up] + vy[ur]);
     if constexpr (COMP) {
       float hi = a.in.avg[k][id], lo = a.in.lo[k][id];
-      comp_update(hi, lo, a.fx[k][id], a.fx[k][rt], a.gy[k][id], a.gy[k][up]);
+      comp_update(hi, lo, lam * fl, lam * fr, lam * gb, lam * gt);
       a.out.avg[k][id] = hi;
       a.out.lo[k][id] = lo;
-      if (!isfinite(hi)) bad |= FLAG_NONFINITE;
+      if (!is_finite(hi)) bad |= FLAG_NONFINITE;
     } else {
-      T v = a.in.avg[k][id] - (a.fx[k][rt] - a.fx[k][id]) - (a.gy[k][up] - a.gy[k][id]);
+      const T v = fma(-lam, (fr - fl) + (gt - gb), a.in.avg[k][id]);
       a.out.avg[k][id] = v;
-      if (!isfinite(v)) bad |= FLAG_NONFINITE;
+      if (!is_finite(v)) bad |= FLAG_NONFINITE;
     }
   }
   raise_flag(a.flags, bad);
