@@ -113,7 +113,7 @@ enum {
  *
  * The handle allocates two states and the step's scratch planes here (about
  * 84 planes of nx * ny values of the working precision); af_adjoint_step
- * allocates its own work area (92 planes) on its first call, host transfers
+ * allocates its own work area (56 planes) on its first call, host transfers
  * of pageable planes a staging buffer of 16 FP64 planes on their first use,
  * af_exchange_state another 16 FP64 planes and a second stream with host
  * planes; af_destroy frees all of them.  Kernel choices, read from the environment when the handle is created
@@ -205,9 +205,8 @@ af_status af_reduce_invariants(af_handle *h, double *out);
  * `where`, owned by the caller (they may not overlap).  Adjoints are with
  * respect to the stored variables (cell averages and primitive point values).
  * The step's forward intermediates are recomputed in the handle's precision:
- * in the FP32 modes on grids the pipelined fused kernel accepts, one launch
- * recomputes each tile's step and reverses its fluxes and point updates in
- * shared memory.  Synchronises the stream; returns the latched device error,
+ * in the FP32 modes one launch recomputes each tile's step and reverses its
+ * fluxes and point updates in shared memory.  Synchronises the stream; returns the latched device error,
  * if any. AF_FC handles are refused with AF_ERR_ARG (no adjoint of the
  * foot-centred update is provided). */
 af_status af_adjoint_step(af_handle *h, double dt, const af_state_f64 *lam_in,

@@ -6,7 +6,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libaf.so")
-SOURCES = ["af_api.cu", "af_tiles.cu", "af_noalloc.cu", "af_fc.cu"]
+SOURCES = ["af_api.cu", "af_tiles.cu", "af_adj_tiles.cu", "af_noalloc.cu", "af_fc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -1,19 +1,20 @@
 // af_adjoint.cuh -- hand-written discrete adjoint of one step (Sec. 6.1):
 // lambda^n = (d state^{n+1} / d state^n)^T lambda^{n+1}, linearised about the
-// state at t^n.  The forward intermediates are recomputed by the unfused step
-// kernels (af_ref_kernels.cuh); the reverse sweep then runs, one thread per
-// cell, through
-//   k_adj_flux      average update and space-time Simpson fluxes (gather)
-//   k_adj_points    transported / additive point update, Q2 evaluation at the
-//                   foot, the two Picard stages (all three point families)
+// state at t^n.  The forward intermediates are recomputed (the fused kernel's
+// tiles, or the kernels of af_ref_kernels.cuh); the reverse sweep then runs
+//   points      the space-time Simpson fluxes the point enters (a gather from the
+//               averages' lambda) and its transported / additive update: the Q2
+//               evaluation at the foot and the two Picard stages, both durations
+//               (k_adj_points, or tile_reverse in the fused sweeps)
 //   k_adj_acoustic  Horner in r, node freezing (c, Z, r) and the transposed
 //                   acoustic stencils (all four node families)
-//   k_adj_center    Simpson inversion
-// The scattering kernels add each contribution to global memory with one
-// vector reduction: the adjoints of the lattice nodes and of the increments
-// are kept as 4-wide records per node (FP32: one float4 atomic).  Adjoints are
-// with respect to the stored variables; the storage offsets of the FP32 modes
-// are constant shifts and do not change them.
+//   k_adj_center, k_adj_out  Simpson inversion, lambda^n out
+// The scatters add each contribution to global memory with one vector reduction:
+// the adjoints of the lattice nodes and of the increments are kept as 4-wide
+// records per node (FP32: one float4 atomic), which start at zero and are cleared
+// by the kernel that consumes them.  Adjoints are with respect to the stored
+// variables; the storage offsets of the FP32 modes are constant shifts and do not
+// change them.
 #pragma once
 
 #include "af_common.cuh"
@@ -30,25 +31,21 @@ struct AdjView {
   const T* sto;  // state^{n+1} of the recomputed step: same layout
   const T* scr;  // intermediates: centres 0-3, increments 4 + 12 s + 3 fam + k,
                  // half-step points 28 + 4 fam + k
-  T* lam;        // adjoints, in units of ps: lambda^{n+1} 0-15 and lambda^n of
-                 // the averages 16-19 (planes); node records of family fam at
-                 // 20 + 4 fam (4 values per cell: rho, u, v, p; family 3 is the
-                 // centre); increment records of (s, fam) at 36 + 4 (4 s + fam)
-                 // (du, dv, dp, 0); half- and full-step points 68 + 4 fam + k and
-                 // 80 + 4 fam + k (planes); the centre adjoint lambda_U of each
-                 // cell 92 + k (planes)
+  T* lam;        // adjoints, in units of ps: lambda^n of the averages 0-3 (planes);
+                 // node records of family fam at 4 + 4 fam (4 values per cell: rho,
+                 // u, v, p; family 3 is the centre); increment records of (s, fam)
+                 // at 20 + 4 (4 s + fam) (du, dv, dp, 0); the centre adjoint
+                 // lambda_U of each cell 52 + k (planes)
   size_t ps;
   int nx, ny;
-  T h, dt;
+  T h, dt, dth;  // dth = dt / h
   Gas<T> gas;
   int variant;
-  const double* lin64[16];  // lambda^{n+1} as given (FP64 device planes), read by
-                            // the fused reverse sweep in place of planes 0-15
+  const double* lin64[16];  // lambda^{n+1} as given (FP64 device planes)
 };
 
-constexpr int LAM_IN = 0, LAM_OUT = 16, LAM_NODE = 20, LAM_INC = 36, LAM_HALF = 68, LAM_FULL = 80;
-constexpr int LAM_LU = 92;
-constexpr int LAM_PLANES = 96;
+constexpr int LAM_OUT = 0, LAM_NODE = 4, LAM_INC = 20, LAM_LU = 52;
+constexpr int LAM_PLANES = 56;
 constexpr int SCR_INC = 4, SCR_HALF = 28;
 
 // cell index wrapped into [0, n): one conditional step for |i| < 2n
@@ -70,19 +67,6 @@ __device__ __forceinline__ Prim<T> node_w(const AdjView<T>& v, int fam, size_t i
   return w;
 }
 
-// increments (u + du, v + dv, dp) of duration s at the node of family fam of cell id
-template <typename T>
-__device__ __forceinline__ void node_d(const AdjView<T>& v, int s, int fam, size_t id, T d[3]) {
-  const T* b = v.scr + (size_t)(SCR_INC + 12 * s + 3 * fam) * v.ps + id;
-  d[0] = b[0];
-  d[1] = b[v.ps];
-  d[2] = b[2 * v.ps];
-}
-
-// Shared-memory accumulator over the footprint of a BX x BY block: cells
-// [i0-1, i0+BX+2) x [j0-1, j0+BY+2), NPL planes; local plane lp < 16 is the
-// adjoint of lattice plane 4 fam + k (global LAM_NODE + lp), lp >= 16 the
-// adjoint of increment 12 s + 3 fam + k (global LAM_INC + lp - 16).
 // adds (a, b, c, d) to the 4-wide record at p (16-byte aligned), without
 // looking for zeros
 __device__ __forceinline__ void add4_always(float* p, float a, float b, float c, float d) {
@@ -93,6 +77,16 @@ __device__ __forceinline__ void add4_always(double* p, double a, double b, doubl
   atomicAdd(p + 1, b);
   atomicAdd(p + 2, c);
   atomicAdd(p + 3, d);
+}
+
+// the same for the three values of an increment record
+__device__ __forceinline__ void add3_always(float* p, float a, float b, float c) {
+  atomicAdd(reinterpret_cast<float4*>(p), make_float4(a, b, c, 0.f));
+}
+__device__ __forceinline__ void add3_always(double* p, double a, double b, double c) {
+  atomicAdd(p, a);
+  atomicAdd(p + 1, b);
+  atomicAdd(p + 2, c);
 }
 
 // clears the 4-wide record at p once its consumer has read it, so that the
@@ -117,55 +111,29 @@ __device__ __forceinline__ void add4(double* p, double a, double b, double c, do
   if (d != 0.0) atomicAdd(p + 3, d);
 }
 
-// Accumulator of node and increment adjoints (records of the adjoint arena).
-template <typename T>
-struct VecAdj {
-  T* lam;
-  size_t ps;
-  int nx, ny;
-  __device__ __forceinline__ size_t cell(int cx, int cy) const {
-    return (size_t)wrapc(cy, ny) * nx + wrapc(cx, nx);
-  }
-  // adjoint of the node of family fam of (unwrapped) cell (cx, cy)
-  __device__ __forceinline__ void node(int fam, int cx, int cy, T r, T u, T w, T p) const {
-    add4(lam + (size_t)(LAM_NODE + 4 * fam) * ps + 4 * cell(cx, cy), r, u, w, p);
-  }
-  __device__ __forceinline__ void inc(int s, int fam, int cx, int cy, T du, T dv, T dp) const {
-    add4(lam + (size_t)(LAM_INC + 4 * (4 * s + fam)) * ps + 4 * cell(cx, cy), du, dv, dp, T(0));
-  }
-};
-
-template <typename T>
-__device__ __forceinline__ VecAdj<T> vec_adj(const AdjView<T>& v) {
-  VecAdj<T> a = {v.lam, v.ps, v.nx, v.ny};
-  return a;
-}
-
-// Transposed Euler flux Jacobians: out += J_F(w)^T l  (stored primitives)
+// Transposed Euler flux Jacobians: o += J_F(w)^T l  (stored primitives)
 template <typename T>
 __device__ __forceinline__ void flux_x_adj(const Prim<T>& w, const Gas<T>& g, const T l[4],
-                                           T s, T o[4]) {
-  const T rho = g.rho_ref + w.r, p = g.p_ref + w.p;
-  const T q2 = w.u * w.u + w.v * w.v;
-  const T hh = p * g.g_gm1 + T(0.5) * rho * q2;
-  o[0] += s * (w.u * l[0] + w.u * w.u * l[1] + w.u * w.v * l[2] + T(0.5) * w.u * q2 * l[3]);
-  o[1] += s * (rho * l[0] + T(2) * rho * w.u * l[1] + rho * w.v * l[2] +
-               (hh + rho * w.u * w.u) * l[3]);
-  o[2] += s * (rho * w.u * l[2] + rho * w.u * w.v * l[3]);
-  o[3] += s * (l[1] + g.g_gm1 * w.u * l[3]);
+                                           T o[4]) {
+  const T rho = with_ref(g.rho_ref, w.r), p = with_ref(g.p_ref, w.p);
+  const T ke = T(0.5) * fma(w.u, w.u, w.v * w.v), hh = fma(p, g.g_gm1, rho * ke);
+  const T t = fma(w.v, l[2], fma(w.u, l[1], l[0]));
+  o[0] = fma(w.u, fma(ke, l[3], t), o[0]);
+  o[1] = fma(rho, fma(w.u, fma(w.u, l[3], l[1]), t), fma(hh, l[3], o[1]));
+  o[2] = fma(rho * w.u, fma(w.v, l[3], l[2]), o[2]);
+  o[3] = fma(g.g_gm1 * w.u, l[3], o[3] + l[1]);
 }
 
 template <typename T>
 __device__ __forceinline__ void flux_y_adj(const Prim<T>& w, const Gas<T>& g, const T l[4],
-                                           T s, T o[4]) {
-  const T rho = g.rho_ref + w.r, p = g.p_ref + w.p;
-  const T q2 = w.u * w.u + w.v * w.v;
-  const T hh = p * g.g_gm1 + T(0.5) * rho * q2;
-  o[0] += s * (w.v * l[0] + w.u * w.v * l[1] + w.v * w.v * l[2] + T(0.5) * w.v * q2 * l[3]);
-  o[1] += s * (rho * w.v * l[1] + rho * w.u * w.v * l[3]);
-  o[2] += s * (rho * l[0] + rho * w.u * l[1] + T(2) * rho * w.v * l[2] +
-               (hh + rho * w.v * w.v) * l[3]);
-  o[3] += s * (l[2] + g.g_gm1 * w.v * l[3]);
+                                           T o[4]) {
+  const T rho = with_ref(g.rho_ref, w.r), p = with_ref(g.p_ref, w.p);
+  const T ke = T(0.5) * fma(w.u, w.u, w.v * w.v), hh = fma(p, g.g_gm1, rho * ke);
+  const T t = fma(w.v, l[2], fma(w.u, l[1], l[0]));
+  o[0] = fma(w.v, fma(ke, l[3], t), o[0]);
+  o[1] = fma(rho * w.v, fma(w.u, l[3], l[1]), o[1]);
+  o[2] = fma(rho, fma(w.v, fma(w.v, l[3], l[2]), t), fma(hh, l[3], o[2]));
+  o[3] = fma(g.g_gm1 * w.v, l[3], o[3] + l[2]);
 }
 
 // derivative of the Lagrange basis l_-, l_0, l_+ with respect to s
@@ -180,11 +148,11 @@ template <typename T>
 __device__ __forceinline__ void dcons_dprim_T(const Prim<T>& w, const Gas<T>& g, const T l[4],
                                               T s, T o[4]) {
   // o += s (dU/dW)^T l, U = (rho~, rho u, rho v, E~) of the stored primitive
-  const T rho = g.rho_ref + w.r;
-  o[0] += s * (l[0] + w.u * l[1] + w.v * l[2] + T(0.5) * (w.u * w.u + w.v * w.v) * l[3]);
-  o[1] += s * (rho * l[1] + rho * w.u * l[3]);
-  o[2] += s * (rho * l[2] + rho * w.v * l[3]);
-  o[3] += s * (g.gm1inv * l[3]);
+  const T rho = s * with_ref(g.rho_ref, w.r), ke = T(0.5) * fma(w.u, w.u, w.v * w.v);
+  o[0] = fma(s, fma(ke, l[3], fma(w.v, l[2], fma(w.u, l[1], l[0]))), o[0]);
+  o[1] = fma(rho, fma(w.u, l[3], l[1]), o[1]);
+  o[2] = fma(rho, fma(w.v, l[3], l[2]), o[2]);
+  o[3] = fma(s * g.gm1inv, l[3], o[3]);
 }
 
 template <int FAM, typename T, typename Scatter>
@@ -198,11 +166,9 @@ __device__ __forceinline__ void sac_family_adj(const Scatter& S, const T lGp[3][
 
 
 // ---------------------------------------------------------------------------
-// Average update and fluxes (Eq. af-average-update), gathered per cell: the
-// adjoints of the three point families of cell (i,j) at sigma = 0, 1/2, 1.
-// Writes lambda^n of the averages and the sigma = 0 part of lambda^n of the
-// points (the later kernels add to them), and the adjoints of the half- and
-// full-step points.
+// Points, reversed: the average update and the space-time Simpson fluxes (Eq.
+// af-average-update) as a gather, then the point update (Sec. 6.1 steps 3-4;
+// Eq. barsukow-additive).  One thread per point, families by blockIdx.y.
 // ---------------------------------------------------------------------------
 template <typename T>
 __device__ __forceinline__ Prim<T> level_pt(const T* base, size_t ps, int f, size_t id) {
@@ -211,245 +177,245 @@ __device__ __forceinline__ Prim<T> level_pt(const T* base, size_t ps, int f, siz
   return w;
 }
 
+// lambda^{n+1} as given, in the working precision
 template <typename T>
-__global__ void k_adj_flux(const __grid_constant__ AdjView<T> v) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  const int nx = v.nx, ny = v.ny;
-  if (i >= nx || j >= ny) return;
-  const size_t ps = v.ps;
-  const int im = wrapc(i - 1, nx), jm = wrapc(j - 1, ny);
-  const size_t id = (size_t)j * nx + i, idl = (size_t)j * nx + im, idb = (size_t)jm * nx + i,
-               idlb = (size_t)jm * nx + im;
-  T lfx[4], lfxb[4], lgy[4], lgyl[4];
+__device__ __forceinline__ T lam_in(const AdjView<T>& v, int plane, size_t id) {
+  return (T)v.lin64[plane][id];
+}
+
+// Adjoints of the x- and y-fluxes (lex, ley, before the factor dt / (36 h)) that
+// the point of family FAM of cell (i, j) enters, and lambda of the point itself;
+// also passes lambda of the averages through (family 0, one writer per cell).
+// Every load is issued before the first use.
+template <int FAM, typename T>
+__device__ __forceinline__ void flux_lambda(const AdjView<T>& v, int i, int j, size_t id, T lex[4],
+                                            T ley[4], T lpt[4]) {
+  const int im = i == 0 ? v.nx - 1 : i - 1, jm = j == 0 ? v.ny - 1 : j - 1;
+  const size_t idl = (size_t)j * v.nx + im, idb = (size_t)jm * v.nx + i,
+               idlb = (size_t)jm * v.nx + im;
+  T c[4], l[4], b[4], lb[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const T* lk = v.lam + (size_t)(LAM_IN + k) * ps;
-    const T c = lk[id], l = lk[idl], b = lk[idb], lb = lk[idlb];
-    lfx[k] = c - l;    // vertical edge x_i of cell (i,j)
-    lfxb[k] = b - lb;  // vertical edge x_i of cell (i,j-1)
-    lgy[k] = c - b;    // horizontal edge y_j of cell (i,j)
-    lgyl[k] = l - lb;  // horizontal edge y_j of cell (i-1,j)
-    v.lam[(size_t)(LAM_OUT + k) * ps + id] = c;
+    c[k] = lam_in(v, k, id);
+    if (FAM != 2) l[k] = lam_in(v, k, idl);
+    if (FAM != 1) b[k] = lam_in(v, k, idb);
+    if (FAM == 0) lb[k] = lam_in(v, k, idlb);
+    lpt[k] = lam_in(v, 4 + 4 * FAM + k, id);
   }
-  const T cst = v.dt / (T(36) * v.h);
-  T lvx[4], lvy[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    lvx[k] = lfx[k] + lfxb[k];
-    lvy[k] = lgy[k] + lgyl[k];
-  }
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    // point values at sigma = 0 (state^n), 1/2 (recomputed), 1 (state^{n+1})
-    const T* base = s == 0 ? v.st + 4 * ps : s == 1 ? v.scr + (size_t)SCR_HALF * ps : v.sto + 4 * ps;
-    const T sc = cst * (s == 1 ? T(4) : T(1));
-    T oV[4] = {T(0), T(0), T(0), T(0)}, oEv[4] = {T(0), T(0), T(0), T(0)},
-      oEh[4] = {T(0), T(0), T(0), T(0)};
-    const Prim<T> wV = level_pt(base, ps, 0, id);
-    flux_x_adj(wV, v.gas, lvx, sc, oV);
-    flux_y_adj(wV, v.gas, lvy, sc, oV);
-    flux_x_adj(level_pt(base, ps, 1, id), v.gas, lfx, T(4) * sc, oEv);
-    flux_y_adj(level_pt(base, ps, 2, id), v.gas, lgy, T(4) * sc, oEh);
-    const T* oo[3] = {oV, oEv, oEh};
-    if (s == 0) {
-      // lambda^n of the points starts as their node records (the later kernels add)
-#pragma unroll
-      for (int f = 0; f < 3; ++f) {
-        T* rec = v.lam + (size_t)(LAM_NODE + 4 * f) * ps + 4 * id;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) rec[k] = oo[f][k];
-      }
+    if (FAM == 0) {
+      lex[k] = (c[k] - l[k]) + (b[k] - lb[k]);
+      ley[k] = (c[k] - b[k]) + (l[k] - lb[k]);
+      v.lam[(size_t)(LAM_OUT + k) * v.ps + id] = c[k];
+    } else if (FAM == 1) {
+      lex[k] = c[k] - l[k];
     } else {
-      const int dst = s == 1 ? LAM_HALF : LAM_FULL;
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-#pragma unroll
-        for (int f = 0; f < 3; ++f) {
-          T val = oo[f][k];
-          if (s == 2) val += v.lam[(size_t)(LAM_IN + 4 + 4 * f + k) * ps + id];
-          v.lam[(size_t)(dst + 4 * f + k) * ps + id] = val;
-        }
+      ley[k] = c[k] - b[k];
     }
   }
 }
 
-// ---------------------------------------------------------------------------
-// Point update (Sec. 6.1 steps 3-4; Eq. barsukow-additive), reversed.
-// ---------------------------------------------------------------------------
-// the nine nodes of foot cell c in [b][q] order (loaded once: the scatter
-// below reuses them between its atomics)
-template <typename T>
-__device__ __forceinline__ void load_nodes(const AdjView<T>& v, const FootCell<T>& c, Prim<T> w[9]) {
+// o = the share of the fluxes' adjoints that reaches the node value w; lex, ley
+// carry the factor dt / (36 h), sc the time and edge-midpoint weights
+template <int FAM, typename T>
+__device__ __forceinline__ void flux_share(const Prim<T>& w, const Gas<T>& g, const T lex[4],
+                                           const T ley[4], T sc, T o[4]) {
+  T l[4];
 #pragma unroll
-  for (int b = 0; b < 3; ++b)
+  for (int k = 0; k < 4; ++k) o[k] = T(0);
+  if (FAM != 2) {
 #pragma unroll
-    for (int q = 0; q < 3; ++q)
-      w[3 * b + q] = node_w(v, fam_of(q, b), cell_id(v, c.ci + (q >> 1), c.cj + (b >> 1)));
+    for (int k = 0; k < 4; ++k) l[k] = sc * lex[k];
+    flux_x_adj(w, g, l, o);
+  }
+  if (FAM != 1) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) l[k] = sc * ley[k];
+    flux_y_adj(w, g, l, o);
+  }
 }
 
-template <typename T>
-__device__ __forceinline__ void load_incs(const AdjView<T>& v, int s, const FootCell<T>& c,
-                                          T d[9][3]) {
+// Fluxes of the point of family FAM of cell (i, j), reversed: its adjoints at
+// sigma = 0 (own node, value wp), 1/2 and 1 (values wh, wf; lambda^{n+1} of the
+// point included in the last).
+template <int FAM, typename T>
+__device__ __forceinline__ void point_fluxes_adj(const AdjView<T>& v, int i, int j, size_t id,
+                                                 const Prim<T>& wp, const Prim<T>& wh,
+                                                 const Prim<T>& wf, T own[4], T lyh[4], T lyf[4]) {
+  T lex[4], ley[4], lpt[4];
+  flux_lambda<FAM>(v, i, j, id, lex, ley, lpt);
+  const T cst = v.dth / T(36), mid = FAM == 0 ? cst : T(4) * cst;
+  flux_share<FAM>(wp, v.gas, lex, ley, mid, own);
+  flux_share<FAM>(wh, v.gas, lex, ley, T(4) * mid, lyh);
+  flux_share<FAM>(wf, v.gas, lex, ley, mid, lyf);
 #pragma unroll
-  for (int b = 0; b < 3; ++b)
-#pragma unroll
-    for (int q = 0; q < 3; ++q)
-      node_d(v, s, fam_of(q, b), cell_id(v, c.ci + (q >> 1), c.cj + (b >> 1)), d[3 * b + q]);
+  for (int k = 0; k < 4; ++k) lyf[k] += lpt[k];
 }
 
-// sum_qb l_q(xi) l_b(eta) f_qb (rows first, as the forward evaluation)
+// sum over the nine nodes of d/d(xi) and d/d(eta) of the Q2 basis times dot[]
 template <typename T>
-__device__ __forceinline__ T q2_sum(const T* f, int stride, const T lx[3], const T ly[3]) {
-  T out = T(0);
+__device__ __forceinline__ void grad_sum(const T dot[9], const T lx[3], const T ly[3],
+                                         const T dx[3], const T dy[3], T& gx, T& gy) {
+  T rx[3], rl[3];
 #pragma unroll
   for (int b = 0; b < 3; ++b) {
-    T row = T(0);
-#pragma unroll
-    for (int q = 0; q < 3; ++q) row = fma(lx[q], f[(3 * b + q) * stride], row);
-    out = fma(ly[b], row, out);
+    rx[b] = fma(dx[0], dot[3 * b], fma(dx[1], dot[3 * b + 1], dx[2] * dot[3 * b + 2]));
+    rl[b] = fma(lx[0], dot[3 * b], fma(lx[1], dot[3 * b + 1], lx[2] * dot[3 * b + 2]));
   }
-  return out;
+  gx = fma(ly[0], rx[0], fma(ly[1], rx[1], ly[2] * rx[2]));
+  gy = fma(dy[0], rl[0], fma(dy[1], rl[1], dy[2] * rl[2]));
 }
 
 // the point of family FAM of cell (i, j), both durations
-template <int FAM, typename T, typename Acc>
-__device__ __forceinline__ void point_adj(const AdjView<T>& v, const Acc& acc, int i, int j) {
-  const size_t ps = v.ps, id = (size_t)j * v.nx + i;
-  const int I = 2 * i + (FAM == 2 ? 1 : 0);
-  const int J = 2 * j + (FAM == 1 ? 1 : 0);
-  const Prim<T> wp = node_w(v, FAM, id);
-  const T hinv = T(1) / v.h;
+template <int FAM, typename T>
+__device__ __forceinline__ void point_adj(const AdjView<T>& v, int i, int j, size_t id) {
+  const size_t ps = v.ps;
+  const int nx = v.nx, ny = v.ny;
+  constexpr int OX = FAM == 2 ? 1 : 0, OY = FAM == 1 ? 1 : 0;
   const Gas<T>& g = v.gas;
-  T luP = T(0), lvP = T(0), lrP = T(0), lpP = T(0);
+  const Prim<T> wp = level_pt(v.st + 4 * ps, ps, FAM, id);
+  auto wplane = [&](int k) {  // time-n values: component k of family f
+    return [&v, k](int f) {
+      return f < 3 ? v.st + (size_t)(4 + 4 * f + k) * v.ps : v.scr + (size_t)k * v.ps;
+    };
+  };
+  auto node_rec = [&](int f, size_t q) {
+    return v.lam + (size_t)(LAM_NODE + 4 * f) * ps + 4 * q;
+  };
+  T own[4], lyh[4], lyf[4];
+  point_fluxes_adj<FAM>(v, i, j, id, wp,
+                        level_pt(v.scr + (size_t)SCR_HALF * ps, ps, FAM, id),
+                        level_pt(v.sto + 4 * ps, ps, FAM, id), own, lyh, lyf);
 #pragma unroll 1
   for (int s = 0; s < 2; ++s) {
-    const T th = (s == 0 ? T(0.5) * v.dt : v.dt) * hinv;
-    const T* lsrc = v.lam + (size_t)((s == 0 ? LAM_HALF : LAM_FULL) + 4 * FAM) * ps + id;
-    const T ly[4] = {lsrc[0], lsrc[ps], lsrc[2 * ps], lsrc[3 * ps]};
-    if (ly[0] == T(0) && ly[1] == T(0) && ly[2] == T(0) && ly[3] == T(0)) continue;
+    const T th = s == 0 ? T(0.5) * v.dth : v.dth;
+    T ly[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) ly[k] = s == 0 ? lyh[k] : lyf[k];
+    auto iplane = [&](int k) {
+      return [&v, s, k](int f) { return v.scr + (size_t)(SCR_INC + 12 * s + 3 * f + k) * v.ps; };
+    };
     // forward recomputation of the foot (Eq. adv-footpoint)
-    const T d1x = -th * wp.u, d1y = -th * wp.v;
-    const FootCell<T> c1 = locate<T>(I, J, d1x, d1y);
-    T uv1[9][2];  // (u, v) of the first stage's nodes
-#pragma unroll
-    for (int b = 0; b < 3; ++b)
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        const Prim<T> w = node_w(v, fam_of(q, b), cell_id(v, c1.ci + (q >> 1), c1.cj + (b >> 1)));
-        uv1[3 * b + q][0] = w.u;
-        uv1[3 * b + q][1] = w.v;
-      }
-    T lx1[3], ly1[3];
-    lagrange3(c1.xi, lx1);
-    lagrange3(c1.eta, ly1);
-    const T u1 = q2_sum(&uv1[0][0], 2, lx1, ly1), v1 = q2_sum(&uv1[0][1], 2, lx1, ly1);
-    const T dfx = -th * u1, dfy = -th * v1;
-    const FootCell<T> fc = locate<T>(I, J, dfx, dfy);
-    Prim<T> nf[9];
-    load_nodes(v, fc, nf);
-    T lx[3], lyb[3], dx3[3], dy3[3];
-    lagrange3(fc.xi, lx);
-    lagrange3(fc.eta, lyb);
-    lagrange3_d(fc.xi, dx3);
-    lagrange3_d(fc.eta, dy3);
-    Prim<T> wf;
-    wf.r = q2_sum(&nf[0].r, 4, lx, lyb);
-    wf.p = q2_sum(&nf[0].p, 4, lx, lyb);
-    T lwf[4], ld[3];  // adjoints of W_f and of the interpolated increments
-    T df[9][3];
-    if (v.variant == 0) {
-      load_incs(v, s, fc, df);
-      const T d2 = q2_sum(&df[0][2], 3, lx, lyb);
-      const T rf = g.rho_ref + wf.r, pf = g.p_ref + wf.p;
-      const T gp = g.gamma * pf;
-      lwf[0] = ly[0] * (T(1) + d2 / gp);
-      lwf[1] = ly[1];
-      lwf[2] = ly[2];
-      lwf[3] = ly[3] - ly[0] * d2 * rf / (gp * pf);
-      ld[0] = ly[1];
-      ld[1] = ly[2];
-      ld[2] = ly[3] + ly[0] * rf / gp;
-    } else {
-      T d[3];
-      node_d(v, s, FAM, id, d);
-      const T rp = g.rho_ref + wp.r, pp = g.p_ref + wp.p;
-      const T gp = g.gamma * pp;
-      lwf[0] = ly[0];
-      lwf[1] = ly[1];
-      lwf[2] = ly[2];
-      lwf[3] = ly[3];
-      // nw.r = wf.r + dp rho_P / (gamma p_P), with the increments at P itself
-      acc.inc(s, FAM, i, j, ly[1], ly[2], ly[3] + ly[0] * rp / gp);
-      lrP += ly[0] * d[2] / gp;
-      lpP += -ly[0] * d[2] * rp / (gp * pp);
-      ld[0] = ld[1] = ld[2] = T(0);
+    int c1x, c1y, cfx, cfy;
+    T lx1[3], ly1[3], lx[3], lyb[3], dx1[3], dy1[3], dx3[3], dy3[3];
+    {
+      const T sx = foot_coord<OX>(-th * wp.u, c1x), sy = foot_coord<OY>(-th * wp.v, c1y);
+      lagrange3_fma(sx, lx1);
+      lagrange3_fma(sy, ly1);
+      lagrange3_d(sx, dx1);
+      lagrange3_d(sy, dy1);
     }
-    // adjoint of the foot's local coordinates through the Q2 evaluation there
-    T lxi = T(0), leta = T(0);
+    const FootNodes n1 = foot_nodes(i + c1x, j + c1y, nx, ny);
+    {
+      const T u1 = row_sum(n1, lx1, ly1, wplane(1)), v1 = row_sum(n1, lx1, ly1, wplane(2));
+      const T sx = foot_coord<OX>(-th * u1, cfx), sy = foot_coord<OY>(-th * v1, cfy);
+      lagrange3_fma(sx, lx);
+      lagrange3_fma(sy, lyb);
+      lagrange3_d(sx, dx3);
+      lagrange3_d(sy, dy3);
+    }
+    const FootNodes nf = foot_nodes(i + cfx, j + cfy, nx, ny);
+    T w[9];
 #pragma unroll
-    for (int b = 0; b < 3; ++b)
+    for (int m = 0; m < 9; ++m) w[m] = lx[m % 3] * lyb[m / 3];
+    const T rft = nine_sum(nf, w, wplane(0)), pft = nine_sum(nf, w, wplane(3));
+    T lwf[4], ldp = T(0);  // adjoints of W_f and of the interpolated dp (du, dv: lwf[1], lwf[2])
+    if (v.variant == 0) {
+      const T d2 = nine_sum(nf, w, iplane(2));
+      const T rf = with_ref(g.rho_ref, rft), pf = with_ref(g.p_ref, pft);
+      const T igp = T(1) / (g.gamma * pf);
+      const T a0 = ly[0] * igp;
+      lwf[0] = fma(a0, d2, ly[0]);
+      lwf[1] = ly[1];
+      lwf[2] = ly[2];
+      lwf[3] = fma(-(a0 * d2) * rf, igp * g.gamma, ly[3]);
+      ldp = fma(a0, rf, ly[3]);
+    } else {
+      const T d2 = iplane(2)(FAM)[id];
+      const T rp = with_ref(g.rho_ref, wp.r), pp = with_ref(g.p_ref, wp.p);
+      const T igp = T(1) / (g.gamma * pp);
+      const T a0 = ly[0] * igp;
 #pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        const int n = 3 * b + q;
-        // (u and du enter the transported update with the same weight, and the
-        // increment planes hold u + du, v + dv)
-        T dot = v.variant == 0
-                    ? nf[n].r * lwf[0] + df[n][0] * lwf[1] + df[n][1] * lwf[2] +
-                          nf[n].p * lwf[3] + df[n][2] * ld[2]
-                    : nf[n].r * lwf[0] + nf[n].u * lwf[1] + nf[n].v * lwf[2] + nf[n].p * lwf[3];
-        lxi += dx3[q] * lyb[b] * dot;
-        leta += lx[q] * dy3[b] * dot;
+      for (int k = 0; k < 4; ++k) lwf[k] = ly[k];
+      // nw.r = wf.r + dp rho_P / (gamma p_P), with the increments at P itself
+      add4(v.lam + (size_t)(LAM_INC + 4 * (4 * s + FAM)) * ps + 4 * id, ly[1], ly[2],
+           fma(a0, rp, ly[3]), T(0));
+      own[0] = fma(a0, d2, own[0]);
+      own[3] = fma(-(a0 * d2) * rp, igp * g.gamma, own[3]);
+    }
+    // adjoint of the foot's local coordinates through the Q2 evaluation there (u
+    // and du enter the transported update with the same weight; the increment
+    // planes hold their sum)
+    T dot[9], gx, gy;
+#pragma unroll
+    for (int m = 0; m < 9; ++m) {
+      const int f = fam_of(m % 3, m / 3);
+      const size_t q = nf.n[m / 3 >> 1][m % 3 >> 1];
+      T t = fma(wplane(0)(f)[q], lwf[0], wplane(3)(f)[q] * lwf[3]);
+      if (v.variant == 0) {
+        t = fma(iplane(0)(f)[q], lwf[1], t);
+        t = fma(iplane(1)(f)[q], lwf[2], t);
+        dot[m] = fma(iplane(2)(f)[q], ldp, t);
+      } else {
+        t = fma(wplane(1)(f)[q], lwf[1], t);
+        dot[m] = fma(wplane(2)(f)[q], lwf[2], t);
       }
+    }
+    grad_sum(dot, lx, lyb, dx3, dy3, gx, gy);
     // xi = 2 (foot - cell) - 1; the foot moved by df = -th (u1, v1)
-    const T lu1 = -th * (T(2) * lxi), lv1 = -th * (T(2) * leta);
+    const T lu1 = T(-2) * th * gx, lv1 = T(-2) * th * gy;
     // first Picard stage: (u1, v1) = R_h(u, v) at P + d1
-    T dx31[3], dy31[3];
-    lagrange3_d(c1.xi, dx31);
-    lagrange3_d(c1.eta, dy31);
-    T lxi1 = T(0), leta1 = T(0);
 #pragma unroll
-    for (int b = 0; b < 3; ++b)
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        const int n = 3 * b + q;
-        const T dot = uv1[n][0] * lu1 + uv1[n][1] * lv1;
-        lxi1 += dx31[q] * ly1[b] * dot;
-        leta1 += lx1[q] * dy31[b] * dot;
-      }
-    luP += -th * (T(2) * lxi1);
-    lvP += -th * (T(2) * leta1);
+    for (int m = 0; m < 9; ++m) {
+      const int f = fam_of(m % 3, m / 3);
+      const size_t q = n1.n[m / 3 >> 1][m % 3 >> 1];
+      dot[m] = fma(wplane(1)(f)[q], lu1, wplane(2)(f)[q] * lv1);
+    }
+    grad_sum(dot, lx1, ly1, dx1, dy1, gx, gy);
+    own[1] = fma(T(-2) * th, gx, own[1]);
+    own[2] = fma(T(-2) * th, gy, own[2]);
     // scatter to the nodes of the foot cell and of the first stage's cell (one
     // record update per node when the two cells coincide, the usual case)
-    const bool same = c1.ci == fc.ci && c1.cj == fc.cj;
+    const bool same = c1x == cfx && c1y == cfy;
 #pragma unroll
-    for (int b = 0; b < 3; ++b)
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        const int fam = fam_of(q, b), cx = fc.ci + (q >> 1), cy = fc.cj + (b >> 1);
-        const T wgt = lx[q] * lyb[b], w1 = same ? lx1[q] * ly1[b] : T(0);
-        acc.node(fam, cx, cy, wgt * lwf[0], wgt * lwf[1] + w1 * lu1, wgt * lwf[2] + w1 * lv1,
-                 wgt * lwf[3]);
-        if (v.variant == 0) acc.inc(s, fam, cx, cy, wgt * ld[0], wgt * ld[1], wgt * ld[2]);
+    for (int m = 0; m < 9; ++m) {
+      const int f = fam_of(m % 3, m / 3);
+      const size_t q = nf.n[m / 3 >> 1][m % 3 >> 1];
+      const T wu = w[m] * lwf[1], wv = w[m] * lwf[2];
+      T nu = wu, nv = wv;
+      if (same) {
+        const T w1 = lx1[m % 3] * ly1[m / 3];
+        nu = fma(w1, lu1, wu);
+        nv = fma(w1, lv1, wv);
       }
+      add4_always(node_rec(f, q), w[m] * lwf[0], nu, nv, w[m] * lwf[3]);
+      if (v.variant == 0)
+        add3_always(v.lam + (size_t)(LAM_INC + 4 * (4 * s + f)) * ps + 4 * q, wu, wv, w[m] * ldp);
+    }
     if (!same) {
 #pragma unroll
-      for (int b = 0; b < 3; ++b)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-          const T w1 = lx1[q] * ly1[b];
-          acc.node(fam_of(q, b), c1.ci + (q >> 1), c1.cj + (b >> 1), T(0), w1 * lu1, w1 * lv1,
-                   T(0));
-        }
+      for (int m = 0; m < 9; ++m) {
+        const T w1 = lx1[m % 3] * ly1[m / 3];
+        add4(node_rec(fam_of(m % 3, m / 3), n1.n[m / 3 >> 1][m % 3 >> 1]), T(0), w1 * lu1,
+             w1 * lv1, T(0));
+      }
     }
   }
-  acc.node(FAM, i, j, lrP, luP, lvP, lpP);
+  add4_always(node_rec(FAM, id), own[0], own[1], own[2], own[3]);
 }
 
-template <int FAM, typename T>
-__global__ void __launch_bounds__(256, 2) k_adj_points(const __grid_constant__ AdjView<T> v) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i < v.nx && j < v.ny) point_adj<FAM>(v, vec_adj(v), i, j);
+template <typename T>
+__global__ void __launch_bounds__(REF_THREADS) k_adj_points(const __grid_constant__ AdjView<T> v) {
+  pdl_wait();
+  const size_t id = (size_t)blockIdx.x * REF_THREADS + threadIdx.x;
+  if (id >= (size_t)v.nx * v.ny) return;
+  const int j = (int)(id / (unsigned)v.nx), i = (int)(id - (size_t)j * v.nx);
+  switch (blockIdx.y) {
+    case 0: point_adj<0>(v, i, j, id); break;
+    case 1: point_adj<1>(v, i, j, id); break;
+    default: point_adj<2>(v, i, j, id); break;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -540,9 +506,8 @@ struct ScatterAdj {
 
 // `row`: the lanes of the calling warp (one row of 32 consecutive nodes) inside
 // the grid
-template <int FAM, typename T, typename Acc>
-__device__ __forceinline__ void acoustic_adj(const AdjView<T>& v, const Acc& acc, int i, int j,
-                                             unsigned row) {
+template <int FAM, typename T>
+__device__ __forceinline__ void acoustic_adj(const AdjView<T>& v, int i, int j, unsigned row) {
   const size_t ps = v.ps, id = (size_t)j * v.nx + i;
   T ld[2][3];
   bool any = false;
@@ -561,10 +526,11 @@ __device__ __forceinline__ void acoustic_adj(const AdjView<T>& v, const Acc& acc
 #pragma unroll
   for (int s = 0; s < 2; ++s) zero4(v.lam + (size_t)(LAM_INC + 4 * (4 * s + FAM)) * ps + 4 * id);
   const Prim<T> wk = node_w(v, FAM, id);
-  const T rk = v.gas.rho_ref + wk.r, pk = v.gas.p_ref + wk.p;
-  const T c = sqrt(v.gas.gamma * pk / rk);
-  const T Z = rk * c, Zinv = T(1) / Z;
-  const T dth = v.dt / v.h;
+  const T rk = with_ref(v.gas.rho_ref, wk.r), pk = with_ref(v.gas.p_ref, wk.p);
+  // Z^2 = gamma p rho, c = gamma p / Z
+  const T gp = v.gas.gamma * pk, z2 = gp * rk;
+  const T Zinv = rsqrt_t(z2), Z = z2 * Zinv, c = gp * Zinv;
+  const T dth = v.dth;
   const T r1 = c * dth;
   T Gp[3][4], Guv[3][4];
   const Nbhd nb = nbhd(i, j, v.nx, v.ny);
@@ -578,24 +544,29 @@ __device__ __forceinline__ void acoustic_adj(const AdjView<T>& v, const Acc& acc
     co[0][q] = fma(Zinv, Gp[1][q], Guv[1][q]);  // du
     co[1][q] = fma(Zinv, Gp[2][q], Guv[2][q]);  // dv
   }
-  T lco[3][4] = {}, lr1 = T(0);
+  T lco[3][4], lr1 = T(0);
+  {
+    // powers of r_s = r1 / 2, r1; d(delta_o)/dr1 = sum_q q r^{q-1} co[o][q], times
+    // 1/2 for s = 0
+    T pw[2][5];
 #pragma unroll
-  for (int s = 0; s < 2; ++s) {
-    const T rs = s == 0 ? T(0.5) * r1 : r1;
-    const T sc = s == 0 ? T(0.5) : T(1);
-    T pw[5];
-    pw[0] = T(1);
+    for (int s = 0; s < 2; ++s) {
+      pw[s][0] = T(1);
+      pw[s][1] = s == 0 ? T(0.5) * r1 : r1;
 #pragma unroll
-    for (int q = 1; q <= 4; ++q) pw[q] = pw[q - 1] * rs;
+      for (int q = 2; q <= 4; ++q) pw[s][q] = pw[s][q - 1] * pw[s][1];
+    }
 #pragma unroll
     for (int o = 0; o < 3; ++o) {
-      T dr = T(0);
 #pragma unroll
-      for (int q = 1; q <= 4; ++q) {
-        lco[o][q - 1] += pw[q] * ld[s][o];
-        dr += T(q) * pw[q - 1] * co[o][q - 1];
+      for (int q = 1; q <= 4; ++q) lco[o][q - 1] = fma(pw[0][q], ld[0][o], pw[1][q] * ld[1][o]);
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        const T r = pw[s][1];
+        const T dr = fma(r, fma(r, fma(r, T(4) * co[o][3], T(3) * co[o][2]), T(2) * co[o][1]),
+                         co[o][0]);
+        lr1 = fma(s == 0 ? T(0.5) * dr : dr, ld[s][o], lr1);
       }
-      lr1 += sc * dr * ld[s][o];
     }
   }
   T lGp[3][4], lGuv[3][4], lZ = T(0), lZinv = T(0);
@@ -603,37 +574,49 @@ __device__ __forceinline__ void acoustic_adj(const AdjView<T>& v, const Acc& acc
   for (int q = 0; q < 4; ++q) {
     lGp[0][q] = lco[2][q];
     lGuv[0][q] = Z * lco[2][q];
-    lZ += Guv[0][q] * lco[2][q];
+    lZ = fma(Guv[0][q], lco[2][q], lZ);
     lGp[1][q] = Zinv * lco[0][q];
     lGuv[1][q] = lco[0][q];
-    lZinv += Gp[1][q] * lco[0][q];
+    lZinv = fma(Gp[1][q], lco[0][q], lZinv);
     lGp[2][q] = Zinv * lco[1][q];
     lGuv[2][q] = lco[1][q];
-    lZinv += Gp[2][q] * lco[1][q];
+    lZinv = fma(Gp[2][q], lco[1][q], lZinv);
   }
-  lZ -= lZinv * Zinv * Zinv;
-  const T lc = dth * lr1 + rk * lZ;
-  const T lrho = c * lZ - lc * c / (T(2) * rk);
-  const T lp = lc * c / (T(2) * pk);
+  lZ = fma(-lZinv * Zinv, Zinv, lZ);
+  // c^2 = gamma p / rho: dc/drho = -c / (2 rho), dc/dp = c / (2 p) = gamma / (2 Z)
+  const T lc = fma(dth, lr1, rk * lZ), hz = T(0.5) * Zinv;
+  const T lrho = fma(c, lZ, -lc * (c * c) * hz);  // c / rho = c^2 / Z
+  const T lp = lc * (v.gas.gamma * hz);
   T lpK = T(0), luK = T(0), lvK = T(0);
   const ScatterAdj<FAM, T> S = {v.lam, v.ps, nb, act};
   sac_family_adj<FAM, T>(S, lGp, lGuv, lpK, luK, lvK);
-  acc.node(FAM, i, j, lrho, luK, lvK, lp + lpK);
+  add4(v.lam + (size_t)(LAM_NODE + 4 * FAM) * ps + 4 * id, lrho, luK, lvK, lp + lpK);
 }
 
-// resident 256-thread blocks per SM requested of the acoustic and centre
-// adjoints (their register budget follows; they wait on scattered loads)
-#ifndef AF_ADJ_NODE_MINB
-#define AF_ADJ_NODE_MINB 3
-#endif
+// Blocks of the acoustic adjoint: BY rows of 32 consecutive nodes.  FP32 waits on
+// scattered loads and atomics: 256 threads, three blocks per SM (at most 85
+// registers).  FP64 is bound by its arithmetic unit and would spill: two warps,
+// registers as needed.
+template <typename T>
+struct AdjBlock {
+  static constexpr int BY = sizeof(T) == 4 ? 8 : 2, MINB = sizeof(T) == 4 ? 3 : 1;
+};
 
-template <int FAM, typename T>
-__global__ void __launch_bounds__(256, AF_ADJ_NODE_MINB)
+// the families by blockIdx.z
+template <typename T>
+__global__ void __launch_bounds__(32 * AdjBlock<T>::BY, AdjBlock<T>::MINB)
     k_adj_acoustic(const __grid_constant__ AdjView<T> v) {
+  pdl_wait();
   // a warp is one row of 32 consecutive nodes (blockDim.x == 32)
   const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
   const unsigned row = __ballot_sync(0xffffffffu, i < v.nx && j < v.ny);
-  if (i < v.nx && j < v.ny) acoustic_adj<FAM>(v, vec_adj(v), i, j, row);
+  if (i >= v.nx || j >= v.ny) return;
+  switch (blockIdx.z) {
+    case 0: acoustic_adj<0>(v, i, j, row); break;
+    case 1: acoustic_adj<1>(v, i, j, row); break;
+    case 2: acoustic_adj<2>(v, i, j, row); break;
+    default: acoustic_adj<3>(v, i, j, row); break;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -645,33 +628,34 @@ __global__ void __launch_bounds__(256, AF_ADJ_NODE_MINB)
 // vertex, two for an edge, no atomics) before writing lambda^n out.
 // ---------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(256, AF_ADJ_NODE_MINB)
-    k_adj_center(const __grid_constant__ AdjView<T> v) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
-  const size_t ps = v.ps;
-  if (i < v.nx && j < v.ny) {
-    const size_t id = (size_t)j * v.nx + i;
-    T* lc = v.lam + (size_t)(LAM_NODE + 12) * ps + 4 * id;  // the centre node's record
-    const T lw[4] = {lc[0], lc[1], lc[2], lc[3]};
-    T lU[4] = {T(0), T(0), T(0), T(0)};
-    if (lw[0] != T(0) || lw[1] != T(0) || lw[2] != T(0) || lw[3] != T(0)) {
-      zero4(lc);
-      const Gas<T>& g = v.gas;
-      // the recovered centre (rho~, u, v, p~) is W(U_c); lambda_U = (dW/dU)^T lambda_W
-      const T rho = g.rho_ref + v.scr[id], u = v.scr[ps + id], w = v.scr[2 * ps + id];
-      const T ri = T(1) / rho;
-      lU[0] = lw[0] - u * ri * lw[1] - w * ri * lw[2] + g.gm1 * T(0.5) * (u * u + w * w) * lw[3];
-      lU[1] = ri * lw[1] - g.gm1 * u * lw[3];
-      lU[2] = ri * lw[2] - g.gm1 * w * lw[3];
-      lU[3] = g.gm1 * lw[3];
-      // U_c = 9/4 Ubar - 1/16 sum_corners U(W) - 1/4 sum_edges U(W); the
-      // average of this cell has no other writer in this kernel
+__global__ void __launch_bounds__(128) k_adj_center(const __grid_constant__ AdjView<T> v) {
+  pdl_wait();
+  const size_t id = (size_t)blockIdx.x * 128 + threadIdx.x, ps = v.ps;
+  if (id >= (size_t)v.nx * v.ny) return;
+  T* lc = v.lam + (size_t)(LAM_NODE + 12) * ps + 4 * id;  // the centre node's record
+  const T lw[4] = {lc[0], lc[1], lc[2], lc[3]};
+  T lU[4] = {T(0), T(0), T(0), T(0)};
+  if (lw[0] != T(0) || lw[1] != T(0) || lw[2] != T(0) || lw[3] != T(0)) {
+    zero4(lc);
+    const Gas<T>& g = v.gas;
+    // the recovered centre (rho~, u, v, p~) is W(U_c); lambda_U = (dW/dU)^T lambda_W
+    const T rho = with_ref(g.rho_ref, v.scr[id]), u = v.scr[ps + id], w = v.scr[2 * ps + id];
+    const T ri = T(1) / rho, gl = g.gm1 * lw[3];
+    const T a1 = ri * lw[1], a2 = ri * lw[2];
+    lU[0] = fma(gl, T(0.5) * fma(u, u, w * w), fma(-w, a2, fma(-u, a1, lw[0])));
+    lU[1] = fma(-u, gl, a1);
+    lU[2] = fma(-w, gl, a2);
+    lU[3] = gl;
+    // U_c = 9/4 Ubar - 1/16 sum_corners U(W) - 1/4 sum_edges U(W); the
+    // average of this cell has no other writer in this kernel
 #pragma unroll
-      for (int k = 0; k < 4; ++k) v.lam[(size_t)(LAM_OUT + k) * ps + id] += T(2.25) * lU[k];
+    for (int k = 0; k < 4; ++k) {
+      T* o = v.lam + (size_t)(LAM_OUT + k) * ps + id;
+      *o = fma(T(2.25), lU[k], *o);
     }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v.lam[(size_t)(LAM_LU + k) * ps + id] = lU[k];
   }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) v.lam[(size_t)(LAM_LU + k) * ps + id] = lU[k];
 }
 
 // ---------------------------------------------------------------------------
@@ -692,10 +676,10 @@ __device__ __forceinline__ void tile_reverse(const StepArgs<float>& a, const Adj
   const int nx = a.nx, ny = a.ny;
   const size_t ps = v.ps;
   const Gas<float> gas = a.gas;
-  const VecAdj<float> acc = vec_adj(v);
   const float th_full = a.dt / a.h;
-  const float cst = a.dt / (36.f * a.h);
-  static_assert(TX == 32 && (3 * TX * TY) % NT == 0, "a warp is one row of one family");
+  // (a warp is consecutive points of whole rows of one family, and a round is taken
+  // or left by all its lanes)
+  static_assert(32 % TX == 0 && (TX * TY) % 32 == 0, "a warp holds rows of one family");
   const int lane = threadIdx.x & 31;
   for (int t = threadIdx.x; t < 3 * TX * TY; t += NT) {
     const int fam = t / (TX * TY), u = t - fam * (TX * TY);
@@ -706,66 +690,20 @@ __device__ __forceinline__ void tile_reverse(const StepArgs<float>& a, const Adj
     if (gi >= nx || gj >= ny) continue;
     const size_t id = (size_t)gj * nx + gi;
     // ---- fluxes (Eq. af-average-update), reversed ----
-    const int im = wrapc(gi - 1, nx), jm = wrapc(gj - 1, ny);
-    const size_t idl = (size_t)gj * nx + im, idb = (size_t)jm * nx + gi,
-                 idlb = (size_t)jm * nx + im;
-    float lex[4], ley[4];  // adjoints of the x- and y-fluxes the point enters
-    if (fam == 0) {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const double* lk = v.lin64[k];
-        const float c = (float)lk[id], l = (float)lk[idl], b = (float)lk[idb],
-                    lb = (float)lk[idlb];
-        lex[k] = (c - l) + (b - lb);
-        ley[k] = (c - b) + (l - lb);
-        v.lam[(size_t)(LAM_OUT + k) * ps + id] = c;
-      }
-    } else if (fam == 1) {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const double* lk = v.lin64[k];
-        lex[k] = (float)lk[id] - (float)lk[idl];
-        ley[k] = 0.f;
-      }
-    } else {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const double* lk = v.lin64[k];
-        lex[k] = 0.f;
-        ley[k] = (float)lk[id] - (float)lk[idb];
-      }
-    }
     const int wcP = (py + 2) * CW + (px + 2);
     const float4 wp = W[fam * WPL + wcP];
     float o0[4], lyh[4], lyf[4];  // sigma = 0 (own node), 1/2 and 1 (the point)
-#pragma unroll
-    for (int s = 0; s < 3; ++s) {
-      Prim<float> w;
-      if (s == 0) {
-        w = prim4(wp);
-      } else {
-        float* const* src = s == 1 ? a.half[fam] : a.out.pt[fam];
-        w.r = src[0][id];
-        w.u = src[1][id];
-        w.v = src[2][id];
-        w.p = src[3][id];
-      }
-      const float sc = cst * (s == 1 ? 4.f : 1.f);
-      float o[4] = {0.f, 0.f, 0.f, 0.f};
-      if (fam == 0) {
-        flux_x_adj(w, gas, lex, sc, o);
-        flux_y_adj(w, gas, ley, sc, o);
-      } else if (fam == 1) {
-        flux_x_adj(w, gas, lex, 4.f * sc, o);
-      } else {
-        flux_y_adj(w, gas, ley, 4.f * sc, o);
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if (s == 0) o0[k] = o[k];
-        else if (s == 1) lyh[k] = o[k];
-        else lyf[k] = o[k] + (float)v.lin64[4 + 4 * fam + k][id];
-      }
+    {
+      float* const* hp = a.half[fam];
+      float* const* np = a.out.pt[fam];
+      const Prim<float> wh = {hp[0][id], hp[1][id], hp[2][id], hp[3][id]};
+      const Prim<float> wf = {np[0][id], np[1][id], np[2][id], np[3][id]};
+      if (fam == 0)
+        point_fluxes_adj<0>(v, gi, gj, id, prim4(wp), wh, wf, o0, lyh, lyf);
+      else if (fam == 1)
+        point_fluxes_adj<1>(v, gi, gj, id, prim4(wp), wh, wf, o0, lyh, lyf);
+      else
+        point_fluxes_adj<2>(v, gi, gj, id, prim4(wp), wh, wf, o0, lyh, lyf);
     }
     // ---- point update (Sec. 6.1 steps 3-4), reversed, both durations ----
     const int ox = fam == 2 ? 1 : 0, oy = fam == 1 ? 1 : 0;
@@ -825,7 +763,8 @@ __device__ __forceinline__ void tile_reverse(const StepArgs<float>& a, const Adj
 #pragma unroll
         for (int k = 0; k < 4; ++k) lwf[k] = ly[k];
         // rho = rho_f + dp rho_P / (gamma p_P), with the increments at P itself
-        acc.inc(s, fam, gi, gj, ly[1], ly[2], fmaf(ly[0] * rp, igp, ly[3]));
+        add4(v.lam + (size_t)(LAM_INC + 4 * (4 * s + fam)) * ps + 4 * id, ly[1], ly[2],
+             fmaf(ly[0] * rp, igp, ly[3]), 0.f);
         lrP += ly[0] * d2 * igp;
         lpP += -ly[0] * d2 * rp * igp * ipp;
         ld[0] = ld[1] = ld[2] = 0.f;
@@ -878,8 +817,8 @@ __device__ __forceinline__ void tile_reverse(const StepArgs<float>& a, const Adj
       const size_t row1 = (row0 + nx == (size_t)ny * nx) ? 0 : row0 + nx;
       const int key = (ix + 2) + 8 * (iy + 2);
       const int lkey = __shfl_up_sync(mask, key, 1), rkey = __shfl_down_sync(mask, key, 1);
-      const bool give = lane > 0 && ((mask >> (lane - 1)) & 1u) && lkey == key;
-      const bool take = lane < 31 && ((mask >> (lane + 1)) & 1u) && rkey == key;
+      const bool give = px > 0 && ((mask >> (lane - 1)) & 1u) && lkey == key;
+      const bool take = px < TX - 1 && ((mask >> (lane + 1)) & 1u) && rkey == key;
 #pragma unroll
       for (int b = 0; b < 3; ++b) {
         float nd[3][4], ic[3][3];
@@ -926,12 +865,14 @@ __device__ __forceinline__ void tile_reverse(const StepArgs<float>& a, const Adj
 #pragma unroll
           for (int q = 0; q < 3; ++q) {
             const float w1 = lx1[q] * ly1[b];
-            acc.node(fam_of(q, b), gi + ix1 + (q >> 1), gj + iy1 + (b >> 1), 0.f, w1 * lu1,
-                     w1 * lv1, 0.f);
+            add4(v.lam + (size_t)(LAM_NODE + 4 * fam_of(q, b)) * ps +
+                     4 * cell_id(v, gi + ix1 + (q >> 1), gj + iy1 + (b >> 1)),
+                 0.f, w1 * lu1, w1 * lv1, 0.f);
           }
       }
     }
-    acc.node(fam, gi, gj, o0[0] + lrP, o0[1] + luP, o0[2] + lvP, o0[3] + lpP);
+    add4(v.lam + (size_t)(LAM_NODE + 4 * fam) * ps + 4 * id, o0[0] + lrP, o0[1] + luP, o0[2] + lvP,
+         o0[3] + lpP);
   }
 }
 
@@ -954,6 +895,7 @@ __global__ void __launch_bounds__(NT, MINB)
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(pc.bar) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  pdl_wait();
   __syncthreads();
   const int tcols = (a.nx + TX - 1) / TX, ntiles = tcols * ((a.ny + TY - 1) / TY);
   int tile = blockIdx.x;
@@ -972,37 +914,84 @@ __global__ void __launch_bounds__(NT, MINB)
   }
 }
 
-// Launches the fused reverse sweep when the pipelined kernel accepts the grid
-// (cudaErrorNotSupported otherwise).
+// The fused reverse sweep, one CTA per tile of TX x TY cells (any grid).
+template <int TX, int TY, int NT, int MINB, bool COMP>
+__global__ void __launch_bounds__(NT, MINB)
+    k_fused_adj(const __grid_constant__ StepArgs<float> a, const __grid_constant__ AdjView<float> v) {
+  using G = FusedGeom<TX, TY>;
+  extern __shared__ __align__(16) float4 smem4[];
+  pdl_wait();
+  PipeCtx none = {nullptr, 0u, 0u};
+  const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY;
+  fused_tile<TX, TY, NT, COMP, false, false, true>(a, none, i0, j0, -1, -1, false);
+  tile_reverse<TX, TY, NT>(a, v, smem4, reinterpret_cast<const float*>(smem4 + 4 * G::WPL), i0,
+                           j0);
+}
+
+template <int TX, int TY, int NT, int MINB, bool COMP>
+inline cudaError_t launch_adj_tiles(cudaStream_t s, const StepArgs<float>& a,
+                                    const AdjView<float>& v) {
+  using G = FusedGeom<TX, TY>;
+  constexpr auto kern = k_fused_adj<TX, TY, NT, MINB, COMP>;
+  const cudaError_t e = allow_smem<kern>(G::SMEM);
+  if (e != cudaSuccess) return e;
+  return launch_dependent(kern, dim3((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY), NT, G::SMEM, s,
+                          a, v);
+}
+
+// Tile geometries of the fused reverse sweep, chosen as the step's (STEP_GEOMS):
+// the least (waves x measured time of one wave, FP32_COMP, GB300).  Two CTAs of
+// 256 threads share an SM on 32 x 8 tiles: one recomputes its step (FP32 issue)
+// while the other waits on its scatter, which makes up for the larger halo at
+// every size (one CTA of 32 x 16 tiles 840, the pipelined 32 x 32 tiles 804, 786 us
+// per adjoint step at 1024^2); the pipelined sweep is as fast on the largest grids
+// (2048^2: 2.95 against 2.99 ms).  Adjoint step, pipelined 32 x 32 tiles -> chosen:
+// 64^2 116 -> 49 us, 128^2 118 -> 54, 192^2 119 -> 66, 256^2 123 -> 84; 1021 x 1024,
+// which the pipelined sweep does not take, 1.69 (per stage) -> 0.81 ms.
+enum { ADJ_8x8, ADJ_16x8, ADJ_16x16, ADJ_32x8, ADJ_32x24, ADJ_PIPE, N_ADJ_GEOMS };
+struct AdjGeometry {
+  int tx, ty;
+  int per_sm;      // resident CTAs per SM
+  float us, fill;  // time of one wave, and once per sweep
+};
+constexpr AdjGeometry ADJ_GEOMS[N_ADJ_GEOMS] = {
+    {8, 8, 1, 15.f, 0.f},     {16, 8, 1, 18.f, 0.f},  {16, 16, 1, 30.f, 0.f},
+    {32, 8, 2, 34.6f, 12.f},  {32, 24, 1, 72.f, 0.f}, {FUSED_TX, FUSED_TY, 1, 68.5f, 20.f}};
+
+inline int choose_adj_geometry(const StepArgs<float>& a, int sms) {
+  int best = ADJ_32x8;
+  float best_us = 1e30f;
+  for (int g = 0; g < N_ADJ_GEOMS; ++g) {
+    const AdjGeometry& q = ADJ_GEOMS[g];
+    if (g == ADJ_PIPE && !pipe_eligible(a)) continue;
+    const int64_t tiles = (int64_t)((a.nx + q.tx - 1) / q.tx) * ((a.ny + q.ty - 1) / q.ty);
+    const int64_t wave = (int64_t)sms * q.per_sm;
+    const float us = (float)((tiles + wave - 1) / wave) * q.us + q.fill;
+    if (us < best_us) {
+      best_us = us;
+      best = g;
+    }
+  }
+  return best;
+}
+
+// The fused reverse sweep on one CTA per tile (af_adj_tiles.cu).
 template <bool COMP>
-inline cudaError_t launch_fused_adjoint(cudaStream_t s, const StepArgs<float>& a, int ctas,
-                                        const TileMaps* maps, const AdjView<float>& v) {
+cudaError_t launch_adj_small(int geom, cudaStream_t s, const StepArgs<float>& a,
+                             const AdjView<float>& v);
+
+// The persistent pipelined sweep on `ctas` CTAs (grids it accepts).
+template <bool COMP>
+inline cudaError_t launch_adj_pipe(cudaStream_t s, const StepArgs<float>& a, int ctas,
+                                   const TileMaps* maps, const AdjView<float>& v) {
   using G = FusedGeom<FUSED_TX, FUSED_TY>;
-  if (!(ctas > 0 && pipe_eligible(a))) return cudaErrorNotSupported;
   constexpr auto kern = k_fused_adj_pipe<FUSED_TX, FUSED_TY, FUSED_NT, AF_FUSED_MINB, COMP>;
   const cudaError_t e = allow_smem<kern>(G::SMEM_PIPE);
   if (e != cudaSuccess) return e;
   static TileMaps none;
   const int ntiles = ((a.nx + FUSED_TX - 1) / FUSED_TX) * ((a.ny + FUSED_TY - 1) / FUSED_TY);
-  kern<<<ntiles < ctas ? ntiles : ctas, FUSED_NT, G::SMEM_PIPE, s>>>(a, maps ? *maps : none,
-                                                                       maps ? 1 : 0, v);
-  return cudaGetLastError();
-}
-
-// Sixteen planes converted in one launch (the adjoint state in and out).
-template <typename A, typename B>
-struct Cast16 {
-  const A* src[16];
-  B* dst[16];
-};
-
-template <typename A, typename B>
-__global__ void k_cast16(const __grid_constant__ Cast16<A, B> c, size_t n) {
-  for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n;
-       t += (size_t)gridDim.x * blockDim.x) {
-#pragma unroll
-    for (int p = 0; p < 16; ++p) c.dst[p][t] = (B)c.src[p][t];
-  }
+  return launch_dependent(kern, dim3(ntiles < ctas ? ntiles : ctas), FUSED_NT, G::SMEM_PIPE, s, a,
+                          maps ? *maps : none, maps ? 1 : 0, v);
 }
 
 // lambda^n out: the averages' planes and the point families' node records into
@@ -1015,6 +1004,7 @@ struct AdjOut {
 template <typename T>
 __global__ void k_adj_out(const __grid_constant__ AdjView<T> v,
                           const __grid_constant__ AdjOut<T> o, size_t n) {
+  pdl_wait();
   const size_t ps = v.ps;
   const Gas<T>& g = v.gas;
   for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n;

@@ -484,94 +484,63 @@ af_status adjoint_impl(af_handle* h, double dt, const af_state_f64* lin, const a
   v.ny = h->ny;
   v.h = f.h;
   v.dt = f.dt;
+  v.dth = f.dth;
   v.gas = f.gas;
   v.variant = f.variant;
   cudaStream_t s = h->stream;
-  // lambda^{n+1} in (FP64 -> working precision, no storage offsets)
-  af_status st = ensure_staging(h);
-  if (st != AF_OK) return st;
-  Cast16<double, T> cin;
-  const af_state_f64 staged = planes_at(h->staging, h->N);
-  if (where == AF_HOST &&
-      copy_planes(&staged, lin, h->N, cudaMemcpyHostToDevice, s) != cudaSuccess)
-    return cuda_fail(h);
-  for (int p = 0; p < 16; ++p) {
-    const double* src = where == AF_HOST ? plane_in(&staged, p) : plane_in(lin, p);
-    cin.src[p] = src;
-    cin.dst[p] = v.lam + (size_t)(LAM_IN + p) * v.ps;
-    v.lin64[p] = src;
+  // lambda^{n+1}: FP64 device planes, the caller's or staged ones
+  af_state_f64 staged;
+  if (where == AF_HOST) {
+    const af_status st = ensure_staging(h);
+    if (st != AF_OK) return st;
+    staged = planes_at(h->staging, h->N);
+    if (copy_planes(&staged, lin, h->N, cudaMemcpyHostToDevice, s) != cudaSuccess)
+      return cuda_fail(h);
   }
-  dim3 blk(32, 8), grd((h->nx + 31) / 32, (h->ny + 7) / 8);
-  // FP32 modes on grids the pipelined kernel accepts: one fused launch
-  // recomputes each tile's step in shared memory and reverses its fluxes and
-  // point updates there (AF_ADJ_FUSED=0 selects the kernel-per-stage sweep)
-  if constexpr (std::is_same<T, float>::value) {
-    const char* fz = getenv("AF_ADJ_FUSED");
-    if (h->fused && h->pipe_ctas > 0 && pipe_eligible(f) && !(fz && fz[0] == '0')) {
-      // node and increment records start at zero (planes LAM_NODE ... LAM_INC + 31):
-      // cleared here only after an incomplete step or on first use, since
-      // their consumers clear them as they read them
-      if (!h->adj_clean &&
-          cudaMemsetAsync(v.lam + (size_t)LAM_NODE * v.ps, 0, plane * 48, s) != cudaSuccess)
-        return cuda_fail(h);
-      h->adj_clean = 0;
-      if (launch_fused_adjoint<COMP>(s, f, h->pipe_ctas, h->tma ? &h->tmaps[h->cur] : nullptr,
-                                     v) != cudaSuccess)
-        return cuda_fail(h);
-      k_adj_acoustic<0, T><<<grd, blk, 0, s>>>(v);
-      k_adj_acoustic<1, T><<<grd, blk, 0, s>>>(v);
-      k_adj_acoustic<2, T><<<grd, blk, 0, s>>>(v);
-      k_adj_acoustic<3, T><<<grd, blk, 0, s>>>(v);
-      k_adj_center<T><<<grd, blk, 0, s>>>(v);
-      AdjOut<T> out;
-      for (int p = 0; p < 16; ++p)
-        out.dst[p] = where == AF_HOST ? h->staging + (size_t)p * h->N : (double*)plane_in(lout, p);
-      k_adj_out<T><<<grid1d(h->N), 256, 0, s>>>(v, out, h->N);
-      if (where == AF_HOST &&
-          copy_planes(lout, &staged, h->N, cudaMemcpyDeviceToHost, s) != cudaSuccess)
-        return cuda_fail(h);
-      if (cudaGetLastError() != cudaSuccess) return cuda_fail(h);
-      return adjoint_done(h);
-    }
-  }
-  // the stage-by-stage sweep reads lambda^{n+1} in the working precision
-  k_cast16<<<grid1d(h->N), 256, 0, s>>>(cin, h->N);
-  // forward intermediates of the step from the handle's current state: the
-  // pipelined fused kernel stores them where it runs (FP32 modes), else the
-  // unfused kernels
-  bool fused_inter = false;
-  if constexpr (std::is_same<T, float>::value) {
-    if (h->fused && h->pipe_ctas > 0 && pipe_eligible(f)) {
-      if (launch_fused_step<COMP, true>(s, f, true, h->pipe_ctas,
-                                        h->tma ? &h->tmaps[h->cur] : nullptr) != cudaSuccess)
-        return cuda_fail(h);
-      fused_inter = true;
-    }
-  }
-  if (!fused_inter) {
-    if (launch_ref_intermediates<T, COMP>(f, s) != cudaSuccess) return cuda_fail(h);
-  }
-  // reverse sweep: the centre and increment records start at zero (planes
-  // LAM_NODE + 12 ... LAM_INC + 31 are contiguous; the sweep writes the other
-  // node records before adding to them)
+  for (int p = 0; p < 16; ++p) v.lin64[p] = plane_in(where == AF_HOST ? &staged : lin, p);
+  // node and increment records start at zero (planes LAM_NODE ... LAM_INC + 31):
+  // cleared here only after an incomplete step or on first use, since their
+  // consumers clear them as they read them
   if (!h->adj_clean &&
-      cudaMemsetAsync(v.lam + (size_t)(LAM_NODE + 12) * v.ps, 0, plane * 36, s) != cudaSuccess)
+      cudaMemsetAsync(v.lam + (size_t)LAM_NODE * v.ps, 0, plane * 48, s) != cudaSuccess)
     return cuda_fail(h);
   h->adj_clean = 0;
-  k_adj_flux<T><<<grd, blk, 0, s>>>(v);
-  k_adj_points<0, T><<<grd, blk, 0, s>>>(v);
-  k_adj_points<1, T><<<grd, blk, 0, s>>>(v);
-  k_adj_points<2, T><<<grd, blk, 0, s>>>(v);
-  k_adj_acoustic<0, T><<<grd, blk, 0, s>>>(v);
-  k_adj_acoustic<1, T><<<grd, blk, 0, s>>>(v);
-  k_adj_acoustic<2, T><<<grd, blk, 0, s>>>(v);
-  k_adj_acoustic<3, T><<<grd, blk, 0, s>>>(v);
-  k_adj_center<T><<<grd, blk, 0, s>>>(v);
+  // FP32 modes: one fused launch recomputes each tile's step in shared memory and
+  // reverses its fluxes and point updates there (AF_PATH=ref, AF_PIPE=0 or
+  // AF_ADJ_FUSED=0 select the kernels per stage)
+  cudaError_t e = cudaSuccess;
+  bool fused = false;
+  if constexpr (std::is_same<T, float>::value) {
+    const char* fz = getenv("AF_ADJ_FUSED");
+    const TileMaps* maps = h->tma ? &h->tmaps[h->cur] : nullptr;
+    const bool pipe = h->pipe_ctas > 0 && pipe_eligible(f);
+    fused = h->fused && h->pipe_ctas > 0 && !(fz && fz[0] == '0');
+    if (fused) {
+      // (geom < 0: an explicit AF_PIPE, on the pipelined kernel's tiles)
+      const int g = h->geom >= 0 ? choose_adj_geometry(f, h->pipe_ctas)
+                                 : (pipe ? ADJ_PIPE : ADJ_32x8);
+      e = g == ADJ_PIPE ? launch_adj_pipe<COMP>(s, f, h->pipe_ctas, maps, v)
+                        : launch_adj_small<COMP>(g, s, f, v);
+    } else if (h->fused && pipe) {
+      e = launch_fused_step<COMP, true>(s, f, true, h->pipe_ctas, maps);
+    } else {
+      e = launch_ref_intermediates<T, COMP>(f, s);
+    }
+  } else {
+    e = launch_ref_intermediates<T, COMP>(f, s);
+  }
+  if (e == cudaSuccess && !fused)
+    e = launch_dependent(k_adj_points<T>, dim3(ref_blocks(f), 3), REF_THREADS, 0, s, v);
+  if (e != cudaSuccess) return cuda_fail(h);
+  constexpr int BY = AdjBlock<T>::BY;
+  launch_dependent(k_adj_acoustic<T>, dim3((h->nx + 31) / 32, (h->ny + BY - 1) / BY, 4),
+                   dim3(32, BY), 0, s, v);
+  launch_dependent(k_adj_center<T>, dim3((unsigned)((h->N + 127) / 128)), 128, 0, s, v);
   // lambda^n out
   AdjOut<T> out;
   for (int p = 0; p < 16; ++p)
     out.dst[p] = where == AF_HOST ? h->staging + (size_t)p * h->N : (double*)plane_in(lout, p);
-  k_adj_out<T><<<grid1d(h->N), 256, 0, s>>>(v, out, h->N);
+  launch_dependent(k_adj_out<T>, dim3(grid1d(h->N)), 256, 0, s, v, out, h->N);
   if (where == AF_HOST &&
       copy_planes(lout, &staged, h->N, cudaMemcpyDeviceToHost, s) != cudaSuccess)
     return cuda_fail(h);

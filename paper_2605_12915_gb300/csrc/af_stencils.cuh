@@ -341,12 +341,12 @@ __device__ __forceinline__ void af_sac_V_adj(const Scatter& S, const T lGp[3][4]
     lpK -= T(2) * leep;
     luK -= T(2) * leeu;
     lvK -= T(2) * leev;
-    c0p1[0] = T(0) + leep + leop;
-    c0p1[1] = T(0) + leeu;
-    c0p1[2] = T(0) + leev + leov;
-    c0m1[0] = T(0) + leep - leop;
-    c0m1[1] = T(0) + leeu;
-    c0m1[2] = T(0) + leev - leov;
+    c0p1[0] = leep + leop;
+    c0p1[1] = leeu;
+    c0p1[2] = leev + leov;
+    c0m1[0] = leep - leop;
+    c0m1[1] = leeu;
+    c0m1[2] = leev - leov;
   }
   {  // orbit (+-0, +-2) half cells
     const T leep = fma(T(0.666666666666666666667), lGp[0][3], fma(T(-2.0), lGp[0][2], fma(T(1.95492965855137201461), lGp[0][1], fma(T(-0.5), lGp[0][0], T(0)))));
@@ -357,12 +357,12 @@ __device__ __forceinline__ void af_sac_V_adj(const Scatter& S, const T lGp[3][4]
     lpK -= T(2) * leep;
     luK -= T(2) * leeu;
     lvK -= T(2) * leev;
-    c0p2[0] = T(0) + leep + leop;
-    c0p2[1] = T(0) + leeu;
-    c0p2[2] = T(0) + leev + leov;
-    c0m2[0] = T(0) + leep - leop;
-    c0m2[1] = T(0) + leeu;
-    c0m2[2] = T(0) + leev - leov;
+    c0p2[0] = leep + leop;
+    c0p2[1] = leeu;
+    c0p2[2] = leev + leov;
+    c0m2[0] = leep - leop;
+    c0m2[1] = leeu;
+    c0m2[2] = leev - leov;
   }
   {  // orbit (+-1, +-0) half cells
     const T leep = fma(T(-1.33333333333333333333), lGp[0][3], fma(T(5.0), lGp[0][2], fma(T(-5.81971863420548805845), lGp[0][1], fma(T(2.0), lGp[0][0], T(0)))));
@@ -373,8 +373,8 @@ __device__ __forceinline__ void af_sac_V_adj(const Scatter& S, const T lGp[3][4]
     lpK -= T(2) * leep;
     luK -= T(2) * leeu;
     lvK -= T(2) * leev;
-    S.pair(1, 0, T(0) + leep + loep, T(0) + leeu + loeu, T(0) + leev,
-           T(0) + leep - loep, T(0) + leeu - loeu, T(0) + leev);
+    S.pair(1, 0, leep + loep, leeu + loeu, leev,
+           leep - loep, leeu - loeu, leev);
   }
   {  // orbit (+-1, +-1) half cells
     const T leep = fma(T(1.33333333333333333333), lGp[0][3], fma(T(-4.0), lGp[0][2], fma(T(2.5464790894703253723), lGp[0][1], T(0))));
@@ -389,10 +389,10 @@ __device__ __forceinline__ void af_sac_V_adj(const Scatter& S, const T lGp[3][4]
     lpK -= T(4) * leep;
     luK -= T(4) * leeu;
     lvK -= T(4) * leev;
-    S.pair(1, 1, T(0) + leep + loep + leop, T(0) + leeu + loeu + loou, T(0) + leev + leov + loov,
-           T(0) + leep - loep + leop, T(0) + leeu - loeu - loou, T(0) + leev + leov - loov);
-    S.pair(1, -1, T(0) + leep + loep - leop, T(0) + leeu + loeu - loou, T(0) + leev - leov - loov,
-           T(0) + leep - loep - leop, T(0) + leeu - loeu + loou, T(0) + leev - leov + loov);
+    S.pair(1, 1, leep + loep + leop, leeu + loeu + loou, leev + leov + loov,
+           leep - loep + leop, leeu - loeu - loou, leev + leov - loov);
+    S.pair(1, -1, leep + loep - leop, leeu + loeu - loou, leev - leov - loov,
+           leep - loep - leop, leeu - loeu + loou, leev - leov + loov);
   }
   {  // orbit (+-1, +-2) half cells
     const T leep = fma(T(-0.666666666666666666667), lGp[0][3], fma(T(1.5), lGp[0][2], fma(T(-0.636619772367581343076), lGp[0][1], T(0))));
@@ -407,10 +407,10 @@ __device__ __forceinline__ void af_sac_V_adj(const Scatter& S, const T lGp[3][4]
     lpK -= T(4) * leep;
     luK -= T(4) * leeu;
     lvK -= T(4) * leev;
-    S.pair(1, 2, T(0) + leep + loep + leop, T(0) + leeu + loeu + loou, T(0) + leev + leov + loov,
-           T(0) + leep - loep + leop, T(0) + leeu - loeu - loou, T(0) + leev + leov - loov);
-    S.pair(1, -2, T(0) + leep + loep - leop, T(0) + leeu + loeu - loou, T(0) + leev - leov - loov,
-           T(0) + leep - loep - leop, T(0) + leeu - loeu + loou, T(0) + leev - leov + loov);
+    S.pair(1, 2, leep + loep + leop, leeu + loeu + loou, leev + leov + loov,
+           leep - loep + leop, leeu - loeu - loou, leev + leov - loov);
+    S.pair(1, -2, leep + loep - leop, leeu + loeu - loou, leev - leov - loov,
+           leep - loep - leop, leeu - loeu + loou, leev - leov + loov);
   }
   {  // orbit (+-2, +-0) half cells
     const T leep = fma(T(0.666666666666666666667), lGp[0][3], fma(T(-2.0), lGp[0][2], fma(T(1.95492965855137201461), lGp[0][1], fma(T(-0.5), lGp[0][0], T(0)))));
@@ -421,8 +421,8 @@ __device__ __forceinline__ void af_sac_V_adj(const Scatter& S, const T lGp[3][4]
     lpK -= T(2) * leep;
     luK -= T(2) * leeu;
     lvK -= T(2) * leev;
-    S.pair(2, 0, T(0) + leep + loep, T(0) + leeu + loeu, T(0) + leev,
-           T(0) + leep - loep, T(0) + leeu - loeu, T(0) + leev);
+    S.pair(2, 0, leep + loep, leeu + loeu, leev,
+           leep - loep, leeu - loeu, leev);
   }
   {  // orbit (+-2, +-1) half cells
     const T leep = fma(T(-0.666666666666666666667), lGp[0][3], fma(T(1.5), lGp[0][2], fma(T(-0.636619772367581343076), lGp[0][1], T(0))));
@@ -437,11 +437,11 @@ __device__ __forceinline__ void af_sac_V_adj(const Scatter& S, const T lGp[3][4]
     lpK -= T(4) * leep;
     luK -= T(4) * leeu;
     lvK -= T(4) * leev;
-    S.triple(1, T(0) + leep + loep + leop, T(0) + leeu + loeu + loou, T(0) + leev + leov + loov,
-             T(0) + leep - loep + leop, T(0) + leeu - loeu - loou, T(0) + leev + leov - loov,
+    S.triple(1, leep + loep + leop, leeu + loeu + loou, leev + leov + loov,
+             leep - loep + leop, leeu - loeu - loou, leev + leov - loov,
              c0p1[0], c0p1[1], c0p1[2]);
-    S.triple(-1, T(0) + leep + loep - leop, T(0) + leeu + loeu - loou, T(0) + leev - leov - loov,
-             T(0) + leep - loep - leop, T(0) + leeu - loeu + loou, T(0) + leev - leov + loov,
+    S.triple(-1, leep + loep - leop, leeu + loeu - loou, leev - leov - loov,
+             leep - loep - leop, leeu - loeu + loou, leev - leov + loov,
              c0m1[0], c0m1[1], c0m1[2]);
   }
   {  // orbit (+-2, +-2) half cells
@@ -457,11 +457,11 @@ __device__ __forceinline__ void af_sac_V_adj(const Scatter& S, const T lGp[3][4]
     lpK -= T(4) * leep;
     luK -= T(4) * leeu;
     lvK -= T(4) * leev;
-    S.triple(2, T(0) + leep + loep + leop, T(0) + leeu + loeu + loou, T(0) + leev + leov + loov,
-             T(0) + leep - loep + leop, T(0) + leeu - loeu - loou, T(0) + leev + leov - loov,
+    S.triple(2, leep + loep + leop, leeu + loeu + loou, leev + leov + loov,
+             leep - loep + leop, leeu - loeu - loou, leev + leov - loov,
              c0p2[0], c0p2[1], c0p2[2]);
-    S.triple(-2, T(0) + leep + loep - leop, T(0) + leeu + loeu - loou, T(0) + leev - leov - loov,
-             T(0) + leep - loep - leop, T(0) + leeu - loeu + loou, T(0) + leev - leov + loov,
+    S.triple(-2, leep + loep - leop, leeu + loeu - loou, leev - leov - loov,
+             leep - loep - leop, leeu - loeu + loou, leev - leov + loov,
              c0m2[0], c0m2[1], c0m2[2]);
   }
 }
@@ -644,12 +644,12 @@ __device__ __forceinline__ void af_sac_EV_adj(const Scatter& S, const T lGp[3][4
     lpK -= T(2) * leep;
     luK -= T(2) * leeu;
     lvK -= T(2) * leev;
-    c0p1[0] = T(0) + leep + leop;
-    c0p1[1] = T(0) + leeu;
-    c0p1[2] = T(0) + leev + leov;
-    c0m1[0] = T(0) + leep - leop;
-    c0m1[1] = T(0) + leeu;
-    c0m1[2] = T(0) + leev - leov;
+    c0p1[0] = leep + leop;
+    c0p1[1] = leeu;
+    c0p1[2] = leev + leov;
+    c0m1[0] = leep - leop;
+    c0m1[1] = leeu;
+    c0m1[2] = leev - leov;
   }
   {  // orbit (+-1, +-0) half cells
     const T leep = fma(T(2.66666666666666666667), lGp[0][3], fma(T(-4.0), lGp[0][2], fma(T(-2.0), lGp[0][1], fma(T(2.0), lGp[0][0], T(0)))));
@@ -660,8 +660,8 @@ __device__ __forceinline__ void af_sac_EV_adj(const Scatter& S, const T lGp[3][4
     lpK -= T(2) * leep;
     luK -= T(2) * leeu;
     lvK -= T(2) * leev;
-    S.pair(1, 0, T(0) + leep + loep, T(0) + leeu + loeu, T(0) + leev,
-           T(0) + leep - loep, T(0) + leeu - loeu, T(0) + leev);
+    S.pair(1, 0, leep + loep, leeu + loeu, leev,
+           leep - loep, leeu - loeu, leev);
   }
   {  // orbit (+-1, +-1) half cells
     const T leep = fma(T(-1.33333333333333333333), lGp[0][3], fma(T(2.0), lGp[0][2], T(0)));
@@ -676,10 +676,10 @@ __device__ __forceinline__ void af_sac_EV_adj(const Scatter& S, const T lGp[3][4
     lpK -= T(4) * leep;
     luK -= T(4) * leeu;
     lvK -= T(4) * leev;
-    S.pair(1, 1, T(0) + leep + loep + leop, T(0) + leeu + loeu + loou, T(0) + leev + leov + loov,
-           T(0) + leep - loep + leop, T(0) + leeu - loeu - loou, T(0) + leev + leov - loov);
-    S.pair(1, -1, T(0) + leep + loep - leop, T(0) + leeu + loeu - loou, T(0) + leev - leov - loov,
-           T(0) + leep - loep - leop, T(0) + leeu - loeu + loou, T(0) + leev - leov + loov);
+    S.pair(1, 1, leep + loep + leop, leeu + loeu + loou, leev + leov + loov,
+           leep - loep + leop, leeu - loeu - loou, leev + leov - loov);
+    S.pair(1, -1, leep + loep - leop, leeu + loeu - loou, leev - leov - loov,
+           leep - loep - leop, leeu - loeu + loou, leev - leov + loov);
   }
   {  // orbit (+-2, +-0) half cells
     const T leep = fma(T(-1.33333333333333333333), lGp[0][3], fma(T(1.0), lGp[0][2], fma(T(1.0), lGp[0][1], fma(T(-0.5), lGp[0][0], T(0)))));
@@ -690,8 +690,8 @@ __device__ __forceinline__ void af_sac_EV_adj(const Scatter& S, const T lGp[3][4
     lpK -= T(2) * leep;
     luK -= T(2) * leeu;
     lvK -= T(2) * leev;
-    S.pair(2, 0, T(0) + leep + loep, T(0) + leeu + loeu, T(0) + leev,
-           T(0) + leep - loep, T(0) + leeu - loeu, T(0) + leev);
+    S.pair(2, 0, leep + loep, leeu + loeu, leev,
+           leep - loep, leeu - loeu, leev);
   }
   {  // orbit (+-2, +-1) half cells
     const T leep = fma(T(0.666666666666666666667), lGp[0][3], fma(T(-0.5), lGp[0][2], T(0)));
@@ -706,11 +706,11 @@ __device__ __forceinline__ void af_sac_EV_adj(const Scatter& S, const T lGp[3][4
     lpK -= T(4) * leep;
     luK -= T(4) * leeu;
     lvK -= T(4) * leev;
-    S.triple(1, T(0) + leep + loep + leop, T(0) + leeu + loeu + loou, T(0) + leev + leov + loov,
-             T(0) + leep - loep + leop, T(0) + leeu - loeu - loou, T(0) + leev + leov - loov,
+    S.triple(1, leep + loep + leop, leeu + loeu + loou, leev + leov + loov,
+             leep - loep + leop, leeu - loeu - loou, leev + leov - loov,
              c0p1[0], c0p1[1], c0p1[2]);
-    S.triple(-1, T(0) + leep + loep - leop, T(0) + leeu + loeu - loou, T(0) + leev - leov - loov,
-             T(0) + leep - loep - leop, T(0) + leeu - loeu + loou, T(0) + leev - leov + loov,
+    S.triple(-1, leep + loep - leop, leeu + loeu - loou, leev - leov - loov,
+             leep - loep - leop, leeu - loeu + loou, leev - leov + loov,
              c0m1[0], c0m1[1], c0m1[2]);
   }
 }
@@ -891,8 +891,8 @@ __device__ __forceinline__ void af_sac_EH_adj(const Scatter& S, const T lGp[3][4
     lpK -= T(2) * leep;
     luK -= T(2) * leeu;
     lvK -= T(2) * leev;
-    S(0, 1, T(0) + leep + leop, T(0) + leeu, T(0) + leev + leov);
-    S(0, -1, T(0) + leep - leop, T(0) + leeu, T(0) + leev - leov);
+    S(0, 1, leep + leop, leeu, leev + leov);
+    S(0, -1, leep - leop, leeu, leev - leov);
   }
   {  // orbit (+-0, +-2) half cells
     const T leep = fma(T(-1.33333333333333333333), lGp[0][3], fma(T(1.0), lGp[0][2], fma(T(1.0), lGp[0][1], fma(T(-0.5), lGp[0][0], T(0)))));
@@ -903,8 +903,8 @@ __device__ __forceinline__ void af_sac_EH_adj(const Scatter& S, const T lGp[3][4
     lpK -= T(2) * leep;
     luK -= T(2) * leeu;
     lvK -= T(2) * leev;
-    S(0, 2, T(0) + leep + leop, T(0) + leeu, T(0) + leev + leov);
-    S(0, -2, T(0) + leep - leop, T(0) + leeu, T(0) + leev - leov);
+    S(0, 2, leep + leop, leeu, leev + leov);
+    S(0, -2, leep - leop, leeu, leev - leov);
   }
   {  // orbit (+-1, +-0) half cells
     const T leep = fma(T(1.33333333333333333333), lGp[0][3], fma(T(-3.0), lGp[0][2], fma(T(2.0), lGp[0][1], T(0))));
@@ -915,8 +915,8 @@ __device__ __forceinline__ void af_sac_EH_adj(const Scatter& S, const T lGp[3][4
     lpK -= T(2) * leep;
     luK -= T(2) * leeu;
     lvK -= T(2) * leev;
-    S.pair(1, 0, T(0) + leep + loep, T(0) + leeu + loeu, T(0) + leev,
-           T(0) + leep - loep, T(0) + leeu - loeu, T(0) + leev);
+    S.pair(1, 0, leep + loep, leeu + loeu, leev,
+           leep - loep, leeu - loeu, leev);
   }
   {  // orbit (+-1, +-1) half cells
     const T leep = fma(T(-1.33333333333333333333), lGp[0][3], fma(T(2.0), lGp[0][2], T(0)));
@@ -931,10 +931,10 @@ __device__ __forceinline__ void af_sac_EH_adj(const Scatter& S, const T lGp[3][4
     lpK -= T(4) * leep;
     luK -= T(4) * leeu;
     lvK -= T(4) * leev;
-    S.pair(1, 1, T(0) + leep + loep + leop, T(0) + leeu + loeu + loou, T(0) + leev + leov + loov,
-           T(0) + leep - loep + leop, T(0) + leeu - loeu - loou, T(0) + leev + leov - loov);
-    S.pair(1, -1, T(0) + leep + loep - leop, T(0) + leeu + loeu - loou, T(0) + leev - leov - loov,
-           T(0) + leep - loep - leop, T(0) + leeu - loeu + loou, T(0) + leev - leov + loov);
+    S.pair(1, 1, leep + loep + leop, leeu + loeu + loou, leev + leov + loov,
+           leep - loep + leop, leeu - loeu - loou, leev + leov - loov);
+    S.pair(1, -1, leep + loep - leop, leeu + loeu - loou, leev - leov - loov,
+           leep - loep - leop, leeu - loeu + loou, leev - leov + loov);
   }
   {  // orbit (+-1, +-2) half cells
     const T leep = fma(T(0.666666666666666666667), lGp[0][3], fma(T(-0.5), lGp[0][2], T(0)));
@@ -949,10 +949,10 @@ __device__ __forceinline__ void af_sac_EH_adj(const Scatter& S, const T lGp[3][4
     lpK -= T(4) * leep;
     luK -= T(4) * leeu;
     lvK -= T(4) * leev;
-    S.pair(1, 2, T(0) + leep + loep + leop, T(0) + leeu + loeu + loou, T(0) + leev + leov + loov,
-           T(0) + leep - loep + leop, T(0) + leeu - loeu - loou, T(0) + leev + leov - loov);
-    S.pair(1, -2, T(0) + leep + loep - leop, T(0) + leeu + loeu - loou, T(0) + leev - leov - loov,
-           T(0) + leep - loep - leop, T(0) + leeu - loeu + loou, T(0) + leev - leov + loov);
+    S.pair(1, 2, leep + loep + leop, leeu + loeu + loou, leev + leov + loov,
+           leep - loep + leop, leeu - loeu - loou, leev + leov - loov);
+    S.pair(1, -2, leep + loep - leop, leeu + loeu - loou, leev - leov - loov,
+           leep - loep - leop, leeu - loeu + loou, leev - leov + loov);
   }
 }
 
@@ -1043,8 +1043,8 @@ __device__ __forceinline__ void af_sac_C_adj(const Scatter& S, const T lGp[3][4]
     lpK -= T(2) * leep;
     luK -= T(2) * leeu;
     lvK -= T(2) * leev;
-    S(0, 1, T(0) + leep + leop, T(0) + leeu, T(0) + leev + leov);
-    S(0, -1, T(0) + leep - leop, T(0) + leeu, T(0) + leev - leov);
+    S(0, 1, leep + leop, leeu, leev + leov);
+    S(0, -1, leep - leop, leeu, leev - leov);
   }
   {  // orbit (+-1, +-0) half cells
     const T leep = fma(T(-2.66666666666666666667), lGp[0][3], fma(T(2.0), lGp[0][1], T(0)));
@@ -1055,8 +1055,8 @@ __device__ __forceinline__ void af_sac_C_adj(const Scatter& S, const T lGp[3][4]
     lpK -= T(2) * leep;
     luK -= T(2) * leeu;
     lvK -= T(2) * leev;
-    S.pair(1, 0, T(0) + leep + loep, T(0) + leeu + loeu, T(0) + leev,
-           T(0) + leep - loep, T(0) + leeu - loeu, T(0) + leev);
+    S.pair(1, 0, leep + loep, leeu + loeu, leev,
+           leep - loep, leeu - loeu, leev);
   }
   {  // orbit (+-1, +-1) half cells
     const T leep = fma(T(1.33333333333333333333), lGp[0][3], T(0));
@@ -1071,9 +1071,9 @@ __device__ __forceinline__ void af_sac_C_adj(const Scatter& S, const T lGp[3][4]
     lpK -= T(4) * leep;
     luK -= T(4) * leeu;
     lvK -= T(4) * leev;
-    S.pair(1, 1, T(0) + leep + loep + leop, T(0) + leeu + loeu + loou, T(0) + leev + leov + loov,
-           T(0) + leep - loep + leop, T(0) + leeu - loeu - loou, T(0) + leev + leov - loov);
-    S.pair(1, -1, T(0) + leep + loep - leop, T(0) + leeu + loeu - loou, T(0) + leev - leov - loov,
-           T(0) + leep - loep - leop, T(0) + leeu - loeu + loou, T(0) + leev - leov + loov);
+    S.pair(1, 1, leep + loep + leop, leeu + loeu + loou, leev + leov + loov,
+           leep - loep + leop, leeu - loeu - loou, leev + leov - loov);
+    S.pair(1, -1, leep + loep - leop, leeu + loeu - loou, leev - leov - loov,
+           leep - loep - leop, leeu - loeu + loou, leev - leov + loov);
   }
 }

@@ -307,8 +307,9 @@ def emit_family_adjoint(name, reps):
                         # two-member orbits: the one odd combination is n0 - n1
                         sgn = 1 if (dx, dy) == members[0] else -1
                     expr.append(("+" if sgn > 0 else "-") + " " + nm)
-                e = " ".join(expr) if expr else "+ T(0)"
-                vals.append("T(0) " + e)
+                # (a leading zero would cost an addition: x + 0 is not x for x = -0)
+                e = " ".join(expr) if expr else "T(0)"
+                vals.append(e[2:] if e.startswith("+ ") else e)
             member_vals[(dx, dy)] = vals
         for (dx, dy) in members:
             vals = member_vals[(dx, dy)]
