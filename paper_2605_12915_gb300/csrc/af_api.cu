@@ -100,6 +100,7 @@ struct NvtxRange {
 // the exchange streams (a cudaMemcpyAsync of the word can queue behind them
 // and hold up the step stream for a whole state transfer).
 __global__ void k_flags_to_host(const unsigned* d, unsigned* h) {
+  pdl_wait();
   if (threadIdx.x == 0) {
     *(volatile unsigned*)h = *(volatile const unsigned*)d;
     __threadfence_system();
@@ -149,42 +150,82 @@ struct Offsets {
   double rho, p, e;  // subtracted from rho, p and the energy average on import
 };
 
+// FP64 planes to the working precision and back.  Memory is the floor (208 B per
+// cell in FP32_COMP, 0.13 ms at 2048^2); what bound these was the FP64 unit, which
+// also runs the conversion instructions (36 and 40 of its instructions per cell,
+// 0.27 and 0.32 ms), and loads that waited for the stores between them.  The
+// conversions are integer work now (narrow, widen), only the offsets and the
+// compensated words are FP64 additions (12 per cell), and a cell's loads are all
+// issued first: 0.160 and 0.138 ms.
+constexpr int COPY_THREADS = 128;
+
+// `flags`: the error word to clear, or null
 template <typename T, bool COMP>
-__global__ void k_import(F64Planes src, Planes<T> dst, size_t N, Offsets o) {
-  for (size_t id = (size_t)blockIdx.x * blockDim.x + threadIdx.x; id < N;
-       id += (size_t)gridDim.x * blockDim.x) {
+__global__ void __launch_bounds__(COPY_THREADS)
+    k_import(const __grid_constant__ F64Planes src, const __grid_constant__ Planes<T> dst,
+             size_t N, Offsets o, unsigned* flags) {
+  pdl_wait();
+  if (flags && blockIdx.x == 0 && threadIdx.x == 0) *flags = 0u;
+  for (size_t id = (size_t)blockIdx.x * COPY_THREADS + threadIdx.x; id < N;
+       id += (size_t)gridDim.x * COPY_THREADS) {
+    double x[16];
+#pragma unroll
+    for (int p = 0; p < 16; ++p) x[p] = src.p[p][id];
+#pragma unroll
     for (int k = 0; k < 4; ++k) {
-      double x = src.p[k][id] - (k == 0 ? o.rho : (k == 3 ? o.e : 0.0));
-      T hi = (T)x;
-      dst.avg[k][id] = hi;
-      if (COMP) dst.lo[k][id] = (T)(x - (double)hi);
+      if constexpr (sizeof(T) == 8) {
+        dst.avg[k][id] = x[k];
+      } else {
+        const double y = k == 0 ? x[k] - o.rho : (k == 3 ? x[k] - o.e : x[k]);
+        const float hi = narrow(y);
+        dst.avg[k][id] = hi;
+        if (COMP) dst.lo[k][id] = narrow(y - widen(hi));
+      }
     }
+#pragma unroll
     for (int f = 0; f < 3; ++f)
-      for (int k = 0; k < 4; ++k)
-        dst.pt[f][k][id] =
-            (T)(src.p[4 + 4 * f + k][id] - (k == 0 ? o.rho : (k == 3 ? o.p : 0.0)));
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const double y = x[4 + 4 * f + k];
+        if constexpr (sizeof(T) == 8)
+          dst.pt[f][k][id] = y;
+        else
+          dst.pt[f][k][id] = narrow(k == 0 ? y - o.rho : (k == 3 ? y - o.p : y));
+      }
   }
 }
 
 template <typename T, bool COMP>
-__global__ void k_export(Planes<T> src, F64Out dst, size_t N, Offsets o) {
-  for (size_t id = (size_t)blockIdx.x * blockDim.x + threadIdx.x; id < N;
-       id += (size_t)gridDim.x * blockDim.x) {
-    for (int k = 0; k < 4; ++k)
-      dst.p[k][id] = ((double)src.avg[k][id] + (COMP ? (double)src.lo[k][id] : 0.0)) +
-                     (k == 0 ? o.rho : (k == 3 ? o.e : 0.0));
+__global__ void __launch_bounds__(COPY_THREADS)
+    k_export(const __grid_constant__ Planes<T> src, const __grid_constant__ F64Out dst, size_t N,
+             Offsets o) {
+  pdl_wait();
+  for (size_t id = (size_t)blockIdx.x * COPY_THREADS + threadIdx.x; id < N;
+       id += (size_t)gridDim.x * COPY_THREADS) {
+    T x[16], lo[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      x[k] = src.avg[k][id];
+      if (COMP) lo[k] = src.lo[k][id];
+    }
+#pragma unroll
     for (int f = 0; f < 3; ++f)
-      for (int k = 0; k < 4; ++k)
-        dst.p[4 + 4 * f + k][id] =
-            (double)src.pt[f][k][id] + (k == 0 ? o.rho : (k == 3 ? o.p : 0.0));
+#pragma unroll
+      for (int k = 0; k < 4; ++k) x[4 + 4 * f + k] = src.pt[f][k][id];
+#pragma unroll
+    for (int p = 0; p < 16; ++p) {
+      const int k = p & 3;
+      if constexpr (sizeof(T) == 8) {
+        dst.p[p][id] = x[p];
+      } else {
+        double y = widen(x[p]);
+        if (COMP && p < 4) y += widen(lo[k]);
+        if (k == 0) y += o.rho;
+        if (k == 3) y += p < 4 ? o.e : o.p;
+        dst.p[p][id] = y;
+      }
+    }
   }
-}
-
-template <typename A, typename B>
-__global__ void k_cast(const A* src, B* dst, size_t N) {
-  for (size_t id = (size_t)blockIdx.x * blockDim.x + threadIdx.x; id < N;
-       id += (size_t)gridDim.x * blockDim.x)
-    dst[id] = (B)src[id];
 }
 
 Offsets offsets_of(const af_handle* h) {
@@ -192,8 +233,8 @@ Offsets offsets_of(const af_handle* h) {
   return o;
 }
 
-int grid1d(size_t N) {
-  size_t b = (N + 255) / 256;
+int grid1d(size_t N, int threads = 256) {
+  size_t b = (N + threads - 1) / threads;
   if (b > 152 * 32) b = 152 * 32;
   return (int)(b < 1 ? 1 : b);
 }
@@ -353,8 +394,10 @@ af_status cuda_fail(af_handle* h) {
 // Enqueues the copy of the device error word into the host mirror (read by the
 // next call without waiting).
 af_status flags_to_host(af_handle* h) {
-  k_flags_to_host<<<1, 32, 0, h->stream>>>(h->d_flags, h->h_flags_dev);
-  return cudaGetLastError() == cudaSuccess ? AF_OK : AF_ERR_CUDA;
+  return launch_dependent(k_flags_to_host, dim3(1), dim3(32), 0, h->stream, h->d_flags,
+                          h->h_flags_dev) == cudaSuccess
+             ? AF_OK
+             : AF_ERR_CUDA;
 }
 
 // Address under which the current device reaches the host plane p directly:
@@ -374,8 +417,10 @@ const void* mapped_host_plane(const af_handle* h, const void* p) {
 }
 
 // Enqueues the conversion of `in` into the current state on the handle's
-// stream (pageable host planes are first copied to the staging buffer).
-af_status import_enqueue(af_handle* h, const af_state_f64* in, af_memory where) {
+// stream (pageable host planes are first copied to the staging buffer); the same
+// kernel clears the error word `flags`, if not null.
+af_status import_enqueue(af_handle* h, const af_state_f64* in, af_memory where,
+                         unsigned* flags = nullptr) {
   F64Planes src;
   if (where == AF_HOST) {
     // pinned planes are read in place by the import kernel, pageable ones are
@@ -393,14 +438,24 @@ af_status import_enqueue(af_handle* h, const af_state_f64* in, af_memory where) 
   } else {
     for (int p = 0; p < 16; ++p) src.p[p] = plane_in(in, p);
   }
-  int g = grid1d(h->N);
+  const dim3 g(grid1d(h->N, COPY_THREADS)), t(COPY_THREADS);
+  const Offsets o = offsets_of(h);
+  cudaError_t e = cudaSuccess;
   switch (h->prec) {
-    case AF_FP64: k_import<double, false><<<g, 256, 0, h->stream>>>(src, planes_of<double>(h, h->cur), h->N, offsets_of(h)); break;
-    case AF_FP32: k_import<float, false><<<g, 256, 0, h->stream>>>(src, planes_of<float>(h, h->cur), h->N, offsets_of(h)); break;
-    case AF_FP32_COMP: k_import<float, true><<<g, 256, 0, h->stream>>>(src, planes_of<float>(h, h->cur), h->N, offsets_of(h)); break;
+    case AF_FP64:
+      e = launch_dependent(k_import<double, false>, g, t, 0, h->stream, src,
+                           planes_of<double>(h, h->cur), h->N, o, flags);
+      break;
+    case AF_FP32:
+      e = launch_dependent(k_import<float, false>, g, t, 0, h->stream, src,
+                           planes_of<float>(h, h->cur), h->N, o, flags);
+      break;
+    case AF_FP32_COMP:
+      e = launch_dependent(k_import<float, true>, g, t, 0, h->stream, src,
+                           planes_of<float>(h, h->cur), h->N, o, flags);
+      break;
   }
-  if (cudaGetLastError() != cudaSuccess) return cuda_fail(h);
-  return AF_OK;
+  return e == cudaSuccess ? AF_OK : cuda_fail(h);
 }
 
 // True if `in` shares a byte with the target of an outgoing copy of an
@@ -423,10 +478,10 @@ af_status wait_outgoing(af_handle* h) {
   return AF_OK;
 }
 
-// Clears the latched device error once the stream has passed the new state
-// (and, the caller having called wait_outgoing, any outgoing copies).
+// Waits until the stream has passed the new state (and, the caller having called
+// wait_outgoing, any outgoing copies) and clears the latched device error, whose
+// device word the import has cleared.
 af_status import_finish(af_handle* h) {
-  if (cudaMemsetAsync(h->d_flags, 0, sizeof(unsigned), h->stream) != cudaSuccess) return cuda_fail(h);
   if (cudaGetLastError() != cudaSuccess) return cuda_fail(h);
   if (cudaStreamSynchronize(h->stream) != cudaSuccess) return cuda_fail(h);
   *(volatile unsigned*)h->h_flags = 0;
@@ -436,21 +491,31 @@ af_status import_finish(af_handle* h) {
 }
 
 af_status import_state(af_handle* h, const af_state_f64* in, af_memory where) {
-  af_status st = import_enqueue(h, in, where);
+  af_status st = import_enqueue(h, in, where, h->d_flags);
   return st != AF_OK ? st : import_finish(h);
 }
 
 // Enqueues the conversion of the current state into the FP64 planes dst.
 af_status export_enqueue(af_handle* h, const F64Out& dst) {
-  int g = grid1d(h->N);
+  const dim3 g(grid1d(h->N, COPY_THREADS)), t(COPY_THREADS);
+  const Offsets o = offsets_of(h);
+  cudaError_t e = cudaSuccess;
   switch (h->prec) {
-    case AF_FP64: k_export<double, false><<<g, 256, 0, h->stream>>>(planes_of<double>(h, h->cur), dst, h->N, offsets_of(h)); break;
-    case AF_FP32: k_export<float, false><<<g, 256, 0, h->stream>>>(planes_of<float>(h, h->cur), dst, h->N, offsets_of(h)); break;
-    case AF_FP32_COMP: k_export<float, true><<<g, 256, 0, h->stream>>>(planes_of<float>(h, h->cur), dst, h->N, offsets_of(h)); break;
+    case AF_FP64:
+      e = launch_dependent(k_export<double, false>, g, t, 0, h->stream,
+                           planes_of<double>(h, h->cur), dst, h->N, o);
+      break;
+    case AF_FP32:
+      e = launch_dependent(k_export<float, false>, g, t, 0, h->stream,
+                           planes_of<float>(h, h->cur), dst, h->N, o);
+      break;
+    case AF_FP32_COMP:
+      e = launch_dependent(k_export<float, true>, g, t, 0, h->stream,
+                           planes_of<float>(h, h->cur), dst, h->N, o);
+      break;
   }
-  return cudaGetLastError() == cudaSuccess ? AF_OK : cuda_fail(h);
+  return e == cudaSuccess ? AF_OK : cuda_fail(h);
 }
-
 
 }  // namespace
 extern "C" af_status af_sync(af_handle* h);
@@ -807,7 +872,7 @@ af_status af_exchange_state(af_handle* h, const af_state_f64* out, const af_stat
     F64Out dst;
     for (int p = 0; p < 16; ++p) dst.p[p] = (double*)plane_in(out, p);
     af_status st = export_enqueue(h, dst);
-    if (st == AF_OK) st = import_enqueue(h, in, AF_DEVICE);
+    if (st == AF_OK) st = import_enqueue(h, in, AF_DEVICE, h->d_flags);
     return st != AF_OK ? st : import_finish(h);
   }
   // host: both directions by copy engines, on two streams of their own, so that
@@ -845,7 +910,7 @@ af_status af_exchange_state(af_handle* h, const af_state_f64* out, const af_stat
   if (cudaEventRecord(h->ev_join, h->aux) != cudaSuccess ||
       cudaStreamWaitEvent(h->stream, h->ev_in, 0) != cudaSuccess)
     return cuda_fail(h);
-  st = import_enqueue(h, &staged, AF_DEVICE);
+  st = import_enqueue(h, &staged, AF_DEVICE, h->d_flags);
   if (st == AF_OK) st = import_finish(h);
   if (st == AF_OK) {
     h->out_pending = 1;

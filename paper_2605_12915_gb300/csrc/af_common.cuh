@@ -88,6 +88,29 @@ __device__ __forceinline__ bool at_least_one(double x) { return __double2hiint(x
 __device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsqrt_t(double x) { return rsqrt(x); }
 
+// (float)x and (double)x on the integer units (the conversion instructions run at
+// the FP64 unit's rate): the exponent is rebiased and the mantissa shifted, with
+// round to nearest even on narrowing.  Zeros pass; subnormals, infinities, NaN and
+// values beyond the float range take the conversion instruction.  Same bits as it.
+__device__ __forceinline__ float narrow(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned a = hi & 0x7fffffffu;
+  if (a - 0x38100000u < 0x0fe00000u) {  // exponents of normal floats
+    unsigned m = __funnelshift_l(lo, a - 0x38000000u, 3);
+    m += ((lo << 3) + (m & 1u)) > 0x80000000u ? 1u : 0u;
+    return __uint_as_float(m | (hi & 0x80000000u));
+  }
+  if ((a | lo) == 0u) return __uint_as_float(hi);
+  return (float)x;
+}
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu;
+  if (a - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(u << 29));
+  if (a == 0u) return __hiloint2double((int)u, 0);
+  return (double)x;
+}
+
 // Programmatic dependent launch: the next kernel of the stream may be scheduled
 // now (its blocks then sit in pdl_wait), and this one's input is complete.  A
 // kernel launched without the attribute passes both at once.
