@@ -44,11 +44,13 @@ struct af_handle {
   int cur;               // index of the current state
   void* scratch[44];     // wc 4, inc 24, half 12, fx 4
   double* staging;       // 16 FP64 planes for host/device exchange (lazy)
-  unsigned* d_flags;
+  unsigned* d_flags;     // two words: error bits, then (d_top) the reduction's top wave speed
+  unsigned* d_top;       // (zero between calls)
   unsigned* h_flags;     // pinned mirror, written asynchronously after each step
   unsigned* h_flags_dev; // the device's address of that mirror
-  double* d_red;         // reduction partials + result
-  double* h_red;         // pinned
+  double* d_red;         // reduction partials
+  double* h_red;         // pinned, written by the reduction
+  double* h_red_dev;     // the device's address of it
   int red_blocks;
   int broken;
   int fused;             // 1: fused single-pass kernel for the FP32 modes
@@ -282,7 +284,8 @@ void launch_fc_step(af_handle* h, double dt) {
     n.ex[k] = (double*)h->scratch[12 + k];
     n.ey[k] = (double*)h->scratch[16 + k];
   }
-  launch_dependent(k_center<double, false>, dim3(b), REF_THREADS, 0, h->stream, a);
+  launch_dependent(k_center<double, false>, dim3(b), REF_THREADS, 0, h->stream, a,
+                   (unsigned*)nullptr);
   launch_fc_points(a, h->stream);
   launch_dependent(k_node_flux<double>, dim3(b), REF_THREADS, 0, h->stream, a, n);
   launch_dependent(k_average<double, false>, dim3(b), REF_THREADS, 0, h->stream, a, n);
@@ -696,17 +699,19 @@ af_status af_init(af_handle** out, const af_grid* g, double gamma, const af_stat
   for (int s = 0; s < 2; ++s)
     for (int p = 0; p < 20; ++p) h->state[s][p] = base + plane * (size_t)(20 * s + p);
   for (int p = 0; p < 44; ++p) h->scratch[p] = base + plane * (size_t)(40 + p);
-  h->red_blocks = 152 * 4;
-  bool ok = cudaMalloc(&h->d_flags, sizeof(unsigned)) == cudaSuccess &&
+  h->red_blocks = 152 * 8;
+  bool ok = cudaMalloc(&h->d_flags, 2 * sizeof(unsigned)) == cudaSuccess &&
+            cudaMemsetAsync(h->d_flags, 0, 2 * sizeof(unsigned), h->stream) == cudaSuccess &&
             cudaMallocHost(&h->h_flags, sizeof(unsigned)) == cudaSuccess &&
             cudaHostGetDevicePointer((void**)&h->h_flags_dev, h->h_flags, 0) == cudaSuccess &&
-            cudaMalloc(&h->d_red, sizeof(double) * (RED_VALS * h->red_blocks + AF_NINV)) ==
-                cudaSuccess &&
-            cudaMallocHost(&h->h_red, sizeof(double) * AF_NINV) == cudaSuccess;
+            cudaMalloc(&h->d_red, sizeof(double) * RED_VALS * h->red_blocks) == cudaSuccess &&
+            cudaMallocHost(&h->h_red, sizeof(double) * AF_NINV) == cudaSuccess &&
+            cudaHostGetDevicePointer((void**)&h->h_red_dev, h->h_red, 0) == cudaSuccess;
   if (!ok) {
     af_destroy(h);
     return AF_ERR_ALLOC;
   }
+  h->d_top = h->d_flags + 1;
   if (prec != AF_FP64 && h->pipe_ctas > 0) {
     // tensor maps of both state buffers for the pipelined kernel; AF_TMA=0 (or a
     // driver without the encoder) stages every tile by cp.async instead
@@ -992,36 +997,34 @@ af_status af_reduce_invariants(af_handle* h, double* out) {
   DeviceGuard guard(h->device);
   if (wait_outgoing(h) != AF_OK) return AF_ERR_CUDA;
   double* partial = h->d_red;
-  double* res = h->d_red + (size_t)RED_VALS * h->red_blocks;
+  const int blocks = (int)std::min<size_t>(h->red_blocks, (h->N + RED_THREADS - 1) / RED_THREADS);
   if (h->prec == AF_FP64) {
     StepArgs<double> a = step_args<double>(h, 1.0);
-    k_center<double, false><<<ref_blocks(a), REF_THREADS, 0, h->stream>>>(a);
+    k_center<double, false, true><<<ref_blocks(a), REF_THREADS, 0, h->stream>>>(a, h->d_top);
     RedArgs<double> r;
     r.st = a.in;
     for (int k = 0; k < 4; ++k) r.wc[k] = a.wc[k];
-    r.nx = h->nx; r.ny = h->ny; r.gamma = h->gamma; r.h = h->h; r.partial = partial;
+    r.nx = h->nx; r.ny = h->ny; r.gamma = h->gamma; r.h = h->h; r.partial = partial; r.top = h->d_top;
     r.rho_ref = h->rho_ref; r.p_ref = h->p_ref; r.e_ref = h->p_ref / (h->gamma - 1.0);
-    k_inv_partial<double, false><<<h->red_blocks, RED_THREADS, 0, h->stream>>>(r);
+    k_inv_partial<double, false><<<blocks, RED_THREADS, 0, h->stream>>>(r);
   } else {
     StepArgs<float> a = step_args<float>(h, 1.0);
     RedArgs<float> r;
     r.st = a.in;
     for (int k = 0; k < 4; ++k) r.wc[k] = a.wc[k];
-    r.nx = h->nx; r.ny = h->ny; r.gamma = h->gamma; r.h = h->h; r.partial = partial;
+    r.nx = h->nx; r.ny = h->ny; r.gamma = h->gamma; r.h = h->h; r.partial = partial; r.top = h->d_top;
     r.rho_ref = h->rho_ref; r.p_ref = h->p_ref; r.e_ref = h->p_ref / (h->gamma - 1.0);
     if (h->prec == AF_FP32_COMP) {
-      k_center<float, true><<<ref_blocks(a), REF_THREADS, 0, h->stream>>>(a);
-      k_inv_partial<float, true><<<h->red_blocks, RED_THREADS, 0, h->stream>>>(r);
+      k_center<float, true, true><<<ref_blocks(a), REF_THREADS, 0, h->stream>>>(a, h->d_top);
+      k_inv_partial<float, true><<<blocks, RED_THREADS, 0, h->stream>>>(r);
     } else {
-      k_center<float, false><<<ref_blocks(a), REF_THREADS, 0, h->stream>>>(a);
-      k_inv_partial<float, false><<<h->red_blocks, RED_THREADS, 0, h->stream>>>(r);
+      k_center<float, false, true><<<ref_blocks(a), REF_THREADS, 0, h->stream>>>(a, h->d_top);
+      k_inv_partial<float, false><<<blocks, RED_THREADS, 0, h->stream>>>(r);
     }
   }
-  k_inv_final<<<1, 32, 0, h->stream>>>(partial, h->red_blocks, h->h, res);
+  k_inv_final<<<1, 32 * RED_VALS, 0, h->stream>>>(partial, blocks, h->h, h->h_red_dev,
+                                                      h->d_top);
   if (cudaGetLastError() != cudaSuccess) return cuda_fail(h);
-  if (cudaMemcpyAsync(h->h_red, res, sizeof(double) * (AF_NINV - 1), cudaMemcpyDeviceToHost,
-                      h->stream) != cudaSuccess)
-    return cuda_fail(h);
   af_status st = af_sync(h);
   if (st == AF_ERR_CUDA || st == AF_ERR_STATE) return st;
   for (int k = 0; k < AF_NINV - 1; ++k) out[k] = h->h_red[k];

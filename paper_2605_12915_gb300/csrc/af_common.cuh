@@ -90,25 +90,43 @@ __device__ __forceinline__ double rsqrt_t(double x) { return rsqrt(x); }
 
 // (float)x and (double)x on the integer units (the conversion instructions run at
 // the FP64 unit's rate): the exponent is rebiased and the mantissa shifted, with
-// round to nearest even on narrowing.  Zeros pass; subnormals, infinities, NaN and
-// values beyond the float range take the conversion instruction.  Same bits as it.
+// round to nearest even on narrowing.  Same values as the instructions, subnormals,
+// infinities and NaN included; none of the branches holds an FP64 instruction, which
+// would be issued, predicated off, for every warp.
 __device__ __forceinline__ float narrow(double x) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned a = hi & 0x7fffffffu;
+  const unsigned a = hi & 0x7fffffffu, sign = hi & 0x80000000u;
   if (a - 0x38100000u < 0x0fe00000u) {  // exponents of normal floats
     unsigned m = __funnelshift_l(lo, a - 0x38000000u, 3);
     m += ((lo << 3) + (m & 1u)) > 0x80000000u ? 1u : 0u;
-    return __uint_as_float(m | (hi & 0x80000000u));
+    return __uint_as_float(m | sign);
   }
-  if ((a | lo) == 0u) return __uint_as_float(hi);
-  return (float)x;
+  if (a >= 0x47f00000u)  // beyond the floats: infinity, or NaN
+    return __uint_as_float(a > 0x7ff00000u || (a == 0x7ff00000u && lo) ? 0x7fffffffu
+                                                                      : sign | 0x7f800000u);
+  // below 2^-126: round(|x| 2^149), the bits of a subnormal float
+  const unsigned e = a >> 20, sh = 926u - e;
+  if (sh > 63u) return __uint_as_float(sign);
+  const unsigned long long M =
+      ((unsigned long long)((a & 0xfffffu) | 0x100000u) << 32) | lo;
+  unsigned long long q = M >> sh;
+  const unsigned long long rest = M << (64u - sh), half = 1ull << 63;
+  if (rest > half || (rest == half && (q & 1ull))) ++q;
+  return __uint_as_float(sign | (unsigned)q);
 }
 __device__ __forceinline__ double widen(float x) {
-  const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu;
-  if (a - 0x00800000u < 0x7f000000u)
-    return __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(u << 29));
-  if (a == 0u) return __hiloint2double((int)u, 0);
-  return (double)x;
+  const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu, sign = u & 0x80000000u;
+  unsigned hi = (a >> 3) + 0x38000000u, lo = u << 29;
+  if (a - 0x00800000u >= 0x7f000000u) {
+    if (a >= 0x7f800000u) {  // infinity, NaN
+      hi = 0x7ff00000u | ((a & 0x7fffffu) >> 3);
+    } else {  // zero, or a subnormal: a 2^-149 by way of the float a
+      const unsigned b = __float_as_uint(__uint2float_rn(a));
+      hi = a ? (b >> 3) + 0x38000000u - (149u << 20) : 0u;
+      lo = b << 29;
+    }
+  }
+  return __hiloint2double((int)(sign | hi), (int)lo);
 }
 
 // Programmatic dependent launch: the next kernel of the stream may be scheduled
@@ -170,6 +188,19 @@ __device__ __forceinline__ void flux_y(const Prim<T>& w, const Gas<T>& g, T f[4]
   f[1] = m * w.u;
   f[2] = fma(m, w.v, w.p);
   f[3] = w.v * fma(p, g.g_gm1, (T(0.5) * rho) * fma(w.u, w.u, w.v * w.v));
+}
+
+__device__ __forceinline__ float narrow_any(float x) { return x; }
+__device__ __forceinline__ float narrow_any(double x) { return narrow(x); }
+
+// |u| + c of a node (absolute rho, p) in FP32, within 2e-7 relative (three roundings each in |u| and in the
+// square of c, which its root halves, one in the sum); infinity where FP32 cannot tell
+__device__ __forceinline__ float wave_speed_f32(float r, float u, float v, float p, float gamma) {
+  const float a = fmaxf(fabsf(u), fabsf(v)), b = fminf(fabsf(u), fabsf(v));
+  const float t = a > 0.f ? b / a : 0.f;
+  const float c2 = gamma * (p / r);
+  if (!(c2 > 1e-30f) || (a > 0.f && a < 1e-30f)) return INFINITY;
+  return fmaf(a, sqrtf(fmaf(t, t, 1.f)), sqrtf(c2));
 }
 
 // ---- Q2 Lagrange basis on nodes -1, 0, 1 (Sec. 4) ----------------------------

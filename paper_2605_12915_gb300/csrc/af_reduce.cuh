@@ -3,15 +3,26 @@
 // kinetic energy, wave-speed / positivity extrema and the vorticity integral
 // (Sec. 6.4).  Two passes: per-block partials with warp shuffles, then one
 // block folds the partials in a fixed order (bitwise reproducible).
+//
+// What bounds them: the FP64 unit (two lanes per cycle and SM).  A cell took about
+// 575 of its instructions: ten CUDA logarithms, eight square roots and seven
+// divisions, 32 conversions, minima and maxima.  It takes 160 now: the
+// logarithm by a table (7 instructions, below), conversions on the integer units,
+// the minima on the stored floats, the wave speed evaluated in FP64 only where its
+// FP32 value comes near the grid's largest one, which the centre recovery before it
+// finds; common factors taken out of the sums.
+// A call at 2048^2 in FP32_COMP: 1.34 ms, 4.69 before (of which 0.22 ms was the
+// fold of the partials by one thread per value, now one warp); the FP64 unit is 85%
+// busy in k_inv_partial.
 #pragma once
 
 #include "af_common.cuh"
 
 namespace af {
 
-enum { RED_SUMS = 8, RED_VALS = 11, RED_THREADS = 256 };
-// partial layout: sums mass, mx, my, E, entropy(Simpson), entropy(avg), KE, vorticity;
-// then max(|u|+c), min rho, min p
+enum { RED_SUMS = 8, RED_VALS = 11, RED_THREADS = 128, RED_WARPS = RED_THREADS / 32 };
+// partial layout: sums mass, mx, my, E, 9 x entropy(Simpson), entropy(avg), KE,
+// 6/h x vorticity; then max(|u|+c), min rho, min p
 
 template <typename T>
 struct RedArgs {
@@ -20,85 +31,180 @@ struct RedArgs {
   int nx, ny;
   double gamma, h;
   double rho_ref, p_ref, e_ref;  // storage offsets (see Gas)
-  double* partial;  // [gridDim.x][RED_VALS]
+  const unsigned* top;  // bits of the grid's largest FP32 wave speed
+  double* partial;      // [RED_VALS][gridDim.x]
 };
 
-__device__ __forceinline__ double entropy_density(double r, double p, double gamma) {
-  return -r * (log(p) - gamma * log(r));
+// ---- logarithm by table (P. T. P. Tang, "Table-driven implementation of the
+// logarithm function in IEEE floating-point arithmetic", ACM TOMS 16, 1990) ----
+// x = 2^e m with m in [0.707, 1.414); c the nearest of 512 points (nine bits of
+// m), g = 1/c rounded, r = g m - 1 (one rounding, |r| <= 2^-10): log x = e log 2 -
+// log g + log(1 + r), the last by its series.  The terms from r^4 on are below
+// 2^-30 of r and are summed in FP32; everything else in FP64.  Around x = 1, e = 0
+// and the point nearest to 1 is 1 itself (log g = 0), so small results keep their
+// relative accuracy (2 ulp measured over 1e-9 < |log x| < 20).
+constexpr int LOG_POINTS = 512;
+constexpr unsigned LOG_FIRST = 0x3fe6a000u;  // high word of the first point, 0.70703
+struct LogEntry {
+  double g, mlog_g;  // 1/c and -log(g)
+};
+__device__ __forceinline__ void fill_log_table(LogEntry* tab, int thread, int threads) {
+  for (int i = thread; i < LOG_POINTS; i += threads) {
+    const double g = 1.0 / __hiloint2double((int)(LOG_FIRST + ((unsigned)i << 11)), 0);
+    tab[i].g = g;
+    tab[i].mlog_g = -log(g);
+  }
+}
+__device__ __forceinline__ double log_by_table(double x, const LogEntry* tab) {
+  const unsigned hi = (unsigned)__double2hiint(x);
+  if (hi - 0x00100000u >= 0x7fe00000u) return log(x);  // not a positive normal number
+  const unsigned t = hi - LOG_FIRST + 0x400u;  // (+ half a point: the nearest one)
+  const int e = (int)t >> 20;
+  const LogEntry c = tab[(t & 0xfffffu) >> 11];
+  const double m = __hiloint2double((int)(hi - ((unsigned)e << 20)), __double2loint(x));
+  const double r = fma(m, c.g, -1.0);
+  const double head = fma(widen((float)e), 0.69314718055994530942, c.mlog_g);
+  const float rf = narrow(r);
+  const float tail = fmaf(rf, fmaf(rf, -1.0f / 6.0f, 0.2f), -0.25f);
+  const double q = fma(r, fma(r, widen(tail), 1.0 / 3.0), -0.5);
+  return head + fma(r * r, q, r);
+}
+
+__device__ __forceinline__ double entropy_density(double r, double p, double gamma,
+                                                  const LogEntry* tab) {
+  return r * fma(gamma, log_by_table(r, tab), -log_by_table(p, tab));
+}
+
+// running minimum of stored values (NaN ignored)
+__device__ __forceinline__ void keep_min(float& m, float x) { m = fminf(m, x); }
+__device__ __forceinline__ void keep_min(double& m, double x) {
+  // signed-integer order of the bits (sign-magnitude turned into two's complement)
+  const long long a = __double_as_longlong(x), b = __double_as_longlong(m);
+  const bool nan = (a & 0x7fffffffffffffffll) > 0x7ff0000000000000ll;
+  const long long ka = a < 0 ? a ^ 0x7fffffffffffffffll : a;
+  const long long kb = b < 0 ? b ^ 0x7fffffffffffffffll : b;
+  if (!nan && ka < kb) m = x;
+}
+
+__device__ __forceinline__ double wide(float x) { return widen(x); }
+__device__ __forceinline__ double wide(double x) { return x; }
+__device__ __forceinline__ bool same_bits(float x, float y) {
+  return __float_as_uint(x) == __float_as_uint(y);
+}
+__device__ __forceinline__ bool same_bits(double x, double y) {
+  return __double_as_longlong(x) == __double_as_longlong(y);
+}
+
+// |u| + c of a node (absolute rho, p)
+__device__ __forceinline__ double wave_speed(double r, double u, double v, double p,
+                                             double gamma) {
+  return sqrt(fma(u, u, v * v)) + sqrt(gamma * p / r);
 }
 
 template <typename T, bool COMP>
-__global__ void __launch_bounds__(RED_THREADS) k_inv_partial(RedArgs<T> a) {
-  double acc[RED_VALS];
-  for (int k = 0; k < RED_SUMS; ++k) acc[k] = 0.0;
-  acc[8] = 0.0;
-  acc[9] = INFINITY;
-  acc[10] = INFINITY;
+__global__ void __launch_bounds__(RED_THREADS) k_inv_partial(const __grid_constant__ RedArgs<T> a) {
+  __shared__ LogEntry tab[LOG_POINTS];
+  __shared__ double sh[RED_WARPS][RED_VALS];
+  fill_log_table(tab, threadIdx.x, RED_THREADS);
+  __syncthreads();
+  double acc[RED_SUMS] = {};
+  double smax = 0.0;
+  const float near_top = __uint_as_float(*a.top) * 0.9999995f;
+  T seen[4] = {};          // (rho, u, v, p) of the lane's last FP64 wave speed
+  T rmin = (T)INFINITY, pmin = (T)INFINITY;  // of the stored offsets
   const size_t N = (size_t)a.nx * a.ny;
-  const double sw[3] = {1.0 / 6.0, 4.0 / 6.0, 1.0 / 6.0};
-  for (size_t id = (size_t)blockIdx.x * blockDim.x + threadIdx.x; id < N;
-       id += (size_t)gridDim.x * blockDim.x) {
-    int i = (int)(id % a.nx), j = (int)(id / a.nx);
-    int ip = wrapi(i + 1, a.nx), jp = wrapi(j + 1, a.ny);
-    double ub[4];
+  for (size_t id = (size_t)blockIdx.x * RED_THREADS + threadIdx.x; id < N;
+       id += (size_t)gridDim.x * RED_THREADS) {
+    const int j = (int)(id / (unsigned)a.nx), i = (int)(id - (size_t)j * a.nx);
+    const int ip = i + 1 == a.nx ? 0 : i + 1, jp = j + 1 == a.ny ? 0 : j + 1;
+    // every load of the cell first
+    const T* const* const pl[4] = {a.st.pt[0], a.st.pt[1], a.st.pt[2], a.wc};
+    T w[4][4], av[4], lo[4];
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) w[n][k] = pl[n][k][id];
+#pragma unroll
     for (int k = 0; k < 4; ++k) {
-      ub[k] = (double)a.st.avg[k][id] + (COMP ? (double)a.st.lo[k][id] : 0.0);
-      ub[k] += k == 0 ? a.rho_ref : (k == 3 ? a.e_ref : 0.0);
+      av[k] = a.st.avg[k][id];
+      if (COMP) lo[k] = a.st.lo[k][id];
+    }
+    const size_t q10 = (size_t)j * a.nx + ip, q01 = (size_t)jp * a.nx + i,
+                 q11 = (size_t)jp * a.nx + ip;
+    const T v10 = a.st.pt[0][2][q10], u10 = a.st.pt[0][1][q10];
+    const T v11 = a.st.pt[0][2][q11], u11 = a.st.pt[0][1][q11];
+    const T v01 = a.st.pt[0][2][q01], u01 = a.st.pt[0][1][q01];
+    const T vev10 = a.st.pt[1][2][q10], ueh01 = a.st.pt[2][1][q01];
+    // averages
+    double ub[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      ub[k] = wide(av[k]);
+      if (COMP) ub[k] += wide(lo[k]);
+      if (sizeof(T) == 4 && k == 0) ub[k] += a.rho_ref;
+      if (sizeof(T) == 4 && k == 3) ub[k] += a.e_ref;
       acc[k] += ub[k];
     }
-    double ra = ub[0], ua = ub[1] / ra, va = ub[2] / ra;
-    double pa = (a.gamma - 1.0) * (ub[3] - 0.5 * ra * (ua * ua + va * va));
-    acc[5] += entropy_density(ra, pa, a.gamma);
-    acc[6] += 0.5 * (ub[1] * ub[1] + ub[2] * ub[2]) / ra;
+    const double ke = 0.5 * fma(ub[1], ub[1], ub[2] * ub[2]) / ub[0];
+    acc[5] += entropy_density(ub[0], (a.gamma - 1.0) * (ub[3] - ke), a.gamma, tab);
+    acc[6] += ke;
     // The Simpson entropy integral sums, over the cells, the nine nodes of each
     // with weights (1/6, 4/6, 1/6) x (1/6, 4/6, 1/6).  On the periodic grid every
     // vertex lies in four cells, every edge midpoint in two and every centre in
     // one, so the same total is each cell's own four nodes (vertex (i, j), edges
-    // (i, j+1/2) and (i+1/2, j), centre) with weights 1/9, 2/9, 2/9, 4/9: one
-    // entropy evaluation (two FP64 logarithms) per node instead of per
-    // cell-node pair.
-    auto ld = [&](const T* const* pl, size_t q, double* o) {
-      for (int k = 0; k < 4; ++k) o[k] = (double)pl[k][q];
-      o[0] += a.rho_ref;
-      o[3] += a.p_ref;
-    };
-    double wv[4], wev[4], weh[4], wcn[4];
-    ld(a.st.pt[0], id, wv);
-    ld(a.st.pt[1], id, wev);
-    ld(a.st.pt[2], id, weh);
-    ld(a.wc, id, wcn);
-    acc[4] += (entropy_density(wv[0], wv[3], a.gamma) +
-               2.0 * (entropy_density(wev[0], wev[3], a.gamma) +
-                      entropy_density(weh[0], weh[3], a.gamma)) +
-               4.0 * entropy_density(wcn[0], wcn[3], a.gamma)) /
-              9.0;
-    const double* own[4] = {wv, weh, wev, wcn};
+    // (i, j+1/2) and (i+1/2, j), centre) with weights 1/9, 2/9, 2/9, 4/9.
+    double H[4];
+    float sf[4];
+#pragma unroll
     for (int n = 0; n < 4; ++n) {
-      const double* o = own[n];
-      double s = sqrt(o[1] * o[1] + o[2] * o[2]) + sqrt(a.gamma * o[3] / o[0]);
-      acc[8] = fmax(acc[8], s);
-      acc[9] = fmin(acc[9], o[0]);
-      acc[10] = fmin(acc[10], o[3]);
+      const double r = sizeof(T) == 4 ? wide(w[n][0]) + a.rho_ref : wide(w[n][0]);
+      const double p = sizeof(T) == 4 ? wide(w[n][3]) + a.p_ref : wide(w[n][3]);
+      H[n] = entropy_density(r, p, a.gamma, tab);
+      keep_min(rmin, w[n][0]);
+      keep_min(pmin, w[n][3]);
+      sf[n] = wave_speed_f32(narrow_any(r), narrow_any(w[n][1]), narrow_any(w[n][2]),
+                             narrow_any(p), (float)a.gamma);
     }
+    // the wave speed in FP64 only at nodes whose FP32 value is within 5e-7 of the
+    // grid's largest (k_center found it)
+#pragma unroll 1
+    for (int n = 0; n < 4; ++n) {
+      const float sn = n == 0 ? sf[0] : n == 1 ? sf[1] : n == 2 ? sf[2] : sf[3];
+      if (!(sn >= near_top)) continue;
+      T q[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        q[k] = n == 0 ? w[0][k] : n == 1 ? w[1][k] : n == 2 ? w[2][k] : w[3][k];
+      if (same_bits(q[0], seen[0]) && same_bits(q[1], seen[1]) && same_bits(q[2], seen[2]) &&
+          same_bits(q[3], seen[3]))
+        continue;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) seen[k] = q[k];
+      const double rr = sizeof(T) == 4 ? wide(q[0]) + a.rho_ref : wide(q[0]);
+      const double pp = sizeof(T) == 4 ? wide(q[3]) + a.p_ref : wide(q[3]);
+      smax = fmax(smax, wave_speed(rr, wide(q[1]), wide(q[2]), pp, a.gamma));
+    }
+    acc[4] += fma(4.0, H[3], fma(2.0, H[1] + H[2], H[0]));
     // circulation around the cell: Simpson along its four edges (the right and
-    // top edges' nodes belong to the neighbouring cells)
-    const size_t q10 = (size_t)j * a.nx + ip, q01 = (size_t)jp * a.nx + i,
-                 q11 = (size_t)jp * a.nx + ip;
-    const double v10 = (double)a.st.pt[0][2][q10], u10 = (double)a.st.pt[0][1][q10];
-    const double v11 = (double)a.st.pt[0][2][q11], u11 = (double)a.st.pt[0][1][q11];
-    const double v01 = (double)a.st.pt[0][2][q01], u01 = (double)a.st.pt[0][1][q01];
-    const double vev10 = (double)a.st.pt[1][2][q10], ueh01 = (double)a.st.pt[2][1][q01];
-    const double vr = sw[0] * v10 + sw[1] * vev10 + sw[2] * v11;
-    const double vl = sw[0] * wv[2] + sw[1] * wev[2] + sw[2] * v01;
-    const double ut = sw[0] * u01 + sw[1] * ueh01 + sw[2] * u11;
-    const double ubt = sw[0] * wv[1] + sw[1] * weh[1] + sw[2] * u10;
-    acc[7] += a.h * (vr - vl) - a.h * (ut - ubt);
+    // top edges' nodes belong to the neighbouring cells), differences first
+    const double cv = fma(4.0, wide(vev10) - wide(w[1][2]),
+                          (wide(v10) - wide(w[0][2])) + (wide(v11) - wide(v01)));
+    const double cu = fma(4.0, wide(ueh01) - wide(w[2][1]),
+                          (wide(u01) - wide(w[0][1])) + (wide(u11) - wide(u10)));
+    acc[7] += cv - cu;
   }
-  // block reduction: warp shuffles, then one warp over the warp results
-  __shared__ double sh[RED_THREADS / 32][RED_VALS];
+  // block reduction: warp shuffles, then the warp results in order
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const double off = sizeof(T) == 4 ? 1.0 : 0.0;
+  double vals[RED_VALS];
+#pragma unroll
+  for (int k = 0; k < RED_SUMS; ++k) vals[k] = acc[k];
+  vals[8] = smax;
+  vals[9] = wide(rmin) + off * a.rho_ref;
+  vals[10] = wide(pmin) + off * a.p_ref;
+#pragma unroll
   for (int k = 0; k < RED_VALS; ++k) {
-    double v = acc[k];
+    double v = vals[k];
     for (int o = 16; o > 0; o >>= 1) {
       double t = __shfl_down_sync(0xffffffffu, v, o);
       v = (k < RED_SUMS) ? v + t : (k == 8 ? fmax(v, t) : fmin(v, t));
@@ -109,27 +215,43 @@ __global__ void __launch_bounds__(RED_THREADS) k_inv_partial(RedArgs<T> a) {
   if (threadIdx.x < RED_VALS) {
     int k = threadIdx.x;
     double v = sh[0][k];
-    for (int wi = 1; wi < RED_THREADS / 32; ++wi)
+    for (int wi = 1; wi < RED_WARPS; ++wi)
       v = (k < RED_SUMS) ? v + sh[wi][k] : (k == 8 ? fmax(v, sh[wi][k]) : fmin(v, sh[wi][k]));
-    a.partial[(size_t)blockIdx.x * RED_VALS + k] = v;
+    a.partial[(size_t)k * gridDim.x + blockIdx.x] = v;
   }
 }
 
-// one block of RED_VALS threads folds nblocks partials in index order
-__global__ void k_inv_final(const double* partial, int nblocks, double h, double* out) {
-  int k = threadIdx.x;
-  if (k >= RED_VALS) return;
-  double v = partial[k];
-  for (int b = 1; b < nblocks; ++b) {
-    double t = partial[(size_t)b * RED_VALS + k];
-    v = (k < RED_SUMS) ? v + t : (k == 8 ? fmax(v, t) : fmin(v, t));
-  }
-  double h2 = h * h;
+// One block of RED_VALS warps: warp k folds value k of the nblocks partials, each
+// lane its share in index order, then the lanes by shuffles; `out` is the host's
+// pinned memory, written through the device's mapping.
+__global__ void k_inv_final(const double* partial, int nblocks, double h, double* out,
+                            unsigned* top) {
+  if (threadIdx.x == 0) *top = 0u;  // for the next call
+  const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const double* pk = partial + (size_t)k * nblocks;
+  // (one branch per warp: selecting among sum, max and min inside the loop would
+  // issue all three on the FP64 unit, 20 us instead of 5)
+  auto fold = [&](double v, auto op) {
+#pragma unroll 8
+    for (int b = lane; b < nblocks; b += 32) v = op(v, pk[b]);
+    for (int o = 16; o > 0; o >>= 1) v = op(v, __shfl_down_sync(0xffffffffu, v, o));
+    return v;
+  };
+  double v;
+  if (k < RED_SUMS)
+    v = fold(0.0, [](double x, double y) { return x + y; });
+  else if (k == 8)
+    v = fold(0.0, [](double x, double y) { return fmax(x, y); });
+  else
+    v = fold(INFINITY, [](double x, double y) { return fmin(x, y); });
+  if (lane != 0) return;
   // output order follows AF_INV_*: mass, mx, my, E, entropy, entropy_avg, KE,
   // max speed, min rho, min p, vorticity
-  if (k < 7) out[k] = h2 * v;
-  else if (k == 7) out[10] = v;
+  const double h2 = h * h;
+  if (k < 7) out[k] = (k == 4 ? h2 / 9.0 : h2) * v;
+  else if (k == 7) out[10] = h / 6.0 * v;
   else out[k - 1] = v;
+  __threadfence_system();
 }
 
 }  // namespace af
