@@ -428,15 +428,27 @@ af_status import_enqueue(af_handle* h, const af_state_f64* in, af_memory where,
   if (where == AF_HOST) {
     // pinned planes are read in place by the import kernel, pageable ones are
     // copied to the staging buffer first
+    int mapped = 0;
     for (int p = 0; p < 16; ++p) {
       src.p[p] = (const double*)mapped_host_plane(h, plane_in(in, p));
-      if (src.p[p]) continue;
-      af_status st = ensure_staging(h);
+      mapped += src.p[p] != nullptr;
+    }
+    if (mapped < 16) {
+      const af_status st = ensure_staging(h);
       if (st != AF_OK) return st;
-      if (cudaMemcpyAsync(h->staging + (size_t)p * h->N, plane_in(in, p), sizeof(double) * h->N,
-                          cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
-        return cuda_fail(h);
-      src.p[p] = h->staging + (size_t)p * h->N;
+      const af_state_f64 staged = planes_at(h->staging, h->N);
+      if (mapped == 0) {
+        if (copy_planes(&staged, in, h->N, cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
+          return cuda_fail(h);
+      }
+      for (int p = 0; p < 16; ++p) {
+        if (src.p[p]) continue;
+        src.p[p] = plane_in(&staged, p);
+        if (mapped > 0 &&
+            cudaMemcpyAsync((void*)src.p[p], plane_in(in, p), sizeof(double) * h->N,
+                            cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
+          return cuda_fail(h);
+      }
     }
   } else {
     for (int p = 0; p < 16; ++p) src.p[p] = plane_in(in, p);
@@ -688,10 +700,13 @@ af_status af_init(af_handle** out, const af_grid* g, double gamma, const af_stat
     const char* lw = getenv("AF_TEST_LATE_WAIT");
     h->late_once = (lw && lw[0] == '1') ? 1 : 0;
   }
-  // 2 x 20 state planes + 44 scratch planes, each padded to 256 bytes
+  // 2 x 20 state planes + 44 scratch planes, each padded to 256 bytes, then the
+  // reduction's partials and the two device words: one allocation per handle
   size_t plane = (h->N * h->esize + 255) & ~(size_t)255;
-  size_t nplanes = 2 * 20 + 44;
-  if (cudaMalloc(&h->arena, plane * nplanes) != cudaSuccess) {
+  const size_t nplanes = 2 * 20 + 44;
+  h->red_blocks = 152 * 8;
+  const size_t red = sizeof(double) * RED_VALS * h->red_blocks;
+  if (cudaMalloc(&h->arena, plane * nplanes + red + 256) != cudaSuccess) {
     delete h;
     return AF_ERR_ALLOC;
   }
@@ -699,19 +714,21 @@ af_status af_init(af_handle** out, const af_grid* g, double gamma, const af_stat
   for (int s = 0; s < 2; ++s)
     for (int p = 0; p < 20; ++p) h->state[s][p] = base + plane * (size_t)(20 * s + p);
   for (int p = 0; p < 44; ++p) h->scratch[p] = base + plane * (size_t)(40 + p);
-  h->red_blocks = 152 * 8;
-  bool ok = cudaMalloc(&h->d_flags, 2 * sizeof(unsigned)) == cudaSuccess &&
-            cudaMemsetAsync(h->d_flags, 0, 2 * sizeof(unsigned), h->stream) == cudaSuccess &&
-            cudaMallocHost(&h->h_flags, sizeof(unsigned)) == cudaSuccess &&
-            cudaHostGetDevicePointer((void**)&h->h_flags_dev, h->h_flags, 0) == cudaSuccess &&
-            cudaMalloc(&h->d_red, sizeof(double) * RED_VALS * h->red_blocks) == cudaSuccess &&
-            cudaMallocHost(&h->h_red, sizeof(double) * AF_NINV) == cudaSuccess &&
-            cudaHostGetDevicePointer((void**)&h->h_red_dev, h->h_red, 0) == cudaSuccess;
+  h->d_red = (double*)(base + plane * nplanes);
+  h->d_flags = (unsigned*)(base + plane * nplanes + red);
+  h->d_top = h->d_flags + 1;
+  // pinned: the reduction's result, then the error word's mirror
+  const bool ok =
+      cudaMallocHost(&h->h_red, sizeof(double) * (AF_NINV + 1)) == cudaSuccess &&
+      cudaHostGetDevicePointer((void**)&h->h_red_dev, h->h_red, 0) == cudaSuccess &&
+      cudaMemsetAsync(h->d_flags, 0, 2 * sizeof(unsigned), h->stream) == cudaSuccess;
   if (!ok) {
     af_destroy(h);
     return AF_ERR_ALLOC;
   }
-  h->d_top = h->d_flags + 1;
+  h->h_flags = (unsigned*)(h->h_red + AF_NINV);
+  h->h_flags_dev = (unsigned*)(h->h_red_dev + AF_NINV);
+  *h->h_flags = 0;
   if (prec != AF_FP64 && h->pipe_ctas > 0) {
     // tensor maps of both state buffers for the pipelined kernel; AF_TMA=0 (or a
     // driver without the encoder) stages every tile by cp.async instead
@@ -746,9 +763,8 @@ af_status af_init(af_handle** out, const af_grid* g, double gamma, const af_stat
     }
   }
   if (prec == AF_FP32_COMP || prec == AF_FP32) {
-    // zero the lo planes once (unused in AF_FP32)
-    for (int s = 0; s < 2; ++s)
-      for (int k = 16; k < 20; ++k) cudaMemsetAsync(h->state[s][k], 0, plane, h->stream);
+    // zero the lo planes once (unused in AF_FP32; consecutive in the arena)
+    for (int s = 0; s < 2; ++s) cudaMemsetAsync(h->state[s][16], 0, 4 * plane, h->stream);
   }
   // storage offsets: the initial vertex state at (0,0) (FP32 modes only)
   if (prec != AF_FP64) {
@@ -821,6 +837,7 @@ af_status af_get_state(af_handle* h, const af_state_f64* out, af_memory where) {
   if (wait_outgoing(h) != AF_OK) return AF_ERR_CUDA;
   F64Out dst;
   bool copy_back[16] = {};
+  int copies = 0;
   if (where == AF_HOST) {
     // pinned planes are written in place by the export kernel, pageable ones
     // through the staging buffer
@@ -831,17 +848,24 @@ af_status af_get_state(af_handle* h, const af_state_f64* out, af_memory where) {
       if (st != AF_OK) return st;
       dst.p[p] = h->staging + (size_t)p * h->N;
       copy_back[p] = true;
+      ++copies;
     }
   } else {
     for (int p = 0; p < 16; ++p) dst.p[p] = (double*)plane_in(out, p);
   }
   af_status est = export_enqueue(h, dst);
   if (est != AF_OK) return est;
-  for (int p = 0; p < 16; ++p)
-    if (copy_back[p] &&
-        cudaMemcpyAsync((void*)plane_in(out, p), dst.p[p], sizeof(double) * h->N,
-                        cudaMemcpyDeviceToHost, h->stream) != cudaSuccess)
+  if (copies == 16) {
+    const af_state_f64 staged = planes_at(h->staging, h->N);
+    if (copy_planes(out, &staged, h->N, cudaMemcpyDeviceToHost, h->stream) != cudaSuccess)
       return cuda_fail(h);
+  } else {
+    for (int p = 0; p < 16; ++p)
+      if (copy_back[p] &&
+          cudaMemcpyAsync((void*)plane_in(out, p), dst.p[p], sizeof(double) * h->N,
+                          cudaMemcpyDeviceToHost, h->stream) != cudaSuccess)
+        return cuda_fail(h);
+  }
   return af_sync(h);
 }
 
@@ -1060,9 +1084,6 @@ void af_destroy(af_handle* h) {
   }
   if (h->arena) cudaFree(h->arena);
   if (h->staging) cudaFree(h->staging);
-  if (h->d_flags) cudaFree(h->d_flags);
-  if (h->h_flags) cudaFreeHost(h->h_flags);
-  if (h->d_red) cudaFree(h->d_red);
   if (h->adj_arena) cudaFree(h->adj_arena);
   if (h->xstaging) cudaFree(h->xstaging);
   if (h->astage[0]) {
@@ -1141,14 +1162,13 @@ af_status batch_snapshot(af_batch* b, bool restore) {
   char* p = (char*)b->snapshot;
   for (int k = 0; k < b->n; ++k) {
     af_handle* h = b->h[k];
-    const size_t bytes = state_plane_bytes(h);
-    for (int q = 0; q < 20; ++q) {
-      void* live = h->state[h->cur][q];
-      if (cudaMemcpyAsync(restore ? live : (void*)p, restore ? (void*)p : live, bytes,
-                          cudaMemcpyDeviceToDevice, b->stream) != cudaSuccess)
-        return AF_ERR_CUDA;
-      p += bytes;
-    }
+    // (the twenty planes of a state are consecutive in the handle's arena)
+    const size_t bytes = 20 * state_plane_bytes(h);
+    void* live = h->state[h->cur][0];
+    if (cudaMemcpyAsync(restore ? live : (void*)p, restore ? (void*)p : live, bytes,
+                        cudaMemcpyDeviceToDevice, b->stream) != cudaSuccess)
+      return AF_ERR_CUDA;
+    p += bytes;
   }
   return AF_OK;
 }
