@@ -247,8 +247,8 @@ af_status af_step_noalloc(const af_grid *g, double gamma, double dt, af_variant 
  * over a table of the tiles of all grids, and the launches of an af_batch_step
  * call are captured once in a CUDA graph (re-captured when n_steps changes).
  * Geometries (AF_BATCH_GEOMS): 0, 1, 2 launch one CTA per tile of 32x32,
- * 24x16 or 16x16 cells; 3 launches persistent CTAs (one per SM) that step
- * through the 32x32 tiles of all grids, staging each next tile (tensor copies
+ * 32x16 (24x16 where that makes fewer waves) or 16x16 cells; 3 launches
+ * persistent CTAs (one per SM) that step through the 32x32 tiles of all grids, staging each next tile (tensor copies
  * inside a grid, cp.async on its periodic boundary) while the current one
  * finishes -- offered when every grid has nx a multiple of 4, nx >= 40 and
  * ny >= 38.  The first af_batch_step times the geometries on the actual

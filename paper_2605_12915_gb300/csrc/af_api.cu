@@ -1133,6 +1133,7 @@ struct af_batch {
   int own_stream;           // the batch created its stream (the legacy stream cannot be captured)
   int pipe_ok;              // every grid meets the persistent kernel's staging conditions
   int pipe_ctas;            // its CTAs
+  int use_24x16;            // geometry 1 is 24 x 16 tiles (batch_prefers_24x16)
   TileMaps* d_maps[2];      // device, one per grid and parity (null: cp.async staging only)
 };
 
@@ -1141,10 +1142,11 @@ namespace {
 af_status batch_launch(af_batch* b, int geom, int parity) {
   const StepArgs<float>* args = b->d_args + (size_t)parity * b->n;
   if (BATCH_GEOMS[geom].pipe && !b->pipe_ok) return AF_ERR_ARG;
+  const int kind = geom == 1 && b->use_24x16 ? BATCH_24x16 : geom;
   cudaError_t e = b->prec == AF_FP32_COMP
-                      ? launch_batch<true>(geom, b->stream, args, b->d_tiles[geom], b->ntiles[geom],
+                      ? launch_batch<true>(kind, b->stream, args, b->d_tiles[geom], b->ntiles[geom],
                                            b->d_maps[parity], b->pipe_ctas)
-                      : launch_batch<false>(geom, b->stream, args, b->d_tiles[geom],
+                      : launch_batch<false>(kind, b->stream, args, b->d_tiles[geom],
                                             b->ntiles[geom], b->d_maps[parity], b->pipe_ctas);
   return e == cudaSuccess ? AF_OK : AF_ERR_CUDA;
 }
@@ -1261,11 +1263,20 @@ af_status af_batch_init(af_batch** out, int32_t n, const af_grid* grids, double 
       order[y - 1] = t;
     }
   bool ok = true;
-  for (int g = 0; g < N_BATCH_GEOMS && ok; ++g) {
-    const int tx = BATCH_GEOMS[g].tx, ty = BATCH_GEOMS[g].ty;
+  auto count = [&](const BatchGeometry& q) {
     size_t cnt = 0;
     for (int k = 0; k < n; ++k)
-      cnt += (size_t)((b->h[k]->nx + tx - 1) / tx) * ((b->h[k]->ny + ty - 1) / ty);
+      cnt += (size_t)((b->h[k]->nx + q.tx - 1) / q.tx) * ((b->h[k]->ny + q.ty - 1) / q.ty);
+    return cnt;
+  };
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->h[0]->device);
+  b->use_24x16 = sms > 0 && batch_prefers_24x16((int64_t)count(BATCH_GEOMS[BATCH_24x16]),
+                                                (int64_t)count(BATCH_GEOMS[1]), sms);
+  for (int g = 0; g < N_BATCH_GEOMS && ok; ++g) {
+    const BatchGeometry& q = BATCH_GEOMS[g == 1 && b->use_24x16 ? BATCH_24x16 : g];
+    const int tx = q.tx, ty = q.ty;
+    const size_t cnt = count(q);
     int4* tt = new int4[cnt];
     size_t c = 0;
     for (int o = 0; o < n; ++o) {

@@ -999,6 +999,7 @@ __global__ void __launch_bounds__(NT, MINB)
 template <int TX, int TY, int NT, int MINB, bool COMP>
 __global__ void __launch_bounds__(NT, MINB)
     k_fused_step_batch(const StepArgs<float>* __restrict__ args, const int4* __restrict__ tiles) {
+  pdl_wait();
   const int4 t = tiles[blockIdx.x];
   PipeCtx none = {nullptr, 0u, 0u};
   fused_tile<TX, TY, NT, COMP, false>(args[t.x], none, t.y, t.z, -1, -1, false);
@@ -1027,6 +1028,7 @@ __global__ void __launch_bounds__(NT, MINB)
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(pc.bar) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  pdl_wait();
   __syncthreads();
   int t = blockIdx.x;
   if (t < ntiles) {

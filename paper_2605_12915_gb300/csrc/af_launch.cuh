@@ -158,16 +158,25 @@ inline cudaError_t launch_fused_step(cudaStream_t s, const StepArgs<float>& a, b
   return launch_step_tiles<FUSED_TX, FUSED_TY, FUSED_NT, AF_FUSED_MINB, COMP>(s, a);
 }
 
-// Tile geometries available to the batched launch (the autotuner picks one):
-// one CTA per tile of 32x32, 24x16 or 16x16 cells, or (pipe) persistent CTAs
-// stepping through the 32x32 tiles with the next tile staged asynchronously.
+// Tile geometries available to the batched launch (the autotuner picks one): one
+// CTA per tile of 32x32, 32x16 (or 24x16, two per SM) or 16x16 cells, or (pipe)
+// persistent CTAs stepping through the 32x32 tiles with the next tile staged
+// asynchronously.
 struct BatchGeometry {
   int tx, ty, nt, minb, pipe;
 };
-constexpr int N_BATCH_GEOMS = 4;
-constexpr BatchGeometry BATCH_GEOMS[N_BATCH_GEOMS] = {
-    {32, 32, 512, 1, 0}, {24, 16, 256, 2, 0}, {16, 16, 256, 3, 0},
-    {FUSED_TX, FUSED_TY, FUSED_NT, AF_FUSED_MINB, 1}};
+constexpr int N_BATCH_GEOMS = 4, BATCH_24x16 = N_BATCH_GEOMS;
+constexpr BatchGeometry BATCH_GEOMS[N_BATCH_GEOMS + 1] = {
+    {32, 32, 512, 1, 0}, {32, 16, 512, 1, 0}, {16, 16, 512, 1, 0},
+    {FUSED_TX, FUSED_TY, FUSED_NT, AF_FUSED_MINB, 1}, {24, 16, 256, 2, 0}};
+
+// Whether geometry 1 stands for 24x16 tiles (two CTAs per SM) instead of 32x16 ones,
+// given the ensemble's tile counts in both: the smaller of waves x measured time of
+// a wave (26 and 17 us).  Eight grids of 64^2 and 128^2 (240 and 160 tiles) take
+// 26.6 and 33.1 us a step, eight of 64^2 to 256^2 (624 and 448 tiles) 62.8 and 49.5.
+inline bool batch_prefers_24x16(int64_t n24, int64_t n32, int sms) {
+  return (float)((n24 + 2 * sms - 1) / (2 * sms)) * 26.f < (float)((n32 + sms - 1) / sms) * 17.f;
+}
 
 template <int TX, int TY, int NT, int MINB, bool COMP>
 inline cudaError_t launch_batch_geom(cudaStream_t s, const StepArgs<float>* args,
@@ -176,8 +185,7 @@ inline cudaError_t launch_batch_geom(cudaStream_t s, const StepArgs<float>* args
   constexpr auto kern = k_fused_step_batch<TX, TY, NT, MINB, COMP>;
   const cudaError_t e = allow_smem<kern>(G::SMEM);
   if (e != cudaSuccess) return e;
-  kern<<<ntiles, NT, G::SMEM, s>>>(args, tiles);
-  return cudaGetLastError();
+  return launch_dependent(kern, dim3(ntiles), NT, G::SMEM, s, args, tiles);
 }
 
 // The persistent form: `ctas` CTAs over the tile table; maps (device, one
@@ -190,8 +198,8 @@ inline cudaError_t launch_batch_pipe(cudaStream_t s, const StepArgs<float>* args
   constexpr auto kern = k_fused_step_batch_pipe<FUSED_TX, FUSED_TY, FUSED_NT, AF_FUSED_MINB, COMP>;
   const cudaError_t e = allow_smem<kern>(G::SMEM_PIPE);
   if (e != cudaSuccess) return e;
-  kern<<<ntiles < ctas ? ntiles : ctas, FUSED_NT, G::SMEM_PIPE, s>>>(args, tiles, ntiles, maps);
-  return cudaGetLastError();
+  return launch_dependent(kern, dim3(ntiles < ctas ? ntiles : ctas), FUSED_NT, G::SMEM_PIPE, s,
+                          args, tiles, ntiles, maps);
 }
 
 template <bool COMP>
@@ -199,8 +207,9 @@ inline cudaError_t launch_batch(int geom, cudaStream_t s, const StepArgs<float>*
                                 const int4* tiles, int ntiles, const TileMaps* maps, int ctas) {
   switch (geom) {
     case 0: return launch_batch_geom<32, 32, 512, 1, COMP>(s, args, tiles, ntiles);
-    case 1: return launch_batch_geom<24, 16, 256, 2, COMP>(s, args, tiles, ntiles);
-    case 2: return launch_batch_geom<16, 16, 256, 3, COMP>(s, args, tiles, ntiles);
+    case 1: return launch_batch_geom<32, 16, 512, 1, COMP>(s, args, tiles, ntiles);
+    case 2: return launch_batch_geom<16, 16, 512, 1, COMP>(s, args, tiles, ntiles);
+    case BATCH_24x16: return launch_batch_geom<24, 16, 256, 2, COMP>(s, args, tiles, ntiles);
     default: return launch_batch_pipe<COMP>(s, args, tiles, ntiles, maps, ctas);
   }
 }

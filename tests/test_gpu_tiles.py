@@ -56,3 +56,15 @@ def test_captured_steps_equal_launched_steps(shape):
     torch.cuda.synchronize()
     assert np.array_equal(s.state(), want)
     s.close()
+
+
+def test_batch_on_24x16_tiles_is_bitwise_the_lone_steps(monkeypatch):
+    """Four grids of 160 x 157 cells: 200 tiles of 32 x 16 (two waves) against 280 of
+    24 x 16 (one wave of two per SM), so geometry 1 is the latter."""
+    probs = [I.random_smooth(160, 157, seed=k, amp=0.05) for k in range(4)]
+    monkeypatch.setenv("AF_BATCH_GEOM", "1")
+    b = af.Batch(probs, precision="fp32_comp")
+    b.step([p.dt for p in probs], 4)
+    for k, p in enumerate(probs):
+        assert np.array_equal(b.state(k), _run(p, "fp32_comp", "tai", 4)), k
+    b.close()
