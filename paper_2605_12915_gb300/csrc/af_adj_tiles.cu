@@ -5,7 +5,7 @@
 namespace af {
 
 template <bool COMP>
-cudaError_t launch_adj_small(int geom, cudaStream_t s, const StepArgs<float>& a,
+cudaError_t launch_adj_tiles_geom(int geom, cudaStream_t s, const StepArgs<float>& a,
                              const AdjView<float>& v) {
   switch (geom) {
     case ADJ_8x8: return launch_adj_tiles<8, 8, 256, 1, COMP>(s, a, v);
@@ -17,9 +17,9 @@ cudaError_t launch_adj_small(int geom, cudaStream_t s, const StepArgs<float>& a,
   return cudaErrorNotSupported;
 }
 
-template cudaError_t launch_adj_small<false>(int, cudaStream_t, const StepArgs<float>&,
+template cudaError_t launch_adj_tiles_geom<false>(int, cudaStream_t, const StepArgs<float>&,
                                              const AdjView<float>&);
-template cudaError_t launch_adj_small<true>(int, cudaStream_t, const StepArgs<float>&,
+template cudaError_t launch_adj_tiles_geom<true>(int, cudaStream_t, const StepArgs<float>&,
                                             const AdjView<float>&);
 
 }  // namespace af

@@ -876,44 +876,6 @@ __device__ __forceinline__ void tile_reverse(const StepArgs<float>& a, const Adj
   }
 }
 
-// Persistent kernel of the fused reverse sweep: the pipelined step's tile loop
-// (k_fused_step_pipe) with fused_tile<..., ADJ> and tile_reverse per tile; the
-// next tile's input is staged once the reverse sweep is done with D.
-template <int TX, int TY, int NT, int MINB, bool COMP>
-__global__ void __launch_bounds__(NT, MINB)
-    k_fused_adj_pipe(const __grid_constant__ StepArgs<float> a, const __grid_constant__ TileMaps tm,
-                     int use_tma, const __grid_constant__ AdjView<float> v) {
-  using G = FusedGeom<TX, TY>;
-  extern __shared__ __align__(16) float4 smem4[];
-  float* S = reinterpret_cast<float*>(smem4 + 4 * G::WPL);
-  PipeCtx pc;
-  pc.tm = (use_tma && G::W_BYTES % 128 == 0 && (smem_addr(smem4) & 127u) == 0) ? &tm : nullptr;
-  pc.bar = smem_addr(reinterpret_cast<char*>(smem4) + G::SMEM);
-  pc.phase = 0;
-  pc.late = 0;
-  if (threadIdx.x == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(pc.bar) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  pdl_wait();
-  __syncthreads();
-  const int tcols = (a.nx + TX - 1) / TX, ntiles = tcols * ((a.ny + TY - 1) / TY);
-  int tile = blockIdx.x;
-  if (tile < ntiles)
-    issue_tile_async<TX, TY, NT, COMP>(a, pc, (tile % tcols) * TX, (tile / tcols) * TY, S);
-  for (; tile < ntiles; tile += gridDim.x) {
-    const int nxt = tile + gridDim.x;
-    const int pi0 = nxt < ntiles ? (nxt % tcols) * TX : -1, pj0 = (nxt / tcols) * TY;
-    const int i0 = (tile % tcols) * TX, j0 = (tile / tcols) * TY;
-    if (!fused_tile<TX, TY, NT, COMP, true, false, true>(a, pc, i0, j0, pi0, pj0,
-                                                         a.prefetch_wave > 0 && !pc.tm))
-      break;
-    tile_reverse<TX, TY, NT>(a, v, smem4, S, i0, j0);
-    __syncthreads();  // W and D are dead from here
-    if (pi0 >= 0) issue_tile_async<TX, TY, NT, COMP>(a, pc, pi0, pj0, S);
-  }
-}
-
 // The fused reverse sweep, one CTA per tile of TX x TY cells (any grid).
 template <int TX, int TY, int NT, int MINB, bool COMP>
 __global__ void __launch_bounds__(NT, MINB)
@@ -921,7 +883,7 @@ __global__ void __launch_bounds__(NT, MINB)
   using G = FusedGeom<TX, TY>;
   extern __shared__ __align__(16) float4 smem4[];
   pdl_wait();
-  PipeCtx none = {nullptr, 0u, 0u};
+  PipeCtx none = {nullptr, 0u, 0u, 0, 0u};
   const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY;
   fused_tile<TX, TY, NT, COMP, false, false, true>(a, none, i0, j0, -1, -1, false);
   tile_reverse<TX, TY, NT>(a, v, smem4, reinterpret_cast<const float*>(smem4 + 4 * G::WPL), i0,
@@ -943,27 +905,28 @@ inline cudaError_t launch_adj_tiles(cudaStream_t s, const StepArgs<float>& a,
 // the least (waves x measured time of one wave, FP32_COMP, GB300).  Two CTAs of
 // 256 threads share an SM on 32 x 8 tiles: one recomputes its step (FP32 issue)
 // while the other waits on its scatter, which makes up for the larger halo at
-// every size (one CTA of 32 x 16 tiles 840, the pipelined 32 x 32 tiles 804, 786 us
-// per adjoint step at 1024^2); the pipelined sweep is as fast on the largest grids
-// (2048^2: 2.95 against 2.99 ms).  Adjoint step, pipelined 32 x 32 tiles -> chosen:
-// 64^2 116 -> 49 us, 128^2 118 -> 54, 192^2 119 -> 66, 256^2 123 -> 84; 1021 x 1024,
-// which the pipelined sweep does not take, 1.69 (per stage) -> 0.81 ms.
-enum { ADJ_8x8, ADJ_16x8, ADJ_16x16, ADJ_32x8, ADJ_32x24, ADJ_PIPE, N_ADJ_GEOMS };
+// every size (adjoint step at 1024^2: one CTA of 32 x 16 tiles 840 us, persistent
+// pipelined 32 x 32 tiles 804, this 777; at 2048^2 2.94 ms against 2.97 pipelined,
+// 3.17 before).  Adjoint step, 32 x 32 tiles -> chosen: 64^2 116 -> 46 us, 128^2
+// 118 -> 54, 192^2 119 -> 66, 256^2 123 -> 79; 1021 x 1024, which had no fused sweep,
+// 1.69 -> 0.79 ms.
+enum { ADJ_8x8, ADJ_16x8, ADJ_16x16, ADJ_32x8, ADJ_32x24, N_ADJ_GEOMS };
 struct AdjGeometry {
   int tx, ty;
   int per_sm;      // resident CTAs per SM
   float us, fill;  // time of one wave, and once per sweep
 };
-constexpr AdjGeometry ADJ_GEOMS[N_ADJ_GEOMS] = {
-    {8, 8, 1, 15.f, 0.f},     {16, 8, 1, 18.f, 0.f},  {16, 16, 1, 30.f, 0.f},
-    {32, 8, 2, 34.6f, 12.f},  {32, 24, 1, 72.f, 0.f}, {FUSED_TX, FUSED_TY, 1, 68.5f, 20.f}};
+constexpr AdjGeometry ADJ_GEOMS[N_ADJ_GEOMS] = {{8, 8, 1, 15.f, 0.f},
+                                                {16, 8, 1, 18.f, 0.f},
+                                                {16, 16, 1, 30.f, 0.f},
+                                                {32, 8, 2, 34.6f, 12.f},
+                                                {32, 24, 1, 72.f, 0.f}};
 
 inline int choose_adj_geometry(const StepArgs<float>& a, int sms) {
   int best = ADJ_32x8;
   float best_us = 1e30f;
   for (int g = 0; g < N_ADJ_GEOMS; ++g) {
     const AdjGeometry& q = ADJ_GEOMS[g];
-    if (g == ADJ_PIPE && !pipe_eligible(a)) continue;
     const int64_t tiles = (int64_t)((a.nx + q.tx - 1) / q.tx) * ((a.ny + q.ty - 1) / q.ty);
     const int64_t wave = (int64_t)sms * q.per_sm;
     const float us = (float)((tiles + wave - 1) / wave) * q.us + q.fill;
@@ -977,22 +940,8 @@ inline int choose_adj_geometry(const StepArgs<float>& a, int sms) {
 
 // The fused reverse sweep on one CTA per tile (af_adj_tiles.cu).
 template <bool COMP>
-cudaError_t launch_adj_small(int geom, cudaStream_t s, const StepArgs<float>& a,
+cudaError_t launch_adj_tiles_geom(int geom, cudaStream_t s, const StepArgs<float>& a,
                              const AdjView<float>& v);
-
-// The persistent pipelined sweep on `ctas` CTAs (grids it accepts).
-template <bool COMP>
-inline cudaError_t launch_adj_pipe(cudaStream_t s, const StepArgs<float>& a, int ctas,
-                                   const TileMaps* maps, const AdjView<float>& v) {
-  using G = FusedGeom<FUSED_TX, FUSED_TY>;
-  constexpr auto kern = k_fused_adj_pipe<FUSED_TX, FUSED_TY, FUSED_NT, AF_FUSED_MINB, COMP>;
-  const cudaError_t e = allow_smem<kern>(G::SMEM_PIPE);
-  if (e != cudaSuccess) return e;
-  static TileMaps none;
-  const int ntiles = ((a.nx + FUSED_TX - 1) / FUSED_TX) * ((a.ny + FUSED_TY - 1) / FUSED_TY);
-  return launch_dependent(kern, dim3(ntiles < ctas ? ntiles : ctas), FUSED_NT, G::SMEM_PIPE, s, a,
-                          maps ? *maps : none, maps ? 1 : 0, v);
-}
 
 // lambda^n out: the averages' planes and the point families' node records into
 // sixteen FP64 planes

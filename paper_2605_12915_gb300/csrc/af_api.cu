@@ -596,11 +596,7 @@ af_status adjoint_impl(af_handle* h, double dt, const af_state_f64* lin, const a
     const bool pipe = h->pipe_ctas > 0 && pipe_eligible(f);
     fused = h->fused && h->pipe_ctas > 0 && !(fz && fz[0] == '0');
     if (fused) {
-      // (geom < 0: an explicit AF_PIPE, on the pipelined kernel's tiles)
-      const int g = h->geom >= 0 ? choose_adj_geometry(f, h->pipe_ctas)
-                                 : (pipe ? ADJ_PIPE : ADJ_32x8);
-      e = g == ADJ_PIPE ? launch_adj_pipe<COMP>(s, f, h->pipe_ctas, maps, v)
-                        : launch_adj_small<COMP>(g, s, f, v);
+      e = launch_adj_tiles_geom<COMP>(choose_adj_geometry(f, h->pipe_ctas), s, f, v);
     } else if (h->fused && pipe) {
       e = launch_fused_step<COMP, true>(s, f, true, h->pipe_ctas, maps);
     } else {

@@ -15,8 +15,8 @@
 // cp.async on the periodic boundary), so phase 0 only waits for them and
 // converts them into W.  Phase 3 evaluates the two-Picard foot and the
 // transported (or additive) point update of the points of cells
-// [i0, i0+TX] x [j0, j0+TY] for both durations; the half-step values never
-// leave the SM.  Phase 4 forms the space-time Simpson edge fluxes and updates
+// [i0, i0+TX] x [j0, j0+TY] for both durations together; the results wait in tensor
+// memory until D is dead, and the half-step values never leave the SM.  Phase 4 forms the space-time Simpson edge fluxes and updates
 // the owned cell averages.  Two variants serve the adjoint: one also stores the
 // intermediates it linearises about (centres, increments, half-step points),
 // the other stops after phase 3 with D still in shared memory, for the reverse
@@ -30,6 +30,8 @@
 #pragma once
 
 #include <cuda.h>  // CUtensorMap (the maps are encoded on the host)
+
+#include <type_traits>
 
 #include "af_common.cuh"
 #include "af_ref_kernels.cuh"
@@ -72,7 +74,7 @@ struct FusedGeom {
   // (plane stride SPL rounded up to 128 bytes for the tensor copies)
   static constexpr int SW = TX + 8, SPL = (CH * SW + 31) / 32 * 32;
   static constexpr bool STAGE_FITS = 20 * SPL * sizeof(float) <= 2 * DS_BYTES;
-  static constexpr size_t SMEM_PIPE = SMEM + 16;  // + the staging mbarrier
+  static constexpr size_t SMEM_PIPE = SMEM + 16;  // + the staging mbarrier, tensor memory base
   static_assert(4 * NE * sizeof(float) <= W_BYTES, "fluxes alias W");
   static_assert(3 * PPL * sizeof(float4) <= DS_BYTES, "points of one duration alias its increments");
   static_assert(8 * WPL * sizeof(float) <= 2 * DS_BYTES, "averages wait in the D region");
@@ -339,6 +341,7 @@ struct PipeCtx {
   unsigned bar;        // shared address of the staging mbarrier
   unsigned phase;      // tensor stagings completed so far
   int late;            // testing only: the next wait for a staged tile reports a timeout
+  unsigned tm_base;    // tensor memory of this CTA (tm_alloc)
 };
 
 __device__ __forceinline__ unsigned smem_addr(const void* p) {
@@ -371,6 +374,59 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned bar, unsigned parity,
 template <int TX, int TY>
 __device__ __forceinline__ bool box_inside(int nx, int ny, int i0, int j0) {
   return i0 >= 4 && j0 >= 2 && i0 + TX + 4 <= nx && j0 + TY + 4 <= ny;
+}
+
+// ---- tensor memory as a parking place -------------------------------------------
+// The point pass parks its results (a float4 per point and duration) in the SM's
+// tensor memory until the increments they will overwrite are dead: 256 KB that
+// nothing else uses here, reached a warp at a time (its own 32 lanes, 32-bit columns;
+// warps w and w + 4 share lanes).  A CTA allocates tm_cols() of the 512 columns, 0
+// where each thread has one point at most and keeps it in registers.
+template <int TX, int TY, int NT>
+__host__ __device__ constexpr int tm_cols() {
+  const int per = (3 * (TX + 1) * (TY + 1) + NT - 1) / NT, need = (NT / 128) * 8 * per;
+  int c = 32;
+  while (c < need) c *= 2;
+  return per > 1 ? c : 0;
+}
+__device__ __forceinline__ void tm_store(unsigned addr, const float4& v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr),
+               "r"(__float_as_uint(v.x)), "r"(__float_as_uint(v.y)), "r"(__float_as_uint(v.z)),
+               "r"(__float_as_uint(v.w))
+               : "memory");
+}
+__device__ __forceinline__ float4 tm_load(unsigned addr) {
+  unsigned x, y, z, w;
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(x), "=r"(y), "=r"(z), "=r"(w)
+               : "r"(addr)
+               : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  return make_float4(__uint_as_float(x), __uint_as_float(y), __uint_as_float(z),
+                     __uint_as_float(w));
+}
+// Allocation and release by warp 0; `slot`: a shared word for the base address, which
+// every thread returns after the barrier inside.  (No kernel here holds more than half
+// of the columns, so a CTA of the next kernel can allocate while this one drains.)
+template <int COLS>
+__device__ __forceinline__ unsigned tm_alloc(unsigned* slot) {
+  if constexpr (COLS == 0) return 0u;
+  if (threadIdx.x < 32) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_addr(slot)),
+                 "n"(COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  __syncthreads();
+  return *(volatile unsigned*)slot;
+}
+template <int COLS>
+__device__ __forceinline__ void tm_free(unsigned base) {
+  if constexpr (COLS == 0) return;
+  __syncthreads();
+  if (threadIdx.x < 32)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "n"(COLS));
 }
 
 // Starts the asynchronous copy of the raw input of tile (i0, j0) into the
@@ -685,120 +741,256 @@ __device__ __forceinline__ bool fused_tile(const StepArgs<float>& a, PipeCtx& pc
   __syncthreads();
 
   // ---- phase 3: point updates of cells [i0, i0+TX] x [j0, j0+TY] -------------
-  // duration by duration; the points of duration s replace D(s) once every
-  // thread is done reading it.  The nine nodes of the first Picard stage's
-  // cell are loaded once and reused for the foot when it lies in the same cell.
+  // The nine nodes of a Picard stage's cell are loaded once and reused by the stages
+  // that use the same cell.
   // (ADJ: the owned points only, the ones the reverse sweep reads; the others
   // serve the edge fluxes, which ADJ does not form)
   constexpr int NPTS = ADJ ? 3 * TX * TY : G::NPTS;
   constexpr int PER = (NPTS + NT - 1) / NT;
   const float th_full = a.dt / a.h;
-#pragma unroll 1
-  for (int s = 0; s < 2; ++s) {
+  // the point of work item t: family, cell, W cell and time-n value
+  struct Item {
+    int fam, px, py, wcP;
+    float4 wp;
+  };
+  auto item_of = [&](int t) {
+    Item m;
+    if constexpr (ADJ) {
+      m.fam = t / (TX * TY);
+      const int u = t - m.fam * (TX * TY);
+      m.px = u % TX;
+      m.py = u / TX;
+    } else {
+      point_item<PW, G::PH>(t, m.fam, m.px, m.py);
+    }
+    m.wcP = AF_IDX((m.py + 2) * CW + (m.px + 2), 0, WPL);
+    m.wp = W[m.fam * WPL + m.wcP];
+    return m;
+  };
+  // transported increment at the foot (D cell dcf, weights l); rho from dp / c_f^2
+  // (Sec. 6.1 step 4): u_f + du_f = I_h(u + du)(P_f) since both interpolants share
+  // the basis
+  auto transported = [&](const float* Ds, int dcf, const float lx[3], const float ly[3],
+                         const float2 lxd[3], const float2 lyd[3], const float2& rpf,
+                         unsigned& flag) {
+    const float2 e01 = q2_eval2<DCW>(reinterpret_cast<const float2*>(Ds),
+                                     reinterpret_cast<const float2*>(Ds + 3 * DPL),
+                                     reinterpret_cast<const float2*>(Ds + 6 * DPL),
+                                     reinterpret_cast<const float2*>(Ds + 9 * DPL), dcf, lxd, lyd);
+    const float e2 =
+        q2_eval<DCW>(Ds + 2 * DPL, Ds + 5 * DPL, Ds + 8 * DPL, Ds + 11 * DPL, dcf, lx, ly);
+    const float rf = gas.rho_ref + rpf.x, pf = gas.p_ref + rpf.y;
+    if (!(rf > 0.f && pf > 0.f)) flag |= FLAG_NONPHYSICAL;
+    Prim<float> nw = {rpf.x + __fdividef(e2 * rf, gas.gamma * pf), e01.x, e01.y, rpf.y + e2};
+    return nw;
+  };
+  // additive update (Eq. barsukow-additive), acoustic rho closure at P (D cell dcp)
+  auto additive = [&](const float* Ds, int fam, int dcp, const float4& wp, const float2& rpf,
+                      const float2& uvf) {
+    const float2 uv = reinterpret_cast<const float2*>(Ds + fam * 3 * DPL)[dcp];
+    const float dp = Ds[(fam * 3 + 2) * DPL + dcp];
+    Prim<float> nw = {
+        rpf.x + __fdividef(dp * (gas.rho_ref + wp.z), gas.gamma * (gas.p_ref + wp.w)),
+        uvf.x + (uv.x - wp.x), uvf.y + (uv.y - wp.y), rpf.y + dp};
+    return nw;
+  };
+  // its update over duration s; n holds the nine nodes of cell cn (-1: none yet), and
+  // keeps those of the last cell looked at
+  auto point = [&](const Item& m, int s, float4 n[9], int& cn) {
     const float th = s == 0 ? 0.5f * th_full : th_full;
     const float* Ds = D + s * 12 * DPL;
-    float4 res[PER];
+    const int fam = m.fam, px = m.px, py = m.py, wcP = m.wcP;
+    const float4 wp = m.wp;
+    const int ox = fam == 2 ? 1 : 0, oy = fam == 1 ? 1 : 0;
+    // first Picard stage from the point's own velocity (Eq. adv-footpoint)
+    const float2 d1 = __fmul2_rn(dup2(-th), rec_uv(wp));
+    if (!(fabsf(d1.x) <= 1.f && fabsf(d1.y) <= 1.f)) bad |= FLAG_REACH;
+    float lx[3], ly[3];
+    float2 lxd[3], lyd[3];
+    int ix = foot_axis(ox, clamp1(d1.x), lx), iy = foot_axis(oy, clamp1(d1.y), ly);
+    dup3(lx, lxd);
+    dup3(ly, lyd);
+    // (a cell's nine nodes reach one row and one column beyond it)
+    const int c1 = AF_IDX(wcP + iy * CW + ix, 0, WPL - CW - 1);
+    if (c1 != cn) load_cell<CW, WPL>(W, c1, n);
+    const float2 uv1 = q2_uv(n, lxd, lyd);
+    // the foot
+    const float2 df = __fmul2_rn(dup2(-th), uv1);
+    if (!(fabsf(df.x) <= 1.f && fabsf(df.y) <= 1.f)) bad |= FLAG_REACH;
+    ix = foot_axis(ox, clamp1(df.x), lx);
+    iy = foot_axis(oy, clamp1(df.y), ly);
+    dup3(lx, lxd);
+    dup3(ly, lyd);
+    const int c2 = AF_IDX(wcP + iy * CW + ix, 0, WPL - CW - 1);
+    if (c2 != c1) load_cell<CW, WPL>(W, c2, n);
+    cn = c2;
+    const float2 rpf = q2_rp(n, lxd, lyd);  // rho~_f, p~_f
+    Prim<float> nw;
+    if (a.variant == 0) {
+      const int dcf = AF_IDX((py + 1 + iy) * DCW + (px + 1 + ix), 0, DPL - DCW - 1);
+      nw = transported(Ds, dcf, lx, ly, lxd, lyd, rpf, bad);
+    } else {
+      const int dcp = AF_IDX((py + 1) * DCW + (px + 1), 0, DPL);
+      nw = additive(Ds, fam, dcp, wp, rpf, q2_uv(n, lxd, lyd));
+    }
+    if (!(isfinite(nw.r) && isfinite(nw.u) && isfinite(nw.v) && isfinite(nw.p)))
+      bad |= FLAG_NONFINITE;
+    // owned points go straight to HBM
+    const int gi = i0 + px, gj = j0 + py;
+    if ((INTER || ADJ) && s == 0 && px < TX && py < TY && gi < nx && gj < ny) {
+      const size_t id = (size_t)gj * nx + gi;
+      a.half[fam][0][id] = nw.r;
+      a.half[fam][1][id] = nw.u;
+      a.half[fam][2][id] = nw.v;
+      a.half[fam][3][id] = nw.p;
+    }
+    if (s == 1 && px < TX && py < TY && gi < nx && gj < ny) {
+      const size_t id = (size_t)gj * nx + gi;
+      a.out.pt[fam][0][id] = nw.r;
+      a.out.pt[fam][1][id] = nw.u;
+      a.out.pt[fam][2][id] = nw.v;
+      a.out.pt[fam][3][id] = nw.p;
+    }
+    return rec4(nw.r, nw.u, nw.v, nw.p);
+  };
+  // Both durations at once where every stage of every lane of the warp looks at the
+  // same cell (the usual case): their loads and chains overlap, and the nine nodes
+  // are loaded once.  False: the caller takes them one by one.
+  // (a form of its own for each variant: a branch between them inside would keep
+  // the durations' chains apart, 0.698 against 0.670 ms per step at 2048^2)
+  auto both_of = [&](auto variant, const Item& m, bool on, float4 r[2]) -> bool {
+    const float4 wp = m.wp;
+    const int ox = m.fam == 2 ? 1 : 0, oy = m.fam == 1 ? 1 : 0;
+    float2 lxd[2][3], lyd[2][3];
+    int c1[2], fx[2], fy[2];
+    unsigned far = 0;
 #pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const float th = s == 0 ? 0.5f * th_full : th_full;
+      const float2 d1 = __fmul2_rn(dup2(-th), rec_uv(wp));
+      if (!(fabsf(d1.x) <= 1.f && fabsf(d1.y) <= 1.f)) far |= FLAG_REACH;
+      float lx[3], ly[3];
+      const int ix = foot_axis(ox, clamp1(d1.x), lx), iy = foot_axis(oy, clamp1(d1.y), ly);
+      dup3(lx, lxd[s]);
+      dup3(ly, lyd[s]);
+      c1[s] = AF_IDX(m.wcP + iy * CW + ix, 0, WPL - CW - 1);
+    }
+    float4 n[9];
+    load_cell<CW, WPL>(W, c1[0], n);
+    float lx[2][3], ly[2][3];
+    bool same = c1[0] == c1[1];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const float th = s == 0 ? 0.5f * th_full : th_full;
+      const float2 df = __fmul2_rn(dup2(-th), q2_uv(n, lxd[s], lyd[s]));
+      if (!(fabsf(df.x) <= 1.f && fabsf(df.y) <= 1.f)) far |= FLAG_REACH;
+      fx[s] = foot_axis(ox, clamp1(df.x), lx[s]);
+      fy[s] = foot_axis(oy, clamp1(df.y), ly[s]);
+      dup3(lx[s], lxd[s]);
+      dup3(ly[s], lyd[s]);
+      same = same && m.wcP + fy[s] * CW + fx[s] == c1[0];
+    }
+    if (!__all_sync(0xffffffffu, same || !on)) return false;
+    if (on) bad |= far;
+    const int dcf = AF_IDX((m.py + 1 + fy[0]) * DCW + (m.px + 1 + fx[0]), 0, DPL - DCW - 1);
+    const int dcp = AF_IDX((m.py + 1) * DCW + (m.px + 1), 0, DPL);
+    unsigned b = 0;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const float* Ds = D + s * 12 * DPL;
+      const float2 rpf = q2_rp(n, lxd[s], lyd[s]);
+      Prim<float> nw;
+      if constexpr (decltype(variant)::value == 0)
+        nw = transported(Ds, dcf, lx[s], ly[s], lxd[s], lyd[s], rpf, b);
+      else
+        nw = additive(Ds, m.fam, dcp, wp, rpf, q2_uv(n, lxd[s], lyd[s]));
+      if (!(isfinite(nw.r) && isfinite(nw.u) && isfinite(nw.v) && isfinite(nw.p)))
+        b |= FLAG_NONFINITE;
+      const int gi = i0 + m.px, gj = j0 + m.py;
+      if ((s == 1 || INTER || ADJ) && on && m.px < TX && m.py < TY && gi < nx && gj < ny) {
+        const size_t id = (size_t)gj * nx + gi;
+        float* const* o = s == 1 ? a.out.pt[m.fam] : a.half[m.fam];
+        o[0][id] = nw.r;
+        o[1][id] = nw.u;
+        o[2][id] = nw.v;
+        o[3][id] = nw.p;
+      }
+      r[s] = rec4(nw.r, nw.u, nw.v, nw.p);
+    }
+    if (on) bad |= b;
+    return true;
+  };
+  auto both = [&](const Item& m, bool on, float4 r[2]) -> bool {
+    return a.variant == 0 ? both_of(std::integral_constant<int, 0>{}, m, on, r)
+                          : both_of(std::integral_constant<int, 1>{}, m, on, r);
+  };
+  if constexpr (ADJ) {
+    // both durations of a point back to back (the results only go to HBM)
+#pragma unroll 1
+    for (int t = threadIdx.x; t < NPTS; t += NT) {
+      const Item m = item_of(t);
+      float4 r[2];
+      if (both(m, true, r)) continue;
+      float4 n[9];
+      int cn = -1;
+#pragma unroll 1
+      for (int s = 0; s < 2; ++s) point(m, s, n, cn);
+    }
+  } else {
+    // Both durations of a point together: bound by instruction issue and shared
+    // memory, the pass saves the second load of the foot cell's nine nodes (36 of 134
+    // shared wavefronts per point) and half of the barriers, and the two chains hide
+    // each other's latency.  The results wait in tensor memory until every thread is
+    // done with the increments (in registers they would take 56; held for one
+    // duration at a time they spilled).  2048^2, FP32_COMP: 0.690 -> 0.677 ms per step,
+    // 1024^2 187 -> 180 us, 128^2 7.56 -> 7.14 us.  One duration after the other in the
+    // merged pass took 0.717 ms; the loop over k unrolled 0.5% more than rolled.
+    const int warp = threadIdx.x >> 5;
+    const unsigned park =
+        pc.tm_base + ((unsigned)(warp & 3) << 21) + (unsigned)((warp >> 2) * (8 * PER));
+    float4 held[2];  // (one point per thread: no parking)
+    auto park_store = [&](int k, const float4 r[2]) {
+      if constexpr (PER == 1) {
+        held[0] = r[0];
+        held[1] = r[1];
+      } else {
+        tm_store(park + 8 * k, r[0]);
+        tm_store(park + 8 * k + 4, r[1]);
+      }
+    };
+#pragma unroll 1
     for (int k = 0; k < PER; ++k) {
       const int t = threadIdx.x + k * NT;
-      if (k >= NPTS / NT && t >= NPTS) break;  // rounds k < NPTS / NT are full (NT threads)
-      int fam, px, py;
-      if constexpr (ADJ) {
-        fam = t / (TX * TY);
-        const int u = t - fam * (TX * TY);
-        px = u % TX;
-        py = u / TX;
-      } else {
-        point_item<PW, G::PH>(t, fam, px, py);
+      if ((t & ~31) >= NPTS) break;  // (the whole warp)
+      const bool on = t < NPTS;
+      const Item m = item_of(on ? t : NPTS - 1);
+      float4 r2[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+      if (both(m, on, r2)) {
+        park_store(k, r2);
+        continue;
       }
-      const int ox = fam == 2 ? 1 : 0, oy = fam == 1 ? 1 : 0;
-      const int wcP = AF_IDX((py + 2) * CW + (px + 2), 0, WPL);  // W cell of the point's cell
-      const float4 wp = W[fam * WPL + wcP];
-      // first Picard stage from the point's own velocity (Eq. adv-footpoint)
-      const float2 d1 = __fmul2_rn(dup2(-th), rec_uv(wp));
-      if (!(fabsf(d1.x) <= 1.f && fabsf(d1.y) <= 1.f)) bad |= FLAG_REACH;
-      float lx[3], ly[3];
-      float2 lxd[3], lyd[3];
-      int ix = foot_axis(ox, clamp1(d1.x), lx), iy = foot_axis(oy, clamp1(d1.y), ly);
-      dup3(lx, lxd);
-      dup3(ly, lyd);
-      // (a cell's nine nodes reach one row and one column beyond it)
-      const int c1 = AF_IDX(wcP + iy * CW + ix, 0, WPL - CW - 1);
       float4 n[9];
-      load_cell<CW, WPL>(W, c1, n);
-      const float2 uv1 = q2_uv(n, lxd, lyd);
-      // the foot
-      const float2 df = __fmul2_rn(dup2(-th), uv1);
-      if (!(fabsf(df.x) <= 1.f && fabsf(df.y) <= 1.f)) bad |= FLAG_REACH;
-      ix = foot_axis(ox, clamp1(df.x), lx);
-      iy = foot_axis(oy, clamp1(df.y), ly);
-      dup3(lx, lxd);
-      dup3(ly, lyd);
-      const int c2 = AF_IDX(wcP + iy * CW + ix, 0, WPL - CW - 1);
-      if (c2 != c1) load_cell<CW, WPL>(W, c2, n);
-      const float2 rpf = q2_rp(n, lxd, lyd);  // rho~_f, p~_f
-      const float rft = rpf.x, pft = rpf.y;
-      Prim<float> nw;
-      if (a.variant == 0) {
-        // transported increment at the foot; rho from dp / c_f^2 (Sec. 6.1 step 4):
-        // u_f + du_f = I_h(u + du)(P_f) since both interpolants share the basis
-        const int dcf = AF_IDX((py + 1 + iy) * DCW + (px + 1 + ix), 0, DPL - DCW - 1);
-        const float2 e01 = q2_eval2<DCW>(reinterpret_cast<const float2*>(Ds),
-                                         reinterpret_cast<const float2*>(Ds + 3 * DPL),
-                                         reinterpret_cast<const float2*>(Ds + 6 * DPL),
-                                         reinterpret_cast<const float2*>(Ds + 9 * DPL), dcf, lxd,
-                                         lyd);
-        const float e2 =
-            q2_eval<DCW>(Ds + 2 * DPL, Ds + 5 * DPL, Ds + 8 * DPL, Ds + 11 * DPL, dcf, lx, ly);
-        const float rf = gas.rho_ref + rft, pf = gas.p_ref + pft;
-        if (!(rf > 0.f && pf > 0.f)) bad |= FLAG_NONPHYSICAL;
-        nw.r = rft + __fdividef(e2 * rf, gas.gamma * pf);
-        nw.u = e01.x;
-        nw.v = e01.y;
-        nw.p = pft + e2;
-      } else {
-        // additive update (Eq. barsukow-additive), acoustic rho closure at P
-        const int dcp = AF_IDX((py + 1) * DCW + (px + 1), 0, DPL);
-        const float2 uv = reinterpret_cast<const float2*>(Ds + fam * 3 * DPL)[dcp];
-        const float du = uv.x - wp.x;
-        const float dv = uv.y - wp.y;
-        const float dp = Ds[(fam * 3 + 2) * DPL + dcp];
-        nw.r = rft + __fdividef(dp * (gas.rho_ref + wp.z), gas.gamma * (gas.p_ref + wp.w));
-        const float2 uvf = q2_uv(n, lxd, lyd);
-        nw.u = uvf.x + du;
-        nw.v = uvf.y + dv;
-        nw.p = pft + dp;
-      }
-      if (!(isfinite(nw.r) && isfinite(nw.u) && isfinite(nw.v) && isfinite(nw.p)))
-        bad |= FLAG_NONFINITE;
-      res[k] = rec4(nw.r, nw.u, nw.v, nw.p);
-      // owned points at t^{n+1} go straight to HBM
-      const int gi = i0 + px, gj = j0 + py;
-      if ((INTER || ADJ) && s == 0 && px < TX && py < TY && gi < nx && gj < ny) {
-        const size_t id = (size_t)gj * nx + gi;
-        a.half[fam][0][id] = nw.r;
-        a.half[fam][1][id] = nw.u;
-        a.half[fam][2][id] = nw.v;
-        a.half[fam][3][id] = nw.p;
-      }
-      if (s == 1 && px < TX && py < TY && gi < nx && gj < ny) {
-        const size_t id = (size_t)gj * nx + gi;
-        a.out.pt[fam][0][id] = nw.r;
-        a.out.pt[fam][1][id] = nw.u;
-        a.out.pt[fam][2][id] = nw.v;
-        a.out.pt[fam][3][id] = nw.p;
-      }
+      int cn = -1;
+#pragma unroll 1
+      for (int s = 0; s < 2; ++s)
+        if (on) (s == 0 ? r2[0] : r2[1]) = point(m, s, n, cn);
+      __syncwarp();
+      park_store(k, r2);
     }
-    __syncthreads();  // D(s) is dead from here (except for ADJ)
-    if constexpr (!ADJ) {
-      float4* P = reinterpret_cast<float4*>(D + s * 12 * DPL);
-#pragma unroll
-      for (int k = 0; k < PER; ++k) {
-        const int t = threadIdx.x + k * NT;
-        if (k >= NPTS / NT && t >= NPTS) break;
+    if constexpr (PER > 1) asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    __syncthreads();  // D is dead from here
+#pragma unroll 1
+    for (int k = 0; k < PER; ++k) {
+      const int t = threadIdx.x + k * NT;
+      if ((t & ~31) >= NPTS) break;
+      const float4 r0 = PER == 1 ? held[0] : tm_load(park + 8 * k);
+      const float4 r1 = PER == 1 ? held[1] : tm_load(park + 8 * k + 4);
+      if (t < NPTS) {
         int fam, px, py;
         point_item<PW, G::PH>(t, fam, px, py);
-        P[AF_IDX(fam * PPL + py * PW + px, 0, 3 * PPL)] = res[k];
+        const int at = AF_IDX(fam * PPL + py * PW + px, 0, 3 * PPL);
+        reinterpret_cast<float4*>(D)[at] = r0;
+        reinterpret_cast<float4*>(D + 12 * DPL)[at] = r1;
       }
     }
   }
@@ -946,9 +1138,11 @@ __global__ void __launch_bounds__(NT, MINB)
     pi0 = (nxt % gridDim.x) * TX;
     pj0 = (nxt / gridDim.x) * TY;
   }
-  PipeCtx none = {nullptr, 0u, 0u};
+  __shared__ unsigned tm_slot;
+  PipeCtx none = {nullptr, 0u, 0u, 0, tm_alloc<tm_cols<TX, TY, NT>()>(&tm_slot)};
   fused_tile<TX, TY, NT, COMP, false>(a, none, blockIdx.x * TX, blockIdx.y * TY, pi0, pj0,
                                       pi0 >= 0);
+  tm_free<tm_cols<TX, TY, NT>()>(none.tm_base);
 }
 
 // Persistent pipelined form: CTA b steps through tiles b, b + G, b + 2G, ...
@@ -978,7 +1172,8 @@ __global__ void __launch_bounds__(NT, MINB)
     for (int p = threadIdx.x >> 5; p < 20; p += NT / 32)
       asm volatile("prefetch.tensormap [%0];" ::"l"(&tm.m[p]) : "memory");
   pdl_wait();
-  __syncthreads();
+  pc.tm_base = tm_alloc<tm_cols<TX, TY, NT>()>(
+      reinterpret_cast<unsigned*>(reinterpret_cast<char*>(smem4) + G::SMEM + 8));
   const int tcols = (a.nx + TX - 1) / TX, ntiles = tcols * ((a.ny + TY - 1) / TY);
   int tile = blockIdx.x;
   if (tile < ntiles)
@@ -992,6 +1187,7 @@ __global__ void __launch_bounds__(NT, MINB)
                                                    a.prefetch_wave > 0 && !pc.tm))
       break;
   }
+  tm_free<tm_cols<TX, TY, NT>()>(pc.tm_base);
 }
 
 // Batched form: one CTA per entry (grid, i0, j0, -) of a tile table spanning
@@ -1001,8 +1197,10 @@ __global__ void __launch_bounds__(NT, MINB)
     k_fused_step_batch(const StepArgs<float>* __restrict__ args, const int4* __restrict__ tiles) {
   pdl_wait();
   const int4 t = tiles[blockIdx.x];
-  PipeCtx none = {nullptr, 0u, 0u};
+  __shared__ unsigned tm_slot;
+  PipeCtx none = {nullptr, 0u, 0u, 0, tm_alloc<tm_cols<TX, TY, NT>()>(&tm_slot)};
   fused_tile<TX, TY, NT, COMP, false>(args[t.x], none, t.y, t.z, -1, -1, false);
+  tm_free<tm_cols<TX, TY, NT>()>(none.tm_base);
 }
 
 // Batched persistent pipelined form: CTA b steps through entries b, b + G, ...
@@ -1029,7 +1227,8 @@ __global__ void __launch_bounds__(NT, MINB)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   pdl_wait();
-  __syncthreads();
+  pc.tm_base = tm_alloc<tm_cols<TX, TY, NT>()>(
+      reinterpret_cast<unsigned*>(reinterpret_cast<char*>(smem4) + G::SMEM + 8));
   int t = blockIdx.x;
   if (t < ntiles) {
     const int4 e = tiles[t];
@@ -1046,6 +1245,7 @@ __global__ void __launch_bounds__(NT, MINB)
                                             &args[ne.x], tma ? &maps[ne.x] : nullptr))
       break;
   }
+  tm_free<tm_cols<TX, TY, NT>()>(pc.tm_base);
 }
 
 constexpr int FUSED_TX = AF_FUSED_TX, FUSED_TY = AF_FUSED_TY, FUSED_NT = AF_FUSED_NT;

@@ -104,9 +104,10 @@ inline cudaError_t launch_step_pipe(cudaStream_t s, const StepArgs<float>& a, in
 // them a grid has, so a grid too small to give every SM one of those runs faster
 // on smaller tiles although they recompute more halo.  `us` is the measured time
 // of one wave (FP32_COMP, GB300); the geometry with the smallest sum is taken.
-// Measured per step, 32 x 32 tiles -> chosen: 32^2 27.4 -> 5.3 us (8 x 4), 64^2 30.8 -> 6.5
-// (8 x 8), 128^2 30.8 -> 7.6 (16 x 8), 192^2 30.9 -> 11.2 (16 x 16), 256^2 30.9 -> 16.8
-// (32 x 16), 333 x 250 30.8 -> 21.8 (32 x 24), 448^2 57.7 -> 42.4 (32 x 24).
+// Measured per step, 32 x 32 tiles -> chosen: 32^2 27.4 -> 5.1 us (8 x 4), 64^2 30.8 -> 6.4
+// (8 x 8), 128^2 30.8 -> 7.1 (16 x 8), 192^2 30.9 -> 10.9 (16 x 16), 256^2 30.9 -> 16.5
+// (32 x 16), 333 x 250 30.8 -> 21.6 (32 x 24), 448^2 57.7 -> 42 (32 x 24), 512^2 57.7 ->
+// 48 (persistent, 28 rows: two full waves).
 struct StepGeometry {
   int tx, ty;
   int pipe;      // persistent CTAs with the next tile's input staged asynchronously
@@ -116,10 +117,10 @@ struct StepGeometry {
 enum { GEOM_8x4, GEOM_8x8, GEOM_16x8, GEOM_16x16, GEOM_32x16, GEOM_32x24, GEOM_32x32,
        GEOM_PIPE_32x28, GEOM_PIPE_32x32, N_STEP_GEOMS };
 constexpr StepGeometry STEP_GEOMS[N_STEP_GEOMS] = {
-    {8, 4, 0, 5.9f, 0.f},   {8, 8, 0, 6.6f, 0.f},   {16, 8, 0, 7.5f, 0.f},
-    {16, 16, 0, 11.2f, 0.f}, {32, 16, 0, 16.7f, 0.f}, {32, 24, 0, 21.6f, 0.f},
-    {FUSED_TX, FUSED_TY, 0, 28.5f, 0.f},
-    {FUSED_TX, 28, 1, 22.5f, 4.f}, {FUSED_TX, FUSED_TY, 1, 25.5f, 4.f}};
+    {8, 4, 0, 5.7f, 0.f},   {8, 8, 0, 6.4f, 0.f},   {16, 8, 0, 7.2f, 0.f},
+    {16, 16, 0, 10.9f, 0.f}, {32, 16, 0, 16.5f, 0.f}, {32, 24, 0, 21.5f, 0.f},
+    {FUSED_TX, FUSED_TY, 0, 28.2f, 0.f},
+    {FUSED_TX, 28, 1, 22.f, 4.f}, {FUSED_TX, FUSED_TY, 1, 25.1f, 4.f}};
 
 inline int choose_step_geometry(const StepArgs<float>& a, int sms) {
   int best = GEOM_32x32;
