@@ -71,6 +71,9 @@ struct af_handle {
   cudaEvent_t ev_fork, ev_join, ev_in;
   int late_once;         // testing only (AF_TEST_LATE_WAIT=1 at af_init): the first
                          // pipelined step reports its first staged-tile wait as timed out
+  int after_event;       // 1: the stream was made to wait for another stream's event since
+                         // its last import or export; the next one is launched without
+                         // the programmatic attribute, which speaks of kernels only
   int out_pending;       // 1: the outgoing copies of the last exchange may be in flight
   af_state_f64 pending_out;  // ... into these planes
   // af_exchange_state_async (lazy): two incoming and two outgoing staging
@@ -455,18 +458,20 @@ af_status import_enqueue(af_handle* h, const af_state_f64* in, af_memory where,
   }
   const dim3 g(grid1d(h->N, COPY_THREADS)), t(COPY_THREADS);
   const Offsets o = offsets_of(h);
+  const bool dependent = !h->after_event;
+  h->after_event = 0;
   cudaError_t e = cudaSuccess;
   switch (h->prec) {
     case AF_FP64:
-      e = launch_dependent(k_import<double, false>, g, t, 0, h->stream, src,
+      e = launch_kernel(dependent, k_import<double, false>, g, t, 0, h->stream, src,
                            planes_of<double>(h, h->cur), h->N, o, flags);
       break;
     case AF_FP32:
-      e = launch_dependent(k_import<float, false>, g, t, 0, h->stream, src,
+      e = launch_kernel(dependent, k_import<float, false>, g, t, 0, h->stream, src,
                            planes_of<float>(h, h->cur), h->N, o, flags);
       break;
     case AF_FP32_COMP:
-      e = launch_dependent(k_import<float, true>, g, t, 0, h->stream, src,
+      e = launch_kernel(dependent, k_import<float, true>, g, t, 0, h->stream, src,
                            planes_of<float>(h, h->cur), h->N, o, flags);
       break;
   }
@@ -487,10 +492,9 @@ bool overlaps_pending_out(const af_handle* h, const af_state_f64* in) {
 // (af_exchange_state, af_exchange_state_async), which may still be in flight
 // on the aux stream (ev_join follows the latest of them).
 af_status wait_outgoing(af_handle* h) {
-  if ((h->out_pending || h->apending[0] || h->apending[1]) &&
-      cudaStreamWaitEvent(h->stream, h->ev_join, 0) != cudaSuccess)
-    return cuda_fail(h);
-  return AF_OK;
+  if (!(h->out_pending || h->apending[0] || h->apending[1])) return AF_OK;
+  h->after_event = 1;
+  return cudaStreamWaitEvent(h->stream, h->ev_join, 0) == cudaSuccess ? AF_OK : cuda_fail(h);
 }
 
 // Waits until the stream has passed the new state (and, the caller having called
@@ -514,18 +518,20 @@ af_status import_state(af_handle* h, const af_state_f64* in, af_memory where) {
 af_status export_enqueue(af_handle* h, const F64Out& dst) {
   const dim3 g(grid1d(h->N, COPY_THREADS)), t(COPY_THREADS);
   const Offsets o = offsets_of(h);
+  const bool dependent = !h->after_event;
+  h->after_event = 0;
   cudaError_t e = cudaSuccess;
   switch (h->prec) {
     case AF_FP64:
-      e = launch_dependent(k_export<double, false>, g, t, 0, h->stream,
+      e = launch_kernel(dependent, k_export<double, false>, g, t, 0, h->stream,
                            planes_of<double>(h, h->cur), dst, h->N, o);
       break;
     case AF_FP32:
-      e = launch_dependent(k_export<float, false>, g, t, 0, h->stream,
+      e = launch_kernel(dependent, k_export<float, false>, g, t, 0, h->stream,
                            planes_of<float>(h, h->cur), dst, h->N, o);
       break;
     case AF_FP32_COMP:
-      e = launch_dependent(k_export<float, true>, g, t, 0, h->stream,
+      e = launch_kernel(dependent, k_export<float, true>, g, t, 0, h->stream,
                            planes_of<float>(h, h->cur), dst, h->N, o);
       break;
   }
@@ -935,6 +941,7 @@ af_status af_exchange_state(af_handle* h, const af_state_f64* out, const af_stat
   if (cudaEventRecord(h->ev_join, h->aux) != cudaSuccess ||
       cudaStreamWaitEvent(h->stream, h->ev_in, 0) != cudaSuccess)
     return cuda_fail(h);
+  h->after_event = 1;
   st = import_enqueue(h, &staged, AF_DEVICE, h->d_flags);
   if (st == AF_OK) st = import_finish(h);
   if (st == AF_OK) {
@@ -988,6 +995,7 @@ af_status af_exchange_state_async(af_handle* h, const af_state_f64* out,
   F64Out dst;
   for (int p = 0; p < 16; ++p) dst.p[p] = h->axstage[b] + (size_t)p * N;
   if (cudaStreamWaitEvent(h->stream, h->ev_sent[b], 0) != cudaSuccess) return cuda_fail(h);
+  h->after_event = 1;
   af_status st = export_enqueue(h, dst);
   if (st != AF_OK) return st;
   if (cudaEventRecord(h->ev_exported[b], h->stream) != cudaSuccess ||
@@ -1001,6 +1009,7 @@ af_status af_exchange_state_async(af_handle* h, const af_state_f64* out,
     return cuda_fail(h);
   // the new state, on the handle's stream after the incoming copy
   if (cudaStreamWaitEvent(h->stream, h->ev_staged[b], 0) != cudaSuccess) return cuda_fail(h);
+  h->after_event = 1;
   st = import_enqueue(h, &staged, AF_DEVICE);
   if (st != AF_OK) return st;
   if (cudaEventRecord(h->ev_imported[b], h->stream) != cudaSuccess) return cuda_fail(h);
