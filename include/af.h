@@ -119,8 +119,9 @@ enum {
  * planes; af_destroy frees all of them.  Kernel choices, read from the environment when the handle is created
  * (the results are the same up to rounding; they exist for comparison and
  * testing): AF_PATH=ref runs the FP32 modes on the kernel-per-stage path
- * instead of the fused kernel; AF_PIPE=0 replaces the persistent pipelined
- * fused kernel by one CTA per tile, AF_PIPE=n caps its grid at n CTAs;
+ * instead of the fused kernel, whose tiles are otherwise chosen by the grid's
+ * size; AF_PIPE=n keeps the persistent pipelined kernel on 32x32 tiles with at
+ * most n CTAs, AF_PIPE=0 one CTA per 32x32 tile;
  * AF_TMA=0 stages every tile by cp.async instead of tensor copies;
  * AF_PREFETCH=0 disables the L2 prefetch of the one-CTA-per-tile kernel;
  * AF_ZERO_COPY=0 copies pinned host planes through a staging buffer instead

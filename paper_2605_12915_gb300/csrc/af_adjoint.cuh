@@ -594,12 +594,13 @@ __device__ __forceinline__ void acoustic_adj(const AdjView<T>& v, int i, int j, 
 }
 
 // Blocks of the acoustic adjoint: BY rows of 32 consecutive nodes.  FP32 waits on
-// scattered loads and atomics: 256 threads, three blocks per SM (at most 85
-// registers).  FP64 is bound by its arithmetic unit and would spill: two warps,
-// registers as needed.
+// scattered loads and atomics, and the vertex family spills below 96 registers: 128
+// threads, five blocks per SM (adjoint step at 2048^2 2.89 ms; three of 256 threads at
+// 80 registers 2.94, two at 128 2.98, four of 128 or of 192 2.95 and 2.93).  FP64 is bound
+// by its arithmetic unit and would spill: two warps, registers as needed.
 template <typename T>
 struct AdjBlock {
-  static constexpr int BY = sizeof(T) == 4 ? 8 : 2, MINB = sizeof(T) == 4 ? 3 : 1;
+  static constexpr int BY = sizeof(T) == 4 ? 4 : 2, MINB = sizeof(T) == 4 ? 5 : 1;
 };
 
 // the families by blockIdx.z
@@ -628,9 +629,9 @@ __global__ void __launch_bounds__(32 * AdjBlock<T>::BY, AdjBlock<T>::MINB)
 // vertex, two for an edge, no atomics) before writing lambda^n out.
 // ---------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(128) k_adj_center(const __grid_constant__ AdjView<T> v) {
+__global__ void __launch_bounds__(REF_THREADS) k_adj_center(const __grid_constant__ AdjView<T> v) {
   pdl_wait();
-  const size_t id = (size_t)blockIdx.x * 128 + threadIdx.x, ps = v.ps;
+  const size_t id = (size_t)blockIdx.x * REF_THREADS + threadIdx.x, ps = v.ps;
   if (id >= (size_t)v.nx * v.ny) return;
   T* lc = v.lam + (size_t)(LAM_NODE + 12) * ps + 4 * id;  // the centre node's record
   const T lw[4] = {lc[0], lc[1], lc[2], lc[3]};
