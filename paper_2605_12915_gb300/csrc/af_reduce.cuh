@@ -110,7 +110,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_inv_partial(const __grid_consta
   double acc[RED_SUMS] = {};
   double smax = 0.0;
   const float near_top = __uint_as_float(*a.top) * 0.9999995f;
-  T seen[4] = {};          // (rho, u, v, p) of the lane's last FP64 wave speed
+  T seen[4] = {};          // (rho, u, v, p) of the lane's last FP64 wave speed,
+  bool any_seen = false;   // if it has taken one
   T rmin = (T)INFINITY, pmin = (T)INFINITY;  // of the stored offsets
   const size_t N = (size_t)a.nx * a.ny;
   for (size_t id = (size_t)blockIdx.x * RED_THREADS + threadIdx.x; id < N;
@@ -175,9 +176,10 @@ __global__ void __launch_bounds__(RED_THREADS) k_inv_partial(const __grid_consta
 #pragma unroll
       for (int k = 0; k < 4; ++k)
         q[k] = n == 0 ? w[0][k] : n == 1 ? w[1][k] : n == 2 ? w[2][k] : w[3][k];
-      if (same_bits(q[0], seen[0]) && same_bits(q[1], seen[1]) && same_bits(q[2], seen[2]) &&
-          same_bits(q[3], seen[3]))
+      if (any_seen && same_bits(q[0], seen[0]) && same_bits(q[1], seen[1]) &&
+          same_bits(q[2], seen[2]) && same_bits(q[3], seen[3]))
         continue;
+      any_seen = true;
 #pragma unroll
       for (int k = 0; k < 4; ++k) seen[k] = q[k];
       const double rr = sizeof(T) == 4 ? wide(q[0]) + a.rho_ref : wide(q[0]);

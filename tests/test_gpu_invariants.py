@@ -68,3 +68,18 @@ def test_fp64_sums_and_extrema(shape, spread):
     assert abs(got[7] - speed) < 1e-12 * speed
     assert abs(got[8] - min(w[0].min() for w in nodes)) < 1e-13 * np.max(np.abs(st[0]))
     assert abs(got[9] - min(w[3].min() for w in nodes)) < 1e-13 * np.max(np.abs(st[3]))
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp32_comp", "fp64"])
+@pytest.mark.parametrize("u", [0.0, 0.4])
+def test_uniform_state_has_its_wave_speed(precision, u):
+    """Every stored value of a uniform state at rest is 0 in the FP32 modes (offsets
+    from the reference state): the maximum is still the sound speed."""
+    from workloads import inputs as I
+    P = I.uniform(37, 21, rho=1.3, u=u, v=0.0, p=0.9)
+    s = af.Solver(P.grid, P.gamma, P.state, precision=precision)
+    got = s.invariants()
+    s.close()
+    want = u + np.sqrt(P.gamma * 0.9 / 1.3)
+    # the recovered centre carries the rounding of the averages in the working precision
+    assert abs(got[7] - want) < (1e-6 if precision != "fp64" else 1e-13) * want
