@@ -288,7 +288,7 @@ void launch_fc_step(af_handle* h, double dt) {
     n.ey[k] = (double*)h->scratch[16 + k];
   }
   launch_dependent(k_center<double, false>, dim3(b), REF_THREADS, 0, h->stream, a,
-                   (unsigned*)nullptr);
+                   TopSpeed{});
   launch_fc_points(a, h->stream);
   launch_dependent(k_node_flux<double>, dim3(b), REF_THREADS, 0, h->stream, a, n);
   launch_dependent(k_average<double, false>, dim3(b), REF_THREADS, 0, h->stream, a, n);
@@ -1029,13 +1029,18 @@ af_status af_reduce_invariants(af_handle* h, double* out) {
   if (wait_outgoing(h) != AF_OK) return AF_ERR_CUDA;
   double* partial = h->d_red;
   const int blocks = (int)std::min<size_t>(h->red_blocks, (h->N + RED_THREADS - 1) / RED_THREADS);
+  auto pair = [](double x) {
+    const float hi = (float)x;
+    return RefPair{hi, (float)(x - (double)hi)};
+  };
+  const TopSpeed top = {h->d_top, pair(h->rho_ref), pair(h->p_ref), (float)h->gamma};
   if (h->prec == AF_FP64) {
     StepArgs<double> a = step_args<double>(h, 1.0);
-    k_center<double, false, true><<<ref_blocks(a), REF_THREADS, 0, h->stream>>>(a, h->d_top);
+    k_center<double, false, true><<<ref_blocks(a), REF_THREADS, 0, h->stream>>>(a, top);
     RedArgs<double> r;
     r.st = a.in;
     for (int k = 0; k < 4; ++k) r.wc[k] = a.wc[k];
-    r.nx = h->nx; r.ny = h->ny; r.gamma = h->gamma; r.h = h->h; r.partial = partial; r.top = h->d_top;
+    r.nx = h->nx; r.ny = h->ny; r.gamma = h->gamma; r.h = h->h; r.partial = partial; r.top = top;
     r.rho_ref = h->rho_ref; r.p_ref = h->p_ref; r.e_ref = h->p_ref / (h->gamma - 1.0);
     k_inv_partial<double, false><<<blocks, RED_THREADS, 0, h->stream>>>(r);
   } else {
@@ -1043,13 +1048,13 @@ af_status af_reduce_invariants(af_handle* h, double* out) {
     RedArgs<float> r;
     r.st = a.in;
     for (int k = 0; k < 4; ++k) r.wc[k] = a.wc[k];
-    r.nx = h->nx; r.ny = h->ny; r.gamma = h->gamma; r.h = h->h; r.partial = partial; r.top = h->d_top;
+    r.nx = h->nx; r.ny = h->ny; r.gamma = h->gamma; r.h = h->h; r.partial = partial; r.top = top;
     r.rho_ref = h->rho_ref; r.p_ref = h->p_ref; r.e_ref = h->p_ref / (h->gamma - 1.0);
     if (h->prec == AF_FP32_COMP) {
-      k_center<float, true, true><<<ref_blocks(a), REF_THREADS, 0, h->stream>>>(a, h->d_top);
+      k_center<float, true, true><<<ref_blocks(a), REF_THREADS, 0, h->stream>>>(a, top);
       k_inv_partial<float, true><<<blocks, RED_THREADS, 0, h->stream>>>(r);
     } else {
-      k_center<float, false, true><<<ref_blocks(a), REF_THREADS, 0, h->stream>>>(a, h->d_top);
+      k_center<float, false, true><<<ref_blocks(a), REF_THREADS, 0, h->stream>>>(a, top);
       k_inv_partial<float, false><<<blocks, RED_THREADS, 0, h->stream>>>(r);
     }
   }

@@ -193,14 +193,37 @@ __device__ __forceinline__ void flux_y(const Prim<T>& w, const Gas<T>& g, T f[4]
 __device__ __forceinline__ float narrow_any(float x) { return x; }
 __device__ __forceinline__ float narrow_any(double x) { return narrow(x); }
 
-// |u| + c of a node (absolute rho, p) in FP32, within 2e-7 relative (three roundings each in |u| and in the
-// square of c, which its root halves, one in the sum); infinity where FP32 cannot tell
-__device__ __forceinline__ float wave_speed_f32(float r, float u, float v, float p, float gamma) {
+// A storage offset's reference as the sum of two floats (hi nearest, lo the rest)
+struct RefPair {
+  float hi, lo;
+};
+// The absolute value (hi + lo) + x to 2^-24 of itself (and 2^-49 of the reference), also
+// where hi and x cancel, as they do at a light node beside a dense reference: the
+// rounding of hi + x is recovered exactly.
+__device__ __forceinline__ float with_ref_pair(RefPair ref, float x) {
+  const float s = ref.hi + x, b = s - ref.hi;
+  return s + (((ref.hi - (s - b)) + (x - b)) + ref.lo);
+}
+__device__ __forceinline__ float with_ref_pair(RefPair, double x) { return narrow(x); }
+
+// |u| + c of a stored node in FP32, within 5 x 2^-24 = 3e-7 relative.  Roundings, in
+// units of 2^-24: c^2 five (gamma, rho, p, quotient, product), which the root halves
+// and adds one to; |u| four (1.5 of the quotient t, whose square enters with weight 1/2 at
+// most, 0.5 of the sum under the root, the root, the larger component); the final sum
+// one.  Infinity where FP32 cannot tell: an overflow, an underflow, an infinity or NaN
+// in any of the values.
+template <typename T>
+__device__ __forceinline__ float wave_speed_f32(RefPair rho_ref, RefPair p_ref, T r_, T u_, T v_,
+                                                T p_, float gamma) {
+  const float r = with_ref_pair(rho_ref, r_), p = with_ref_pair(p_ref, p_);
+  const float u = narrow_any(u_), v = narrow_any(v_);
   const float a = fmaxf(fabsf(u), fabsf(v)), b = fminf(fabsf(u), fabsf(v));
   const float t = a > 0.f ? b / a : 0.f;
   const float c2 = gamma * (p / r);
-  if (!(c2 > 1e-30f) || (a > 0.f && a < 1e-30f)) return INFINITY;
-  return fmaf(a, sqrtf(fmaf(t, t, 1.f)), sqrtf(c2));
+  if (!(c2 > 1e-30f) || !(fminf(r, p) > 1e-37f) || (a > 0.f && a < 1e-30f)) return INFINITY;
+  // (the last term is 0, or NaN if u or v is NaN or infinite: maxima and minima drop NaN)
+  const float s = fmaf(a, sqrtf(fmaf(t, t, 1.f)), sqrtf(c2)) + 0.f * (u + v);
+  return s < INFINITY ? s : INFINITY;
 }
 
 // ---- Q2 Lagrange basis on nodes -1, 0, 1 (Sec. 4) ----------------------------

@@ -17,6 +17,7 @@
 #pragma once
 
 #include "af_common.cuh"
+#include "af_ref_kernels.cuh"
 
 namespace af {
 
@@ -31,7 +32,7 @@ struct RedArgs {
   int nx, ny;
   double gamma, h;
   double rho_ref, p_ref, e_ref;  // storage offsets (see Gas)
-  const unsigned* top;  // bits of the grid's largest FP32 wave speed
+  TopSpeed top;         // the grid's largest FP32 wave speed (k_center found it)
   double* partial;      // [RED_VALS][gridDim.x]
 };
 
@@ -109,7 +110,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_inv_partial(const __grid_consta
   __syncthreads();
   double acc[RED_SUMS] = {};
   double smax = 0.0;
-  const float near_top = __uint_as_float(*a.top) * 0.9999995f;
+  const float near_top = __uint_as_float(*a.top.bits) * (1.f - 1e-6f);
   T seen[4] = {};          // (rho, u, v, p) of the lane's last FP64 wave speed,
   bool any_seen = false;   // if it has taken one
   T rmin = (T)INFINITY, pmin = (T)INFINITY;  // of the stored offsets
@@ -163,11 +164,13 @@ __global__ void __launch_bounds__(RED_THREADS) k_inv_partial(const __grid_consta
       H[n] = entropy_density(r, p, a.gamma, tab);
       keep_min(rmin, w[n][0]);
       keep_min(pmin, w[n][3]);
-      sf[n] = wave_speed_f32(narrow_any(r), narrow_any(w[n][1]), narrow_any(w[n][2]),
-                             narrow_any(p), (float)a.gamma);
+      sf[n] = wave_speed_f32(a.top.rho_ref, a.top.p_ref, w[n][0], w[n][1], w[n][2], w[n][3],
+                             a.top.gamma);
     }
-    // the wave speed in FP64 only at nodes whose FP32 value is within 5e-7 of the
-    // grid's largest (k_center found it)
+    // The wave speed in FP64 only at nodes whose FP32 value is within 1e-6 of the
+    // grid's largest.  k_center found that one by the same operations on the same
+    // stored values, so the node that gave it is always among them; each FP32 value is
+    // within 3e-7 of its node's, so the node of the largest FP64 value is too.
 #pragma unroll 1
     for (int n = 0; n < 4; ++n) {
       const float sn = n == 0 ? sf[0] : n == 1 ? sf[1] : n == 2 ? sf[2] : sf[3];

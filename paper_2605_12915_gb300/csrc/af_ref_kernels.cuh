@@ -108,11 +108,16 @@ __device__ __forceinline__ Nbhd nbhd(int ci, int cj, int nx, int ny) {
 // keeps the cancellation small; FP64 as U_c = 9/4 Ubar - sum_corners U_V / 16 -
 // sum_edges U_E / 4 (half the operations).
 // ---------------------------------------------------------------------------
-// TOP: also raises *top to the bits of the largest FP32 wave speed of the cell's
+// TOP: also raises *top.bits to the bits of the largest FP32 wave speed of the cell's
 // own nodes (positive floats compare as their bits).
+struct TopSpeed {
+  unsigned* bits;
+  RefPair rho_ref, p_ref;
+  float gamma;
+};
 template <typename T, bool COMP, bool TOP = false>
 __global__ void __launch_bounds__(REF_THREADS)
-    k_center(const __grid_constant__ StepArgs<T> a, unsigned* top) {
+    k_center(const __grid_constant__ StepArgs<T> a, const __grid_constant__ TopSpeed top) {
   pdl_wait();
   int i, j;
   size_t id;
@@ -171,15 +176,13 @@ __global__ void __launch_bounds__(REF_THREADS)
   a.wc[3][id] = w.p;
   if constexpr (TOP) {
     auto speed = [&](const Prim<T>& n) {
-      const float s = wave_speed_f32(narrow_any(with_ref(a.gas.rho_ref, n.r)), narrow_any(n.u),
-                                     narrow_any(n.v), narrow_any(with_ref(a.gas.p_ref, n.p)),
-                                     (float)a.gas.gamma);
+      const float s = wave_speed_f32(top.rho_ref, top.p_ref, n.r, n.u, n.v, n.p, top.gamma);
       return s < INFINITY ? s : 0.f;  // (the reduction looks at the others itself)
     };
     const float s = fmaxf(fmaxf(speed(corners[0]), speed(edges[0])),
                           fmaxf(speed(edges[2]), speed(w)));
     const unsigned m = __reduce_max_sync(__activemask(), __float_as_uint(s));
-    if (m > *(volatile unsigned*)top) atomicMax(top, m);
+    if (m > *(volatile unsigned*)top.bits) atomicMax(top.bits, m);
   }
   raise_flag(a.flags, (is_positive(with_ref(a.gas.rho_ref, w.r)) &&
                        is_positive(with_ref(a.gas.p_ref, w.p)))

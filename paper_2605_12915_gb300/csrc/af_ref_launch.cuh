@@ -44,7 +44,7 @@ template <typename T, bool COMP>
 inline cudaError_t launch_ref_nodes(const StepArgs<T>& a, cudaStream_t s) {
   const unsigned b = ref_blocks(a);
   const cudaError_t e = launch_dependent(k_center<T, COMP>, dim3(b), REF_THREADS, 0, s, a,
-                                         (unsigned*)nullptr);
+                                         TopSpeed{});
   if (e != cudaSuccess) return e;
   return launch_dependent(k_acoustic<T>, dim3(b, 4), REF_THREADS, 0, s, a);
 }

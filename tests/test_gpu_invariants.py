@@ -83,3 +83,90 @@ def test_uniform_state_has_its_wave_speed(precision, u):
     want = u + np.sqrt(P.gamma * 0.9 / 1.3)
     # the recovered centre carries the rounding of the averages in the working precision
     assert abs(got[7] - want) < (1e-6 if precision != "fp64" else 1e-13) * want
+
+
+def _at_rest(ref, light, p_light, centre, shape=(40, 33)):
+    """Density `ref` (vertex (0, 0), the FP32 modes' storage reference, among it) and
+    pressure 1 with a patch of density `light` and pressure `p_light`; averages whose
+    recovered centres have density `centre` and pressure 1 everywhere."""
+    nx, ny = shape
+    st = np.zeros((16, ny, nx))
+    for base in (4, 8, 12):
+        st[base], st[base + 3] = ref, 1.0
+        st[base, 10:20, 10:20], st[base + 3, 10:20, 10:20] = light, p_light
+    roll = lambda a, dy, dx: np.roll(a, (-dy, -dx), (0, 1))
+    for k, scale in ((0, 1.0), (3, 1 / (G - 1))):
+        V, X, Y = (scale * st[b + k] for b in (4, 8, 12))
+        st[k] = 4 / 9 * (scale * (centre if k == 0 else 1.0) +
+                         (V + roll(V, 0, 1) + roll(V, 1, 0) + roll(V, 1, 1)) / 16 +
+                         (X + roll(X, 0, 1) + Y + roll(Y, 1, 0)) / 4)
+    return st
+
+
+def _points(st):
+    return np.concatenate([st[b:b + 4].reshape(4, -1) for b in (4, 8, 12)], axis=1)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp32_comp", "fp64"])
+@pytest.mark.parametrize("ref,light,p_light", [
+    (1.3, 0.05, 1.0), (2.6, 0.05, 1.0), (0.9, 0.02, 1.0), (1.3, 0.01, 0.3), (2.6, 1e-4, 1e-3),
+    (0.3, 2.0, 7.0)])
+def test_extrema_of_a_light_patch_beside_a_dense_reference(precision, ref, light, p_light):
+    """The storage offset cancels at the light nodes, where the sound speed is largest:
+    the extrema are those of the exported state (the centres are denser, at rest), to
+    FP64 rounding."""
+    centre = max(ref, light)
+    st = _at_rest(ref, light, p_light, centre)
+    s = af.Solver(_Grid(40, 33), G, st, precision=precision)
+    got = s.invariants()
+    r, u, v, p = _points(s.state())
+    s.close()
+    assert abs(got[7] - np.max(np.sqrt(G * p / r))) < 1e-13 * got[7]
+    assert abs(got[8] - min(r.min(), centre)) < 1e-13 * ref
+    assert abs(got[9] - min(p.min(), 1.0)) < (1e-13 if p_light < 1 else 1e-6)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp32_comp", "fp64"])
+def test_largest_of_many_nearly_equal_wave_speeds(precision):
+    """Speeds that differ by less than FP32 resolves: the reported one is the largest of
+    the exported state (the centres are at rest), to FP64 rounding."""
+    rng = np.random.default_rng(4)
+    st = _at_rest(1.3, 1.3, 1.0, 1.3)
+    for base in (4, 8, 12):
+        ang = rng.uniform(0, 2 * np.pi, st[0].shape)
+        mag = 0.4 * (1 + 1e-7 * rng.normal(size=st[0].shape))
+        st[base + 1], st[base + 2] = mag * np.cos(ang), mag * np.sin(ang)
+        st[base] *= 1 + 1e-7 * rng.normal(size=st[0].shape)
+    # averages of centres at rest
+    roll = lambda a, dy, dx: np.roll(a, (-dy, -dx), (0, 1))
+    cons = [[w[0], w[0] * w[1], w[0] * w[2], 2.5 * w[3] + 0.5 * w[0] * (w[1] ** 2 + w[2] ** 2)]
+            for w in (st[4:8], st[8:12], st[12:16])]
+    for k, c in enumerate((1.3, 0.0, 0.0, 2.5)):
+        V, X, Y = cons[0][k], cons[1][k], cons[2][k]
+        st[k] = 4 / 9 * (c + (V + roll(V, 0, 1) + roll(V, 1, 0) + roll(V, 1, 1)) / 16 +
+                         (X + roll(X, 0, 1) + Y + roll(Y, 1, 0)) / 4)
+    s = af.Solver(_Grid(40, 33), G, st, precision=precision)
+    got = s.invariants()
+    r, u, v, p = _points(s.state())
+    s.close()
+    want = np.max(np.sqrt(u * u + v * v) + np.sqrt(G * p / r))
+    assert abs(got[7] - want) < 1e-13 * want
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("u,v", [(np.nan, 1e3), (1e3, np.nan), (np.nan, np.nan), (np.inf, np.inf),
+                                 (np.inf, -np.inf), (1e39, 1e39)])
+def test_nodes_that_are_not_finite(precision, u, v):
+    """A NaN node leaves the largest speed of the others, an infinite one is the largest
+    (1e39 is infinite in FP32)."""
+    st = _at_rest(1.3, 0.7, 1.0, 1.3)
+    st[4 + 1, 3, 5], st[4 + 2, 3, 5] = u, v
+    s = af.Solver(_Grid(40, 33), G, st, precision=precision)
+    out = np.zeros(12)
+    af.af_reduce_invariants(s.handle, out)  # (reports the non-physical centres around it)
+    s.close()
+    want = np.sqrt(G / 0.7)
+    if not (np.isnan(u) or np.isnan(v)):
+        want = np.inf if precision == "fp32" or np.isinf(u) else np.hypot(u, v)
+    # (0.7 is stored as an offset from 1.3 in FP32: half a unit of 2^-24 of 0.6)
+    assert out[7] == want or abs(out[7] - want) < (1e-13 if precision == "fp64" else 1e-7) * want
