@@ -603,16 +603,26 @@ struct AdjBlock {
   static constexpr int BY = sizeof(T) == 4 ? 4 : 2, MINB = sizeof(T) == 4 ? 5 : 1;
 };
 
-// the families by blockIdx.z
+// its blocks per family: 32 columns x BY rows each
+template <typename T>
+inline unsigned adj_acoustic_blocks(int nx, int ny) {
+  constexpr int BY = AdjBlock<T>::BY;
+  return (unsigned)((size_t)((nx + 31) / 32) * ((ny + BY - 1) / BY));
+}
+
+// Blocks of one family along blockIdx.x, row by row (the limit of 65535 on a grid's
+// other dimensions is no limit on the rows); the families by blockIdx.y.
 template <typename T>
 __global__ void __launch_bounds__(32 * AdjBlock<T>::BY, AdjBlock<T>::MINB)
     k_adj_acoustic(const __grid_constant__ AdjView<T> v) {
   pdl_wait();
   // a warp is one row of 32 consecutive nodes (blockDim.x == 32)
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+  const unsigned cols = (unsigned)(v.nx + 31) / 32, br = blockIdx.x / cols;
+  const int i = (int)((blockIdx.x - br * cols) * 32 + threadIdx.x);
+  const int j = (int)(br * AdjBlock<T>::BY + threadIdx.y);
   const unsigned row = __ballot_sync(0xffffffffu, i < v.nx && j < v.ny);
   if (i >= v.nx || j >= v.ny) return;
-  switch (blockIdx.z) {
+  switch (blockIdx.y) {
     case 0: acoustic_adj<0>(v, i, j, row); break;
     case 1: acoustic_adj<1>(v, i, j, row); break;
     case 2: acoustic_adj<2>(v, i, j, row); break;
@@ -928,6 +938,7 @@ inline int choose_adj_geometry(const StepArgs<float>& a, int sms) {
   float best_us = 1e30f;
   for (int g = 0; g < N_ADJ_GEOMS; ++g) {
     const AdjGeometry& q = ADJ_GEOMS[g];
+    if (!tile_rows_fit(a.ny, q.ty)) continue;
     const int64_t tiles = (int64_t)((a.nx + q.tx - 1) / q.tx) * ((a.ny + q.ty - 1) / q.ty);
     const int64_t wave = (int64_t)sms * q.per_sm;
     const float us = (float)((tiles + wave - 1) / wave) * q.us + q.fill;

@@ -614,9 +614,8 @@ af_status adjoint_impl(af_handle* h, double dt, const af_state_f64* lin, const a
   if (e == cudaSuccess && !fused)
     e = launch_dependent(k_adj_points<T>, dim3(ref_blocks(f), 3), REF_THREADS, 0, s, v);
   if (e != cudaSuccess) return cuda_fail(h);
-  constexpr int BY = AdjBlock<T>::BY;
-  launch_dependent(k_adj_acoustic<T>, dim3((h->nx + 31) / 32, (h->ny + BY - 1) / BY, 4),
-                   dim3(32, BY), 0, s, v);
+  launch_dependent(k_adj_acoustic<T>, dim3(adj_acoustic_blocks<T>(h->nx, h->ny), 4),
+                   dim3(32, AdjBlock<T>::BY), 0, s, v);
   launch_dependent(k_adj_center<T>, dim3(ref_blocks(f)), REF_THREADS, 0, s, v);
   // lambda^n out
   AdjOut<T> out;

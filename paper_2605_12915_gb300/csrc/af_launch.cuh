@@ -70,6 +70,11 @@ inline bool encode_tile_maps(const StepArgs<float>& a, TileMaps* out, int ty = F
   return true;
 }
 
+// Whether one CTA per tile of ty rows can be launched: the tile rows are a grid's y
+// dimension, which ends at 65535.  (Only grids of 2 to 16 columns and more than a
+// million rows would choose a tile that does not fit; they get a taller one.)
+inline bool tile_rows_fit(int ny, int ty) { return (ny + (int64_t)ty - 1) / ty <= 65535; }
+
 // One CTA per tile of TX x TY cells.
 template <int TX, int TY, int NT, int MINB, bool COMP>
 inline cudaError_t launch_step_tiles(cudaStream_t s, const StepArgs<float>& a) {
@@ -127,7 +132,7 @@ inline int choose_step_geometry(const StepArgs<float>& a, int sms) {
   float best_us = 1e30f;
   for (int g = 0; g < N_STEP_GEOMS; ++g) {
     const StepGeometry& q = STEP_GEOMS[g];
-    if (q.pipe && !pipe_eligible(a, q.ty)) continue;
+    if (q.pipe ? !pipe_eligible(a, q.ty) : !tile_rows_fit(a.ny, q.ty)) continue;
     const int64_t tiles = (int64_t)((a.nx + q.tx - 1) / q.tx) * ((a.ny + q.ty - 1) / q.ty);
     const float us = (float)((tiles + sms - 1) / sms) * q.us + q.fill;
     if (us < best_us) {
