@@ -908,8 +908,9 @@ inline cudaError_t launch_adj_tiles(cudaStream_t s, const StepArgs<float>& a,
   constexpr auto kern = k_fused_adj<TX, TY, NT, MINB, COMP>;
   const cudaError_t e = allow_smem<kern>(G::SMEM);
   if (e != cudaSuccess) return e;
-  return launch_dependent(kern, dim3((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY), NT, G::SMEM, s,
-                          a, v);
+  // (the first kernel of an adjoint step: launched when the stream's work is done)
+  return launch_kernel(false, kern, dim3((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY), NT, G::SMEM,
+                       s, a, v);
 }
 
 // Tile geometries of the fused reverse sweep, chosen as the step's (STEP_GEOMS):

@@ -71,9 +71,6 @@ struct af_handle {
   cudaEvent_t ev_fork, ev_join, ev_in;
   int late_once;         // testing only (AF_TEST_LATE_WAIT=1 at af_init): the first
                          // pipelined step reports its first staged-tile wait as timed out
-  int after_event;       // 1: the stream was made to wait for another stream's event since
-                         // its last import or export; the next one is launched without
-                         // the programmatic attribute, which speaks of kernels only
   int out_pending;       // 1: the outgoing copies of the last exchange may be in flight
   af_state_f64 pending_out;  // ... into these planes
   // af_exchange_state_async (lazy): two incoming and two outgoing staging
@@ -398,10 +395,10 @@ af_status cuda_fail(af_handle* h) {
 }
 
 // Enqueues the copy of the device error word into the host mirror (read by the
-// next call without waiting).
-af_status flags_to_host(af_handle* h) {
-  return launch_dependent(k_flags_to_host, dim3(1), dim3(32), 0, h->stream, h->d_flags,
-                          h->h_flags_dev) == cudaSuccess
+// next call without waiting).  `dependent`: right after kernels of the same call.
+af_status flags_to_host(af_handle* h, bool dependent) {
+  return launch_kernel(dependent, k_flags_to_host, dim3(1), dim3(32), 0, h->stream, h->d_flags,
+                       h->h_flags_dev) == cudaSuccess
              ? AF_OK
              : AF_ERR_CUDA;
 }
@@ -424,7 +421,9 @@ const void* mapped_host_plane(const af_handle* h, const void* p) {
 
 // Enqueues the conversion of `in` into the current state on the handle's
 // stream (pageable host planes are first copied to the staging buffer); the same
-// kernel clears the error word `flags`, if not null.
+// kernel clears the error word `flags`, if not null.  (Launched, as the export is, when
+// everything before it on the stream is done: it reads the caller's planes, which a
+// copy or another stream may have written.)
 af_status import_enqueue(af_handle* h, const af_state_f64* in, af_memory where,
                          unsigned* flags = nullptr) {
   F64Planes src;
@@ -458,20 +457,18 @@ af_status import_enqueue(af_handle* h, const af_state_f64* in, af_memory where,
   }
   const dim3 g(grid1d(h->N, COPY_THREADS)), t(COPY_THREADS);
   const Offsets o = offsets_of(h);
-  const bool dependent = !h->after_event;
-  h->after_event = 0;
   cudaError_t e = cudaSuccess;
   switch (h->prec) {
     case AF_FP64:
-      e = launch_kernel(dependent, k_import<double, false>, g, t, 0, h->stream, src,
+      e = launch_kernel(false, k_import<double, false>, g, t, 0, h->stream, src,
                            planes_of<double>(h, h->cur), h->N, o, flags);
       break;
     case AF_FP32:
-      e = launch_kernel(dependent, k_import<float, false>, g, t, 0, h->stream, src,
+      e = launch_kernel(false, k_import<float, false>, g, t, 0, h->stream, src,
                            planes_of<float>(h, h->cur), h->N, o, flags);
       break;
     case AF_FP32_COMP:
-      e = launch_kernel(dependent, k_import<float, true>, g, t, 0, h->stream, src,
+      e = launch_kernel(false, k_import<float, true>, g, t, 0, h->stream, src,
                            planes_of<float>(h, h->cur), h->N, o, flags);
       break;
   }
@@ -493,7 +490,6 @@ bool overlaps_pending_out(const af_handle* h, const af_state_f64* in) {
 // on the aux stream (ev_join follows the latest of them).
 af_status wait_outgoing(af_handle* h) {
   if (!(h->out_pending || h->apending[0] || h->apending[1])) return AF_OK;
-  h->after_event = 1;
   return cudaStreamWaitEvent(h->stream, h->ev_join, 0) == cudaSuccess ? AF_OK : cuda_fail(h);
 }
 
@@ -518,20 +514,18 @@ af_status import_state(af_handle* h, const af_state_f64* in, af_memory where) {
 af_status export_enqueue(af_handle* h, const F64Out& dst) {
   const dim3 g(grid1d(h->N, COPY_THREADS)), t(COPY_THREADS);
   const Offsets o = offsets_of(h);
-  const bool dependent = !h->after_event;
-  h->after_event = 0;
   cudaError_t e = cudaSuccess;
   switch (h->prec) {
     case AF_FP64:
-      e = launch_kernel(dependent, k_export<double, false>, g, t, 0, h->stream,
+      e = launch_kernel(false, k_export<double, false>, g, t, 0, h->stream,
                            planes_of<double>(h, h->cur), dst, h->N, o);
       break;
     case AF_FP32:
-      e = launch_kernel(dependent, k_export<float, false>, g, t, 0, h->stream,
+      e = launch_kernel(false, k_export<float, false>, g, t, 0, h->stream,
                            planes_of<float>(h, h->cur), dst, h->N, o);
       break;
     case AF_FP32_COMP:
-      e = launch_kernel(dependent, k_export<float, true>, g, t, 0, h->stream,
+      e = launch_kernel(false, k_export<float, true>, g, t, 0, h->stream,
                            planes_of<float>(h, h->cur), dst, h->N, o);
       break;
   }
@@ -807,7 +801,7 @@ af_status af_step(af_handle* h, double dt, int32_t n_steps) {
     h->cur = 1 - h->cur;
   }
   if (cudaGetLastError() != cudaSuccess) return cuda_fail(h);
-  if (flags_to_host(h) != AF_OK) return cuda_fail(h);
+  if (flags_to_host(h, n_steps > 0) != AF_OK) return cuda_fail(h);
   return AF_OK;
 }
 
@@ -816,7 +810,7 @@ af_status af_sync(af_handle* h) {
   if (h->broken) return AF_ERR_STATE;
   DeviceGuard guard(h->device);
   if (wait_outgoing(h) != AF_OK) return AF_ERR_CUDA;
-  if (flags_to_host(h) != AF_OK || cudaStreamSynchronize(h->stream) != cudaSuccess)
+  if (flags_to_host(h, false) != AF_OK || cudaStreamSynchronize(h->stream) != cudaSuccess)
     return cuda_fail(h);
   h->out_pending = 0;
   h->apending[0] = h->apending[1] = 0;
@@ -942,7 +936,6 @@ af_status af_exchange_state(af_handle* h, const af_state_f64* out, const af_stat
   if (cudaEventRecord(h->ev_join, h->aux) != cudaSuccess ||
       cudaStreamWaitEvent(h->stream, h->ev_in, 0) != cudaSuccess)
     return cuda_fail(h);
-  h->after_event = 1;
   st = import_enqueue(h, &staged, AF_DEVICE, h->d_flags);
   if (st == AF_OK) st = import_finish(h);
   if (st == AF_OK) {
@@ -996,7 +989,6 @@ af_status af_exchange_state_async(af_handle* h, const af_state_f64* out,
   F64Out dst;
   for (int p = 0; p < 16; ++p) dst.p[p] = h->axstage[b] + (size_t)p * N;
   if (cudaStreamWaitEvent(h->stream, h->ev_sent[b], 0) != cudaSuccess) return cuda_fail(h);
-  h->after_event = 1;
   af_status st = export_enqueue(h, dst);
   if (st != AF_OK) return st;
   if (cudaEventRecord(h->ev_exported[b], h->stream) != cudaSuccess ||
@@ -1010,7 +1002,6 @@ af_status af_exchange_state_async(af_handle* h, const af_state_f64* out,
     return cuda_fail(h);
   // the new state, on the handle's stream after the incoming copy
   if (cudaStreamWaitEvent(h->stream, h->ev_staged[b], 0) != cudaSuccess) return cuda_fail(h);
-  h->after_event = 1;
   st = import_enqueue(h, &staged, AF_DEVICE);
   if (st != AF_OK) return st;
   if (cudaEventRecord(h->ev_imported[b], h->stream) != cudaSuccess) return cuda_fail(h);
@@ -1150,14 +1141,15 @@ struct af_batch {
 
 namespace {
 
-af_status batch_launch(af_batch* b, int geom, int parity) {
+// `dependent`: the stream's last operation is another launch of this batch
+af_status batch_launch(af_batch* b, int geom, int parity, bool dependent) {
   const StepArgs<float>* args = b->d_args + (size_t)parity * b->n;
   if (BATCH_GEOMS[geom].pipe && !b->pipe_ok) return AF_ERR_ARG;
   const int kind = geom == 1 && b->use_24x16 ? BATCH_24x16 : geom;
   cudaError_t e = b->prec == AF_FP32_COMP
-                      ? launch_batch<true>(kind, b->stream, args, b->d_tiles[geom], b->ntiles[geom],
-                                           b->d_maps[parity], b->pipe_ctas)
-                      : launch_batch<false>(kind, b->stream, args, b->d_tiles[geom],
+                      ? launch_batch<true>(kind, dependent, b->stream, args, b->d_tiles[geom],
+                                           b->ntiles[geom], b->d_maps[parity], b->pipe_ctas)
+                      : launch_batch<false>(kind, dependent, b->stream, args, b->d_tiles[geom],
                                             b->ntiles[geom], b->d_maps[parity], b->pipe_ctas);
   return e == cudaSuccess ? AF_OK : AF_ERR_CUDA;
 }
@@ -1202,10 +1194,11 @@ af_status batch_tune(af_batch* b) {
     b->tune_ms[g] = -1.f;
     if (BATCH_GEOMS[g].pipe && !b->pipe_ok) continue;
     int parity = batch_parity(b);
-    st = batch_launch(b, g, parity);  // warm-up, attribute set-up
+    st = batch_launch(b, g, parity, false);  // warm-up, attribute set-up
     parity ^= 1;
     cudaEventRecord(e0, b->stream);
-    for (int r = 0; r < 2 && st == AF_OK; ++r, parity ^= 1) st = batch_launch(b, g, parity);
+    for (int r = 0; r < 2 && st == AF_OK; ++r, parity ^= 1)
+      st = batch_launch(b, g, parity, r > 0);
     cudaEventRecord(e1, b->stream);
     cudaEventSynchronize(e1);
     float ms = 0.f;
@@ -1388,7 +1381,8 @@ af_status af_batch_step(af_batch* b, const double* dts, int32_t n_steps) {
     }
     int p = parity;
     af_status st = AF_OK;
-    for (int s = 0; s < n_steps && st == AF_OK; ++s, p ^= 1) st = batch_launch(b, b->geom, p);
+    for (int s = 0; s < n_steps && st == AF_OK; ++s, p ^= 1)
+      st = batch_launch(b, b->geom, p, s > 0);
     cudaError_t e = cudaStreamEndCapture(b->stream, &g);
     if (e != cudaSuccess || st != AF_OK) {
       cudaGetLastError();

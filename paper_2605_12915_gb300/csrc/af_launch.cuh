@@ -97,8 +97,9 @@ inline cudaError_t launch_step_pipe(cudaStream_t s, const StepArgs<float>& a, in
   if (e != cudaSuccess) return e;
   static TileMaps none;
   const int ntiles = ((a.nx + TX - 1) / TX) * ((a.ny + TY - 1) / TY);
-  return launch_dependent(kern, dim3(ntiles < ctas ? ntiles : ctas), NT, G::SMEM_PIPE, s, a,
-                          maps ? *maps : none, maps ? 1 : 0);
+  // (INTER: the first kernel of an adjoint step)
+  return launch_kernel(!INTER, kern, dim3(ntiles < ctas ? ntiles : ctas), NT, G::SMEM_PIPE, s, a,
+                       maps ? *maps : none, maps ? 1 : 0);
 }
 
 // Tile geometries of a lone grid's step.  Results do not depend on the choice
@@ -185,38 +186,41 @@ inline bool batch_prefers_24x16(int64_t n24, int64_t n32, int sms) {
 }
 
 template <int TX, int TY, int NT, int MINB, bool COMP>
-inline cudaError_t launch_batch_geom(cudaStream_t s, const StepArgs<float>* args,
+inline cudaError_t launch_batch_geom(bool dependent, cudaStream_t s, const StepArgs<float>* args,
                                      const int4* tiles, int ntiles) {
   using G = FusedGeom<TX, TY>;
   constexpr auto kern = k_fused_step_batch<TX, TY, NT, MINB, COMP>;
   const cudaError_t e = allow_smem<kern>(G::SMEM);
   if (e != cudaSuccess) return e;
-  return launch_dependent(kern, dim3(ntiles), NT, G::SMEM, s, args, tiles);
+  return launch_kernel(dependent, kern, dim3(ntiles), NT, G::SMEM, s, args, tiles);
 }
 
 // The persistent form: `ctas` CTAs over the tile table; maps (device, one
 // TileMaps per grid) or null for cp.async staging only.
 template <bool COMP>
-inline cudaError_t launch_batch_pipe(cudaStream_t s, const StepArgs<float>* args,
+inline cudaError_t launch_batch_pipe(bool dependent, cudaStream_t s, const StepArgs<float>* args,
                                      const int4* tiles, int ntiles, const TileMaps* maps,
                                      int ctas) {
   using G = FusedGeom<FUSED_TX, FUSED_TY>;
   constexpr auto kern = k_fused_step_batch_pipe<FUSED_TX, FUSED_TY, FUSED_NT, AF_FUSED_MINB, COMP>;
   const cudaError_t e = allow_smem<kern>(G::SMEM_PIPE);
   if (e != cudaSuccess) return e;
-  return launch_dependent(kern, dim3(ntiles < ctas ? ntiles : ctas), FUSED_NT, G::SMEM_PIPE, s,
-                          args, tiles, ntiles, maps);
+  return launch_kernel(dependent, kern, dim3(ntiles < ctas ? ntiles : ctas), FUSED_NT,
+                       G::SMEM_PIPE, s, args, tiles, ntiles, maps);
 }
 
+// `dependent`: the kernel before on the stream is a step of the same batch
 template <bool COMP>
-inline cudaError_t launch_batch(int geom, cudaStream_t s, const StepArgs<float>* args,
-                                const int4* tiles, int ntiles, const TileMaps* maps, int ctas) {
+inline cudaError_t launch_batch(int geom, bool dependent, cudaStream_t s,
+                                const StepArgs<float>* args, const int4* tiles, int ntiles,
+                                const TileMaps* maps, int ctas) {
+  const bool d = dependent;
   switch (geom) {
-    case 0: return launch_batch_geom<32, 32, 512, 1, COMP>(s, args, tiles, ntiles);
-    case 1: return launch_batch_geom<32, 16, 512, 1, COMP>(s, args, tiles, ntiles);
-    case 2: return launch_batch_geom<16, 16, 512, 1, COMP>(s, args, tiles, ntiles);
-    case BATCH_24x16: return launch_batch_geom<24, 16, 256, 2, COMP>(s, args, tiles, ntiles);
-    default: return launch_batch_pipe<COMP>(s, args, tiles, ntiles, maps, ctas);
+    case 0: return launch_batch_geom<32, 32, 512, 1, COMP>(d, s, args, tiles, ntiles);
+    case 1: return launch_batch_geom<32, 16, 512, 1, COMP>(d, s, args, tiles, ntiles);
+    case 2: return launch_batch_geom<16, 16, 512, 1, COMP>(d, s, args, tiles, ntiles);
+    case BATCH_24x16: return launch_batch_geom<24, 16, 256, 2, COMP>(d, s, args, tiles, ntiles);
+    default: return launch_batch_pipe<COMP>(d, s, args, tiles, ntiles, maps, ctas);
   }
 }
 

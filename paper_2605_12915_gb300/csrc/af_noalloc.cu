@@ -130,7 +130,7 @@ extern "C" af_status af_step_noalloc(const af_grid* g, double gamma, double dt, 
   cudaStream_t s = (cudaStream_t)cuda_stream;
   // the work area keeps the previous call's contents: the error word must start at 0
   if (cudaMemsetAsync(a.flags, 0, sizeof(unsigned), s) != cudaSuccess) return AF_ERR_CUDA;
-  if (launch_ref_step<double, false>(a, s) != cudaSuccess) return AF_ERR_CUDA;
+  if (launch_ref_step<double, false>(a, s, false) != cudaSuccess) return AF_ERR_CUDA;
   if (cudaGetLastError() != cudaSuccess) return AF_ERR_CUDA;
   unsigned flags = 0;
   if (cudaMemcpyAsync(&flags, a.flags, sizeof(unsigned), cudaMemcpyDeviceToHost, s) !=
