@@ -1123,7 +1123,9 @@ struct af_batch {
   af_handle** h;
   cudaStream_t stream;
   af_precision prec;
-  StepArgs<float>* h_args;  // pinned host copy [2][n]
+  StepArgs<float>* h_args;  // pinned [2][2][n]: two copies, used by alternate calls
+  cudaEvent_t ev_args[2];   // the device has read copy c (recorded after its transfer)
+  int args_copy;            // copy of the next call
   StepArgs<float>* d_args;  // device [2][n]: parity p = the handles' current buffer
   int4* d_tiles[N_BATCH_GEOMS];
   int ntiles[N_BATCH_GEOMS];
@@ -1294,8 +1296,10 @@ af_status af_batch_init(af_batch** out, int32_t n, const af_grid* grids, double 
     delete[] tt;
   }
   delete[] order;
-  ok = ok && cudaMallocHost(&b->h_args, sizeof(StepArgs<float>) * 2 * n) == cudaSuccess &&
-       cudaMalloc(&b->d_args, sizeof(StepArgs<float>) * 2 * n) == cudaSuccess;
+  ok = ok && cudaMallocHost(&b->h_args, sizeof(StepArgs<float>) * 4 * n) == cudaSuccess &&
+       cudaMalloc(&b->d_args, sizeof(StepArgs<float>) * 2 * n) == cudaSuccess &&
+       cudaEventCreateWithFlags(&b->ev_args[0], cudaEventDisableTiming) == cudaSuccess &&
+       cudaEventCreateWithFlags(&b->ev_args[1], cudaEventDisableTiming) == cudaSuccess;
   if (!ok) {
     af_batch_destroy(b);
     return AF_ERR_ALLOC;
@@ -1352,7 +1356,13 @@ af_status af_batch_step(af_batch* b, const double* dts, int32_t n_steps) {
   }
   if (n_steps == 0) return AF_OK;
   DeviceGuard guard(b->h[0]->device);
-  // step arguments of both parities, with this call's time steps
+  // Step arguments of both parities, with this call's time steps.  The transfer waits on
+  // the stream behind the steps of earlier calls, so the pinned copy is written only
+  // once the device has read what it last held: two copies, so that the call after next
+  // is the first to wait (for the steps before the ones then running).
+  const int c = b->args_copy;
+  StepArgs<float>* args = b->h_args + (size_t)c * 2 * b->n;
+  if (cudaEventSynchronize(b->ev_args[c]) != cudaSuccess) return AF_ERR_CUDA;
   for (int p = 0; p < 2; ++p)
     for (int k = 0; k < b->n; ++k) {
       af_handle* h = b->h[k];
@@ -1361,11 +1371,13 @@ af_status af_batch_step(af_batch* b, const double* dts, int32_t n_steps) {
       StepArgs<float> a = step_args<float>(h, dts[k]);
       a.prefetch_wave = 0;
       h->cur = cur;
-      b->h_args[(size_t)p * b->n + k] = a;
+      args[(size_t)p * b->n + k] = a;
     }
-  if (cudaMemcpyAsync(b->d_args, b->h_args, sizeof(StepArgs<float>) * 2 * b->n,
-                      cudaMemcpyHostToDevice, b->stream) != cudaSuccess)
+  if (cudaMemcpyAsync(b->d_args, args, sizeof(StepArgs<float>) * 2 * b->n,
+                      cudaMemcpyHostToDevice, b->stream) != cudaSuccess ||
+      cudaEventRecord(b->ev_args[c], b->stream) != cudaSuccess)
     return AF_ERR_CUDA;
+  b->args_copy = 1 - c;
   if (b->geom < 0) {
     af_status st = batch_tune(b);
     if (st != AF_OK) return st;
@@ -1438,6 +1450,8 @@ void af_batch_destroy(af_batch* b) {
     if (b->d_maps[p]) cudaFree(b->d_maps[p]);
   if (b->d_args) cudaFree(b->d_args);
   if (b->h_args) cudaFreeHost(b->h_args);
+  for (int c = 0; c < 2; ++c)
+    if (b->ev_args[c]) cudaEventDestroy(b->ev_args[c]);
   if (b->snapshot) cudaFree(b->snapshot);
   if (b->h) {
     for (int k = 0; k < b->n; ++k) af_destroy(b->h[k]);

@@ -104,3 +104,23 @@ def test_ensemble_workload_members_fp32_vs_fp64():
         assert err < 2e-5, (k, err)
     print("ensemble members, 200 steps, batched fp32 vs fp64 rel Linf", worst)
     b.close()
+
+
+def test_queued_calls_keep_their_own_time_steps():
+    """Calls queued without a wait behind a long one, each with other time steps: each
+    steps with its own (bitwise the lone handles given the same sequence)."""
+    probs = [I.random_smooth(64 + 8 * k, 48, seed=k, amp=0.05) for k in range(3)]
+    b = af.Batch(probs, precision="fp32")
+    b.step([p.dt for p in probs], 1)  # (tunes, and waits)
+    b.sync()
+    calls = [(1.0, 600)] + [(f, 1) for f in (0.5, 0.25, 0.75, 0.125, 0.9, 0.3)]
+    for f, n in calls:
+        b.step([f * p.dt for p in probs], n)
+    for k, p in enumerate(probs):
+        s = af.Solver(p.grid, p.gamma, p.state, precision="fp32")
+        s.step(p.dt, 1)
+        for f, n in calls:
+            s.step(f * p.dt, n)
+        assert np.array_equal(b.state(k), s.state()), k
+        s.close()
+    b.close()
