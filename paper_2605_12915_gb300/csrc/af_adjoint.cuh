@@ -527,9 +527,8 @@ __device__ __forceinline__ void acoustic_adj(const AdjView<T>& v, int i, int j, 
   for (int s = 0; s < 2; ++s) zero4(v.lam + (size_t)(LAM_INC + 4 * (4 * s + FAM)) * ps + 4 * id);
   const Prim<T> wk = node_w(v, FAM, id);
   const T rk = with_ref(v.gas.rho_ref, wk.r), pk = with_ref(v.gas.p_ref, wk.p);
-  // Z^2 = gamma p rho, c = gamma p / Z
-  const T gp = v.gas.gamma * pk, z2 = gp * rk;
-  const T Zinv = rsqrt_t(z2), Z = z2 * Zinv, c = gp * Zinv;
+  T c, Z, Zinv;
+  freeze(v.gas.gamma, rk, pk, c, Z, Zinv);
   const T dth = v.dth;
   const T r1 = c * dth;
   T Gp[3][4], Guv[3][4];
@@ -584,9 +583,9 @@ __device__ __forceinline__ void acoustic_adj(const AdjView<T>& v, int i, int j, 
   }
   lZ = fma(-lZinv * Zinv, Zinv, lZ);
   // c^2 = gamma p / rho: dc/drho = -c / (2 rho), dc/dp = c / (2 p) = gamma / (2 Z)
-  const T lc = fma(dth, lr1, rk * lZ), hz = T(0.5) * Zinv;
-  const T lrho = fma(c, lZ, -lc * (c * c) * hz);  // c / rho = c^2 / Z
-  const T lp = lc * (v.gas.gamma * hz);
+  const T lc = fma(dth, lr1, rk * lZ), hc = T(0.5) * lc;
+  const T lrho = fma(c, lZ, -hc * c / rk);
+  const T lp = hc * (v.gas.gamma * Zinv);
   T lpK = T(0), luK = T(0), lvK = T(0);
   const ScatterAdj<FAM, T> S = {v.lam, v.ps, nb, act};
   sac_family_adj<FAM, T>(S, lGp, lGuv, lpK, luK, lvK);

@@ -85,9 +85,6 @@ __device__ __forceinline__ bool is_negative(double x) {
 __device__ __forceinline__ bool at_least_one(float x) { return x >= 1.f; }
 __device__ __forceinline__ bool at_least_one(double x) { return __double2hiint(x) >= 0x3ff00000; }
 
-__device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsqrt_t(double x) { return rsqrt(x); }
-
 // (float)x and (double)x on the integer units (the conversion instructions run at
 // the FP64 unit's rate): the exponent is rebiased and the mantissa shifted, with
 // round to nearest even on narrowing.  Same values as the instructions, subnormals,

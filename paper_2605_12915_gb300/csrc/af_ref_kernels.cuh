@@ -13,7 +13,7 @@
 // (loads, integer work, launches of other warps) is all but free.  Comparisons,
 // conversions, floor and min / max of doubles run on that unit too.  So the FP64
 // instructions are what is counted here: comparisons and floor are done on the
-// bits, 1/Z and c come from one reciprocal square root, increments are kept as
+// bits, increments are kept as
 // (u + du, v + dv, dp) and interpolated together with the velocity (five fields
 // at the foot instead of seven), the nine Q2 weights are formed once, and each
 // node's fluxes are integrated in time once instead of in both edges it bounds.
@@ -205,6 +205,17 @@ __device__ __forceinline__ void sac_family(const Load& L, T pK, T uK, T vK, T Gp
   if constexpr (FAM == 3) af_sac_C<T>(L, pK, uK, vK, Gp, Guv);
 }
 
+// The frozen sound speed c = sqrt(gamma p / rho), impedance Z = rho c and 1 / Z of a
+// node, each rounded by IEEE operations.  (One reciprocal root, 1/Z =
+// rsqrt(gamma p rho), saves the root and two divisions but doubles the error of c and
+// leaves the exponent range where p rho does.)
+template <typename T>
+__device__ __forceinline__ void freeze(T gamma, T rho, T p, T& c, T& Z, T& Zinv) {
+  c = sqrt(gamma * p / rho);
+  Z = rho * c;
+  Zinv = T(1) / Z;
+}
+
 template <int FAM, typename T>
 __device__ __forceinline__ void acoustic_node(const StepArgs<T>& a, int i, int j, size_t id) {
   T* const* own = FAM < 3 ? a.in.pt[FAM < 3 ? FAM : 0] : a.wc;
@@ -212,9 +223,8 @@ __device__ __forceinline__ void acoustic_node(const StepArgs<T>& a, int i, int j
   unsigned bad = 0;
   const T rk = with_ref(a.gas.rho_ref, wk.r), pk = with_ref(a.gas.p_ref, wk.p);
   if (!(is_positive(rk) && is_positive(pk))) bad |= FLAG_NONPHYSICAL;
-  // Z^2 = gamma p rho, c = gamma p / Z
-  const T gp = a.gas.gamma * pk, z2 = gp * rk;
-  const T Zinv = rsqrt_t(z2), Z = z2 * Zinv, c = gp * Zinv;
+  T c, Z, Zinv;
+  freeze(a.gas.gamma, rk, pk, c, Z, Zinv);
   const T r1 = c * a.dth;
   if (abs_above(r1, T(0.5))) bad |= FLAG_CFL;
   T Gp[3][4], Guv[3][4];

@@ -46,3 +46,36 @@ def test_centre_recovery_rounds_the_deviations_only():
         D = 0.07
         assert abs(Fraction(got) - exact) <= EPS * (1.0 + 5.4 * D)
     solver.close()
+
+
+def _scaling(a, b):
+    """Factors of the sixteen planes for density times 2^a and pressure times 2^b, hence
+    velocities times 2^((b - a) / 2)."""
+    r, p, w = 2.0 ** a, 2.0 ** b, 2.0 ** ((b - a) // 2)
+    return np.array([r, r * w, r * w, p] + 3 * [r, w, w, p])[:, None, None]
+
+
+@pytest.mark.parametrize("variant", ["tai", "rb"])
+@pytest.mark.parametrize("a,b,s", [(550, 480, 440), (200, 150, 0), (-100, 60, 0)])
+def test_fp64_step_and_adjoint_scale_exactly(a, b, s, variant):
+    """The same flow in other units, every factor a power of two (lambda's common one is
+    2^s): all operations commute with it, so the step scales bitwise and the adjoint up to
+    the order of its atomic sums.  In the first case the product of density and pressure
+    leaves FP64's range; no value of the frozen coefficients does, nor, the variations
+    being small, the products of the pressure increments with the density."""
+    from workloads import inputs as I
+    P = I.random_smooth(24, 19, seed=5, amp=1e-7)
+    f = _scaling(a, b)
+    dt = P.dt * (0.6 if variant == "rb" else 1.0)
+    lam = np.random.default_rng(3).normal(size=P.state.shape)
+    out = []
+    for st, l, t in ((P.state, lam, dt),
+                     (P.state * f, lam / f * 2.0 ** s, dt * 2.0 ** ((a - b) // 2))):
+        h = af.Solver(P.grid, P.gamma, st, precision="fp64", variant=variant)
+        l = h.adjoint(t, l)
+        h.step(t, 3)
+        out.append((h.state(), l))
+        h.close()
+    assert np.array_equal(out[1][0], out[0][0] * f)
+    got = out[1][1] * f * 2.0 ** -s
+    assert np.max(np.abs(got - out[0][1])) < 1e-13 * np.max(np.abs(out[0][1]))
