@@ -34,7 +34,7 @@ struct StepArgs {
   Planes<T> in;       // state at t^n
   Planes<T> out;      // state at t^{n+1}
   T* wc[4];           // recovered centre (rho, u, v, p)
-  T* inc[2][4][3];    // [tau index][family V,Ev,Eh,C][u + du, v + dv, dp]
+  T* inc[2][4][3];    // [tau index][family V,Ev,Eh,C][u + du, v + dv, dp] (RB: du, dv, dp)
   T* half[3][4];      // point values at t^n + dt/2, [family][rho,u,v,p] (adjoint and AF_FC);
                       // the step keeps the fluxes of the vertices (x, then y) and of the
                       // x-edge midpoints there
@@ -238,11 +238,14 @@ __device__ __forceinline__ void acoustic_node(const StepArgs<T>& a, int i, int j
     cu[q] = fma(Zinv, Gp[1][q], Guv[1][q]);
     cv[q] = fma(Zinv, Gp[2][q], Guv[2][q]);
   }
+  // (the additive update takes the increments at the point itself, without interpolation:
+  // kept alone there, they do not carry a rounding of the velocity)
+  const T u0 = a.variant == 0 ? wk.u : T(0), v0 = a.variant == 0 ? wk.v : T(0);
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
     const T r = s == 0 ? T(0.5) * r1 : r1;
-    a.inc[s][FAM][0][id] = fma(r, fma(r, fma(r, fma(r, cu[3], cu[2]), cu[1]), cu[0]), wk.u);
-    a.inc[s][FAM][1][id] = fma(r, fma(r, fma(r, fma(r, cv[3], cv[2]), cv[1]), cv[0]), wk.v);
+    a.inc[s][FAM][0][id] = fma(r, fma(r, fma(r, fma(r, cu[3], cu[2]), cu[1]), cu[0]), u0);
+    a.inc[s][FAM][1][id] = fma(r, fma(r, fma(r, fma(r, cv[3], cv[2]), cv[1]), cv[0]), v0);
     a.inc[s][FAM][2][id] = r * fma(r, fma(r, fma(r, cp[3], cp[2]), cp[1]), cp[0]);
   }
   raise_flag(a.flags, bad);
@@ -444,8 +447,8 @@ __device__ __forceinline__ void point_node(const StepArgs<T>& a, int i, int j, s
       // additive update: S_ac(P) + S_adv(P) - W(P), acoustic rho closure at P
       const T dp = a.inc[s][FAM][2][id];
       nw.r = rft + dp * with_ref(g.rho_ref, wp.r) / (g.gamma * with_ref(g.p_ref, wp.p));
-      nw.u = nine_sum(c, w, plane(1)) + (a.inc[s][FAM][0][id] - wp.u);
-      nw.v = nine_sum(c, w, plane(2)) + (a.inc[s][FAM][1][id] - wp.v);
+      nw.u = nine_sum(c, w, plane(1)) + a.inc[s][FAM][0][id];
+      nw.v = nine_sum(c, w, plane(2)) + a.inc[s][FAM][1][id];
       nw.p = pft + dp;
     }
     if (!(is_finite(nw.r) && is_finite(nw.u) && is_finite(nw.v) && is_finite(nw.p)))

@@ -1,6 +1,9 @@
 """Rounding of the FP64 path's building blocks, each against exact arithmetic (rational
 numbers, or binary scalings that must commute with every operation), with bounds counted
 from the operations' own roundings (2^-53 of each result)."""
+import ctypes
+import os
+import subprocess
 from fractions import Fraction
 
 import numpy as np
@@ -79,3 +82,65 @@ def test_fp64_step_and_adjoint_scale_exactly(a, b, s, variant):
     assert np.array_equal(out[1][0], out[0][0] * f)
     got = out[1][1] * f * 2.0 ** -s
     assert np.max(np.abs(got - out[0][1])) < 1e-13 * np.max(np.abs(out[0][1]))
+
+
+@pytest.fixture(scope="module")
+def extended_step(tmp_path_factory):
+    """The oracle's step with long double (64 or 113 bits of mantissa) for double."""
+    import oracle
+    tmp = tmp_path_factory.mktemp("extended")
+    src, lib = str(tmp / "extended.c"), str(tmp / "extended.so")
+    path = os.path.join(os.path.dirname(oracle.__file__), "af_oracle.c")
+    with open(src, "w") as f:
+        f.write("#include <complex.h>\n#include <math.h>\n#include <stdlib.h>\n"
+                "#include <string.h>\n#include <tgmath.h>\n#undef M_PI\n"
+                "#define M_PI 3.14159265358979323846264338327950288L\n"
+                "#define double long double\n#include \"%s\"\n" % path)
+    subprocess.check_call(["gcc", "-O2", "-std=gnu11", "-ffp-contract=off", "-fPIC", "-shared",
+                           "-o", lib, src, "-lm"])
+    fn = ctypes.CDLL(lib).orc_step
+    i, d = ctypes.c_int, ctypes.c_longdouble
+    fn.argtypes = [i, i, d, d, d, i, ctypes.c_void_p, ctypes.c_void_p]
+
+    def step(state, h, gamma, dt, variant):
+        a = np.ascontiguousarray(state, dtype=np.longdouble)
+        out = np.empty_like(a)
+        fn(a.shape[2], a.shape[1], h, gamma, dt, variant, a.ctypes.data, out.ctypes.data)
+        return out
+
+    return step
+
+
+def test_additive_update_adds_the_increment_to_the_foot_value(extended_step):
+    """u = u_f + du with u_f exact: on the row of one vertex u is 1.0625 there, 0.75 at the
+    edge midpoint before it and 0.25 at the vertex before that; with dt / h = 1/2 both
+    Picard stages have short dyadic coordinates and u_f = 0.85 without a rounding.  du is
+    small (c dt / h = 2^-11), so its own roundings are far below those of u, except that the
+    recovered centre pressures around the vertex are rounded as parts of an energy of 1/2:
+    2^-54 each, times dt / h / rho and the stencil's weights, 0.2 x 2^-54 or so.  What is
+    left is the rounding of the sum, half a unit in the last place of [0.5, 1) = 2^-54.
+    (du recovered from 1.0625 + du would add that of [1, 2), twice as much.)"""
+    rng = np.random.default_rng(5)
+    nx, ny, gamma, dt = 6, 5, 1.4, 0.5
+    worst = 0.0
+    for _ in range(60):
+        st = np.zeros((16, ny, nx))
+        for b in (4, 8, 12):
+            st[b], st[b + 1] = 1.0, 0.75
+            st[b + 3] = 2.0 ** -20 / gamma * rng.uniform(1.0, 1.1, (ny, nx))
+        st[5, 2, 3], st[5, 2, 2] = 1.0625, 0.25
+        roll = lambda a, dy, dx: np.roll(a, (-dy, -dx), (0, 1))
+        cons = [[w[0], w[0] * w[1], 0 * w[0], w[3] / (gamma - 1) + 0.5 * w[0] * w[1] ** 2]
+                for w in (st[4:8], st[8:12], st[12:16])]
+        for k, c in enumerate((1.0, 0.75, 0.0, 2.0 ** -20 / gamma / (gamma - 1) + 0.5 * 0.75 ** 2)):
+            V, X, Y = (q[k] for q in cons)
+            st[k] = 4 / 9 * (c + (V + roll(V, 0, 1) + roll(V, 1, 0) + roll(V, 1, 1)) / 16 +
+                             (X + roll(X, 0, 1) + Y + roll(Y, 1, 0)) / 4)
+        s = af.Solver(_Grid(nx, ny), gamma, st, precision="fp64", variant="rb")
+        s.step(dt, 1)
+        got = s.state()[5, 2, 3]
+        s.close()
+        want = extended_step(st, 1.0, gamma, dt, 1)[5, 2, 3]
+        assert 0.8 < got < 0.9
+        worst = max(worst, float(abs(got - want)))
+    assert worst <= 1.4 * EPS / 2
