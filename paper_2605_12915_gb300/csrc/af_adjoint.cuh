@@ -319,10 +319,10 @@ __device__ __forceinline__ void point_adj(const AdjView<T>& v, int i, int j, siz
     T w[9];
 #pragma unroll
     for (int m = 0; m < 9; ++m) w[m] = lx[m % 3] * lyb[m / 3];
-    const T rft = nine_sum(nf, w, wplane(0)), pft = nine_sum(nf, w, wplane(3));
+    const T rft = row_sum(nf, lx, lyb, wplane(0)), pft = row_sum(nf, lx, lyb, wplane(3));
     T lwf[4], ldp = T(0);  // adjoints of W_f and of the interpolated dp (du, dv: lwf[1], lwf[2])
     if (v.variant == 0) {
-      const T d2 = nine_sum(nf, w, iplane(2));
+      const T d2 = row_sum(nf, lx, lyb, iplane(2));
       const T rf = with_ref(g.rho_ref, rft), pf = with_ref(g.p_ref, pft);
       const T igp = T(1) / (g.gamma * pf);
       const T a0 = ly[0] * igp;
