@@ -7,7 +7,7 @@
 // What bounds them: the FP64 unit (two lanes per cycle and SM).  A cell took about
 // 575 of its instructions: ten CUDA logarithms, eight square roots and seven
 // divisions, 32 conversions, minima and maxima.  It takes 160 now: the
-// logarithm by a table (7 instructions, below), conversions on the integer units,
+// logarithm by a table (8 instructions, below), conversions on the integer units,
 // the minima on the stored floats, the wave speed evaluated in FP64 only where its
 // FP32 value comes near the grid's largest one, which the centre recovery before it
 // finds; common factors taken out of the sums.
@@ -17,6 +17,7 @@
 #pragma once
 
 #include "af_common.cuh"
+#include "af_log_table.cuh"
 #include "af_ref_kernels.cuh"
 
 namespace af {
@@ -38,41 +39,44 @@ struct RedArgs {
 
 // ---- logarithm by table (P. T. P. Tang, "Table-driven implementation of the
 // logarithm function in IEEE floating-point arithmetic", ACM TOMS 16, 1990) ----
-// x = 2^e m with m in [0.707, 1.414); c the nearest of 512 points (nine bits of
-// m), g = 1/c rounded, r = g m - 1 (one rounding, |r| <= 2^-10): log x = e log 2 -
-// log g + log(1 + r), the last by its series.  The terms from r^4 on are below
-// 2^-30 of r and are summed in FP32; everything else in FP64.  Around x = 1, e = 0
-// and the point nearest to 1 is 1 itself (log g = 0), so small results keep their
-// relative accuracy (2 ulp measured over 1e-9 < |log x| < 20).
-constexpr int LOG_POINTS = 512;
-constexpr unsigned LOG_FIRST = 0x3fe6a000u;  // high word of the first point, 0.70703
-struct LogEntry {
-  double g, mlog_g;  // 1/c and -log(g)
+// x = 2^e m with m in [0.707, 1.414); c the nearest of 512 points (nine bits of m), g
+// near 1/c, r = g m - 1 (|r| < 2^-9.8): log x = e log 2 - log g + log(1 + r), the last by
+// its series.  The leading part e log 2 - log g is exact (both terms are multiples of
+// 2^-42, what they leave is a float, gen_log_table.py); the terms from r^4 on, below 2^-31
+// of r, and the sum of the left-over parts are FP32; everything else is FP64.  At the point
+// next to 1, which is 1 itself, log g = 0 and small results keep their relative
+// accuracy.  Error 1.03 ulp at most (where the sum crosses a power of two next to 1) and
+// 0.27 rms; CUDA's log has 0.54 and 0.25; with the leading part rounded it was 1.8 and
+// 0.44.  The entropies, sums of 3200 cells, are within 2.1 (nodes) and 3.0 (averages)
+// units of 2^-53 rms of extended precision; with CUDA's log they were within 2.5 and 3.1.
+struct LogTable {
+  LogEntry e[LOG_POINTS];
+  float lo[LOG_POINTS];
 };
-__device__ __forceinline__ void fill_log_table(LogEntry* tab, int thread, int threads) {
+__device__ __forceinline__ void fill_log_table(LogTable& tab, int thread, int threads) {
   for (int i = thread; i < LOG_POINTS; i += threads) {
-    const double g = 1.0 / __hiloint2double((int)(LOG_FIRST + ((unsigned)i << 11)), 0);
-    tab[i].g = g;
-    tab[i].mlog_g = -log(g);
+    tab.e[i] = LOG_TABLE[i];
+    tab.lo[i] = LOG_TABLE_LO[i];
   }
 }
-__device__ __forceinline__ double log_by_table(double x, const LogEntry* tab) {
+__device__ __forceinline__ double log_by_table(double x, const LogTable& tab) {
   const unsigned hi = (unsigned)__double2hiint(x);
   if (hi - 0x00100000u >= 0x7fe00000u) return log(x);  // not a positive normal number
   const unsigned t = hi - LOG_FIRST + 0x400u;  // (+ half a point: the nearest one)
-  const int e = (int)t >> 20;
-  const LogEntry c = tab[(t & 0xfffffu) >> 11];
+  const int e = (int)t >> 20, i = (int)((t & 0xfffffu) >> 11);
+  const LogEntry c = tab.e[i];
   const double m = __hiloint2double((int)(hi - ((unsigned)e << 20)), __double2loint(x));
   const double r = fma(m, c.g, -1.0);
-  const double head = fma(widen((float)e), 0.69314718055994530942, c.mlog_g);
-  const float rf = narrow(r);
+  const float ef = (float)e, rf = narrow(r);
+  const double head = fma(widen(ef), LOG_2_HI, c.hi);  // exact
+  const float lo = fmaf(ef, LOG_2_LO, tab.lo[i]);
   const float tail = fmaf(rf, fmaf(rf, -1.0f / 6.0f, 0.2f), -0.25f);
   const double q = fma(r, fma(r, widen(tail), 1.0 / 3.0), -0.5);
-  return head + fma(r * r, q, r);
+  return head + (r + fma(r * r, q, widen(lo)));
 }
 
 __device__ __forceinline__ double entropy_density(double r, double p, double gamma,
-                                                  const LogEntry* tab) {
+                                                  const LogTable& tab) {
   return r * fma(gamma, log_by_table(r, tab), -log_by_table(p, tab));
 }
 
@@ -104,7 +108,7 @@ __device__ __forceinline__ double wave_speed(double r, double u, double v, doubl
 
 template <typename T, bool COMP>
 __global__ void __launch_bounds__(RED_THREADS) k_inv_partial(const __grid_constant__ RedArgs<T> a) {
-  __shared__ LogEntry tab[LOG_POINTS];
+  __shared__ LogTable tab;
   __shared__ double sh[RED_WARPS][RED_VALS];
   fill_log_table(tab, threadIdx.x, RED_THREADS);
   __syncthreads();

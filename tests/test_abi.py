@@ -120,6 +120,12 @@ def test_committed_stencils_match_generator(tmp_path):
     assert out.read_text() == open(STENCILS).read()
 
 
+def test_committed_log_table_matches_generator(tmp_path):
+    out = tmp_path / "af_log_table.cuh"
+    subprocess.check_call(["python", os.path.join(CSRC, "gen_log_table.py"), str(out)])
+    assert out.read_text() == open(os.path.join(CSRC, "af_log_table.cuh")).read()
+
+
 # ---- apply the generated tables on the CPU ---------------------------------
 def parse_stencils():
     """{family: [(a, b, combo, field, dst, o, q, value)]} from the generated code."""

@@ -170,3 +170,28 @@ def test_nodes_that_are_not_finite(precision, u, v):
         want = np.inf if precision == "fp32" or np.isinf(u) else np.hypot(u, v)
     # (0.7 is stored as an offset from 1.3 in FP32: half a unit of 2^-24 of 0.6)
     assert out[7] == want or abs(out[7] - want) < (1e-13 if precision == "fp64" else 1e-7) * want
+
+
+def test_logarithm_rounding():
+    """Uniform states with gamma = 2, p = 1 and h = 1: the averages' entropy is
+    4 fl(rho 2 log rho) exactly (log 1 = 0, sums of four equal terms).  Modelled on the CPU,
+    a correctly rounded logarithm and the table's with its exact leading part both give it
+    an rms error of 0.371 units in the last place, the table's with a rounded leading part
+    0.568; the rms of 3000 errors varies by 1.3%."""
+    class Unit:
+        nx, ny, h = 2, 2, 1.0
+    rng = np.random.default_rng(6)
+    st = np.ones((16, 2, 2))
+    st[[1, 2, 5, 6, 9, 10, 13, 14]] = 0.0
+    s, err = None, []
+    for rho in np.concatenate([np.exp(rng.uniform(-20, 20, 1500)), rng.uniform(0.5, 2.0, 1500)]):
+        st[[0, 4, 8, 12]] = rho
+        if s is None:
+            s = af.Solver(Unit, 2.0, st, precision="fp64")
+        else:
+            s.set_state(st)
+        want = np.longdouble(rho) * 2 * np.log(np.longdouble(rho))
+        ulp = np.spacing(abs(np.float64(want)))
+        err.append(float((np.longdouble(s.invariants()[5] / 4) - want) / ulp))
+    s.close()
+    assert np.sqrt(np.mean(np.square(err))) < 0.44
