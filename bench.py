@@ -117,9 +117,10 @@ PROFILE = "profiles/k_fused_step_pipe_shear2048_fp32comp.md"
 def fused_kernel_name(nx, ny):
     """The FP32 step kernel the library launches for an nx x ny grid of the
     benchmark's sizes: the persistent pipelined kernel when the grid allows it, holds
-    more than one wave of 32 x 32 tiles (152 SMs) and AF_PIPE is not 0."""
+    more than one wave of 32 x 24 tiles (152 SMs; smaller grids choose tiles of their own)
+    and AF_PIPE is not 0."""
     if (os.environ.get("AF_PIPE") == "0" or nx % 4 or nx < 40 or ny < 38 or
-            (nx * ny <= 152 * 32 * 32 and "AF_PIPE" not in os.environ)):
+            (-(-nx // 32) * -(-ny // 24) <= 152 and "AF_PIPE" not in os.environ)):
         return "k_fused_step"
     return "k_fused_step_pipe"
 
