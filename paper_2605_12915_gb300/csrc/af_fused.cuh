@@ -408,6 +408,8 @@ __device__ __forceinline__ float4 tm_load(unsigned addr) {
 // Allocation and release by warp 0; `slot`: a shared word for the base address, which
 // every thread returns after the barrier inside.  (No kernel here holds more than half
 // of the columns, so a CTA of the next kernel can allocate while this one drains.)
+// (With no columns there is no barrier either: the persistent kernels, whose mbarrier
+// it publishes as well, check that they have some.)
 template <int COLS>
 __device__ __forceinline__ unsigned tm_alloc(unsigned* slot) {
   if constexpr (COLS == 0) return 0u;
@@ -1156,6 +1158,7 @@ __global__ void __launch_bounds__(NT, MINB)
     k_fused_step_pipe(const __grid_constant__ StepArgs<float> a,
                       const __grid_constant__ TileMaps tm, int use_tma) {
   using G = FusedGeom<TX, TY>;
+  static_assert(tm_cols<TX, TY, NT>() > 0, "the barrier after mbarrier.init is tm_alloc's");
   extern __shared__ __align__(16) float4 smem4[];
   float* S = reinterpret_cast<float*>(smem4 + 4 * G::WPL);
   PipeCtx pc;
@@ -1214,6 +1217,7 @@ __global__ void __launch_bounds__(NT, MINB)
                             const int4* __restrict__ tiles, int ntiles,
                             const TileMaps* __restrict__ maps) {
   using G = FusedGeom<TX, TY>;
+  static_assert(tm_cols<TX, TY, NT>() > 0, "the barrier after mbarrier.init is tm_alloc's");
   extern __shared__ __align__(16) float4 smem4[];
   float* S = reinterpret_cast<float*>(smem4 + 4 * G::WPL);
   const bool tma = maps && G::W_BYTES % 128 == 0 && (smem_addr(smem4) & 127u) == 0;
