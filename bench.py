@@ -143,8 +143,10 @@ def fused_source_hash():
 
 
 def profiled_traffic(n_cells):
-    """DRAM bytes per launch of the fused kernel from the committed ncu summary,
-    scaled to n_cells; None if the kernel source changed since the capture."""
+    """DRAM bytes per launch of the fused kernel from the committed ncu summary (steps
+    one after another, so that each launch also writes back what the one before left in
+    L2), scaled to n_cells; None if the kernel source changed since the capture, or for
+    fewer cells than captured, whose state L2 may hold in part."""
     try:
         kv = {}
         with open(os.path.join(ROOT, PROFILE)) as f:
@@ -154,7 +156,10 @@ def profiled_traffic(n_cells):
                     kv[k.strip()] = v.strip()
         if kv.get("kernel_source_sha256_16") != fused_source_hash():
             return None
-        return float(kv["traffic_bytes_per_launch"]) * n_cells / float(kv["cells_per_launch"])
+        cells = float(kv["cells_per_launch"])
+        if n_cells < cells:
+            return None
+        return float(kv["traffic_bytes_per_launch"]) * n_cells / cells
     except Exception:
         return None
 

@@ -50,6 +50,14 @@ def test_recorded_traffic_scales_to_a_launch(monkeypatch):
     assert abs(bench.profiled_traffic(2 * 4194304) - 2 * full) < 1e-6 * full
 
 
+def test_recorded_traffic_is_the_whole_of_a_step(monkeypatch):
+    """A step of a state larger than L2 reads and writes twenty planes: 160 B per cell
+    (0.5% for the counters), none of them left out because it was still in L2."""
+    monkeypatch.setattr(bench, "fused_source_hash", _recorded_hash)
+    assert bench.profiled_traffic(4194304) >= 0.995 * 160 * 4194304
+    assert bench.profiled_traffic(512 * 512) is None
+
+
 def test_recorded_traffic_is_dropped_when_the_kernel_changed(monkeypatch):
     monkeypatch.setattr(bench, "fused_source_hash", lambda: "0" * 16)
     assert bench.profiled_traffic(4194304) is None
