@@ -103,10 +103,11 @@ ALU_OPS_PER_CELL = 2365
 # plain FP32 averages: the compensated update (148) is replaced by four
 # three-term updates of the averages (16)
 ALU_OPS_PER_CELL_PLAIN = 2365 - 148 + 16
-# the FP64 step (kernels per stage): centre recovery 98 (direct form), freezing 24,
-# stencils 695, increment mixing and Horner 148, six point updates of 109 (increments
-# interpolated with the velocity), node fluxes over time 156, average update 48
-FP64_OPS_PER_CELL = 1823
+# the FP64 step (kernels per stage): centre recovery 131 (deviation form), freezing 24,
+# stencils 695, increment mixing and Horner 148, six point updates of 114 (seven fields
+# by rows, the increments interpolated with the velocity), node fluxes over time 156,
+# average update 48
+FP64_OPS_PER_CELL = 1886
 FUSED_SOURCES = ["paper_2605_12915_gb300/csrc/af_fused.cuh",
                  "paper_2605_12915_gb300/csrc/af_common.cuh",
                  "paper_2605_12915_gb300/csrc/af_stencils.cuh",
