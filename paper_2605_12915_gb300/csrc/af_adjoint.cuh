@@ -595,7 +595,8 @@ __device__ __forceinline__ void acoustic_adj(const AdjView<T>& v, int i, int j, 
 // Blocks of the acoustic adjoint: BY rows of 32 consecutive nodes.  FP32 waits on
 // scattered loads and atomics, and the vertex family spills below 96 registers: 128
 // threads, five blocks per SM (adjoint step at 2048^2 2.89 ms; three of 256 threads at
-// 80 registers 2.94, two at 128 2.98, four of 128 or of 192 2.95 and 2.93).  FP64 is bound
+// 80 registers 2.94, two at 128 2.98, four of 128 or of 192 2.95 and 2.93; measured with
+// one reciprocal root for the freezing, with IEEE operations the chosen one takes 2.98).  FP64 is bound
 // by its arithmetic unit and would spill: two warps, registers as needed.
 template <typename T>
 struct AdjBlock {
@@ -672,7 +673,7 @@ __global__ void __launch_bounds__(REF_THREADS) k_adj_center(const __grid_constan
 // Fused reverse sweep of a tile (FP32 modes).  fused_tile<..., ADJ> leaves the
 // tile's time-n nodes W and the increments D of both durations in shared
 // memory.  For each owned point: the adjoint of the space-time Simpson fluxes
-// it enters (gathered from the averages' lambda, as k_adj_flux), then the
+// it enters (gathered from the averages' lambda, point_fluxes_adj), then the
 // adjoint of its point update for both durations (as k_adj_points) with the
 // forward values taken from shared memory and the foot traced as the fused
 // step traces it (displacements clamped to one cell).  Results go to the node
@@ -755,7 +756,9 @@ __device__ __forceinline__ void tile_reverse(const StepArgs<float>& a, const Adj
       if (a.variant == 0) {
         const float d2 = q2_eval<DCW>(Ds + 2 * DPL, Ds + 5 * DPL, Ds + 8 * DPL, Ds + 11 * DPL,
                                       dcf, lx, lyb);
-        // (fast reciprocals, as the forward closure's division)
+        // (fast reciprocals, as the forward closure's division: with IEEE divisions and
+        // roots throughout the sweep the errors against FP64 are the same to 1%, 1024^2
+        // takes 809 us instead of 790)
         const float rf = gas.rho_ref + rft, pf = gas.p_ref + pft;
         const float igp = __fdividef(1.f, gas.gamma * pf), ipf = __fdividef(1.f, pf);
         lwf[0] = ly[0] * fmaf(d2, igp, 1.f);

@@ -61,7 +61,8 @@ __device__ __forceinline__ double with_ref(double, double x) { return x; }
 
 // Tests on the bits of a double: a comparison is an instruction of the FP64 unit,
 // which takes 64 cycles for a warp here (two lanes per cycle and SM), an integer
-// one takes one or two.  Same answers as the comparisons, NaN included.
+// one takes one or two.  Same answers as the comparisons, NaN included (at_least_one
+// alone takes a positive NaN for a number: its caller has sorted NaN out).
 __device__ __forceinline__ bool is_positive(float x) { return x > 0.f; }
 __device__ __forceinline__ bool is_positive(double x) {
   const long long b = __double_as_longlong(x);

@@ -939,10 +939,11 @@ __device__ __forceinline__ bool fused_tile(const StepArgs<float>& a, PipeCtx& pc
       for (int s = 0; s < 2; ++s) point(m, s, n, cn);
     }
   } else {
-    // Both durations of a point together: bound by instruction issue and shared
-    // memory, the pass saves the second load of the foot cell's nine nodes (36 of 134
-    // shared wavefronts per point) and half of the barriers, and the two chains hide
-    // each other's latency.  The results wait in tensor memory until every thread is
+    // Both durations of a point together: what bounds the pass is latency with four
+    // warps per scheduler (shared loads, fixed latencies and barriers; issue slots 65%
+    // busy, 0.56 shared wavefronts per cycle).  It saves the second load of the foot
+    // cell's nine nodes (36 of 134 shared wavefronts per point) and half of the barriers,
+    // and the two chains hide each other's latency.  The results wait in tensor memory until every thread is
     // done with the increments (in registers they would take 56; held for one
     // duration at a time they spilled).  2048^2, FP32_COMP: 0.690 -> 0.677 ms per step,
     // 1024^2 187 -> 180 us, 128^2 7.56 -> 7.14 us.  One duration after the other in the

@@ -6,14 +6,16 @@
 //
 // What bounds them: the FP64 unit (two lanes per cycle and SM).  A cell took about
 // 575 of its instructions: ten CUDA logarithms, eight square roots and seven
-// divisions, 32 conversions, minima and maxima.  It takes 160 now: the
+// divisions, 32 conversions, minima and maxima.  It takes 170 now: the
 // logarithm by a table (8 instructions, below), conversions on the integer units,
 // the minima on the stored floats, the wave speed evaluated in FP64 only where its
 // FP32 value comes near the grid's largest one, which the centre recovery before it
 // finds; common factors taken out of the sums.
-// A call at 2048^2 in FP32_COMP: 1.34 ms, 4.69 before (of which 0.22 ms was the
-// fold of the partials by one thread per value, now one warp); the FP64 unit is 85%
-// busy in k_inv_partial.
+// A call at 2048^2 in FP32_COMP: 1.52 ms, 4.69 before (of which 0.22 ms was the
+// fold of the partials by one thread per value, now one warp); the FP64 unit is 82%
+// busy in k_inv_partial.  (1.34 ms with a logarithm whose leading part was rounded and
+// with storage offsets added in plain FP32, which missed the largest speed beside a
+// dense reference.)
 #pragma once
 
 #include "af_common.cuh"

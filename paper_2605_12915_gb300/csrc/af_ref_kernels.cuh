@@ -19,9 +19,11 @@
 // node's fluxes are integrated in time once instead of in both edges it bounds.
 // Small grids are bound by the same unit on the few SMs that hold their warps:
 // the families share a launch (blockIdx.y) and blocks are two warps.
-// GB300, FP64: a step at 512^2 takes 1.01 ms (1.40 with ten launches, comparisons
+// GB300, FP64: a step at 512^2 takes 1.07 ms (1.40 with ten launches, comparisons
 // and floor in FP64, separate increments and per-edge fluxes); a whole
-// set-step-get call at 32^2 from pinned host memory 91 us (277).
+// set-step-get call at 32^2 from pinned host memory 76 us (277).  (Shorter forms of the
+// centre recovery, the freezing and the interpolation at the foot made it 1.01 ms and 71
+// us, but rounded more; see there.)
 #pragma once
 
 #include "af_common.cuh"
